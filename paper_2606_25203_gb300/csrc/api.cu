@@ -117,19 +117,18 @@ struct pamc_handle_s {
     int8_t *d_best = nullptr;
     // dense instances
     int8_t *d_J = nullptr;               // n x n couplings (J = -w)
+    uint32_t *d_Jb = nullptr;            // the same as bits (dense_sweep.cu)
     int32_t *d_H = nullptr;              // [R][n] fields
     uint8_t *d_Sb = nullptr;             // [64][n] e4m3 population for the tcgen05 recompute
     bool dense_tc = false;               // recompute on tcgen05 (n a multiple of 16)
-    bool dense_tcu = false;              // field update of the sweep on tcgen05
     alignas(64) unsigned char tm_J[128];  // tensor maps of J and of d_Sb
     alignas(64) unsigned char tm_S[128];
-    int32_t *d_perm = nullptr, *d_sidx = nullptr, *d_G = nullptr, *d_ident = nullptr, *d_nonc = nullptr;
+    int32_t *d_perm = nullptr, *d_sidx = nullptr, *d_ident = nullptr, *d_nonc = nullptr;
     int32_t *d_boff = nullptr;           // bucket offsets of the order sort
     uint32_t *d_pkey = nullptr;
-    uint32_t *d_T = nullptr, *d_T2 = nullptr;   // bit tiles of the dense chains
-    unsigned long long *d_flip = nullptr, *d_snew = nullptr;
-    void *d_bar = nullptr;
-    int32_t dense_Hc = 0, dense_grid = 0, dense_nupd = 0, dense_rows = 0;
+    uint32_t *d_rowbits = nullptr;       // positions that flipped in some replica (one bit each)
+    int32_t dense_Hc = 0;
+    int dense_cs = 1;                    // CTAs of a replica's cluster in the sweep
     int32_t dense_R = 0;                 // replicas this handle sweeps (p.R unless split over processes)
     int64_t launches = 0;
     // device time of the sweep launches (pamc_set_sweep_timing): events
@@ -431,32 +430,19 @@ pamc_status init_dense(pamc_handle h, pamc_params p, int32_t base, int32_t own, 
     if (p.stagnation && (h->n & 1))
         return fail(h, PAMC_ERR_ARG, "cluster moves on dense instances need even n (no iso-sites then)");
     if (p.sweeps > 64) return fail(h, PAMC_ERR_RANGE, "dense instances support at most 64 sweeps per step");
-    int coop = 0, sms = 0;
-    cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, h->device);
+    int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
-    if (!coop) return fail(h, PAMC_ERR_CUDA, "device lacks cooperative launch");
     const int32_t n = h->n, R = own, Rg = p.R, S = std::max(p.sweeps, 1);
-    const int chain = (R + 3) / 4;
-    const int grid = sms;
-    const int nupd = grid - chain;
-    if (nupd < 1) return fail(h, PAMC_ERR_RANGE, "too few SMs for the dense sweep");
-    // field update on the tensor cores (fields in tensor memory) when n allows TMA-style rows
-    const char *sw_env = getenv("PAMC_DENSE_UPDATE");   // "cuda": the CUDA-core update
-    const bool tcu = dense_tc_supported(n) && !(sw_env && strcmp(sw_env, "cuda") == 0);
-    int32_t rows = (n + nupd - 1) / nupd;
-    if (tcu) rows = (rows + 31) & ~31;
-    const size_t smem = dense_sweep_smem(n, R, rows, tcu);
-    if (rows > dense_sweep_threads() || smem > 227 * 1024)
-        return fail(h, PAMC_ERR_RANGE, "dense instance too large for the on-chip field slices");
+    // the largest instance: 768 vertices for each SM beyond one per four replicas
+    const int cs = dense_sweep_cluster(n, R, sms);
+    const int nupd = sms - (R + 3) / 4;
+    if (nupd < 1 || (n + nupd - 1) / nupd > 768 || cs == 0)
+        return fail(h, PAMC_ERR_RANGE, "dense instance too large for the on-chip fields");
     release_run(h);
     h->p = p;
-    h->dense_grid = grid;
-    h->dense_nupd = nupd;
-    h->dense_rows = rows;
-    h->dense_tcu = tcu;
+    h->dense_cs = cs;
     h->dense_Hc = std::min<int32_t>(n, 32767);
     h->dense_R = R;
-    const int B = dense_block_positions();
     const size_t tabn = (size_t)2 * h->dense_Hc + 1;
     // spin rows: the own replicas, and as many again for received parents
     const size_t rows_sp = split ? 2 * (size_t)R : (size_t)R;
@@ -469,10 +455,8 @@ pamc_status init_dense(pamc_handle h, pamc_params p, int32_t base, int32_t own, 
               alloc_n(h, h->d_tab, tabn, h->bufs) && alloc_n(h, h->d_ctl, 1, h->bufs) &&
               alloc_n(h, h->d_best, n, h->bufs) && alloc_n(h, h->d_H, (size_t)R * n, h->bufs) &&
               alloc_n(h, h->d_perm, (size_t)S * n, h->bufs) && alloc_n(h, h->d_pkey, (size_t)S * n, h->bufs) &&
-              alloc_n(h, h->d_sidx, (size_t)S * n, h->bufs) && alloc_n(h, h->d_G, (size_t)2 * B * 64, h->bufs) &&
-              alloc_n(h, h->d_T, (size_t)2 * B * (B / 32), h->bufs) && alloc_n(h, h->d_T2, (size_t)2 * B * (B / 32), h->bufs) &&
-              alloc_n(h, h->d_flip, (size_t)3 * B, h->bufs) && alloc_n(h, h->d_snew, (size_t)3 * B, h->bufs) &&
-              (h->d_bar = dev_alloc(h, 64, h->bufs)) != nullptr &&
+              alloc_n(h, h->d_sidx, (size_t)S * n, h->bufs) &&
+              alloc_n(h, h->d_rowbits, (size_t)S * ((n + 31) / 32), h->bufs) &&
               alloc_n(h, h->d_ident, R, h->bufs) && alloc_n(h, h->d_nonc, R, h->bufs) &&
               alloc_n(h, h->d_boff, dense_perm_offsets(S), h->bufs);
     if (ok && split) ok = alloc_n(h, h->d_plocal, R, h->bufs) && alloc_n(h, h->d_rows, Rg, h->bufs);
@@ -545,10 +529,9 @@ pamc_status step_dense(pamc_handle h, int32_t nsteps) {
             e = dense_recompute(h, src, h->d_parent, h->d_ncm_idx, -1);
         if (e == cudaSuccess) e = sweep_timer(h, false);
         if (e == cudaSuccess)
-            e = launch_dense_sweep(n, R, p.sweeps, p.rule, h->dense_Hc, (int32_t)t, p.seed, h->dense_nupd,
-                                   h->dense_rows, h->dense_grid, h->d_J, h->d_perm, h->d_tab, src,
-                                   h->d_parent, nullptr, h->d_ncm_idx, h->d_H, dst, Ed, h->d_G, h->d_T,
-                                   h->d_T2, h->d_flip, h->d_snew, h->d_bar, h->d_ctl, h->stream, h->dense_tcu);
+            e = launch_dense_sweep(n, R, p.sweeps, p.rule, h->dense_Hc, (int32_t)t, p.seed, h->dense_cs, h->d_Jb,
+                                   h->d_perm, h->d_tab, src, h->d_parent, h->d_H, dst, Ed, h->d_rowbits, h->d_ctl,
+                                   h->stream);
         if (e == cudaSuccess) e = sweep_timer(h, true);
         if (e == cudaSuccess) e = launch_control(n, h->W, p, Ed, dst, h->d_best, h->d_ctl, h->stream);
         h->launches += 7;
@@ -660,7 +643,8 @@ pamc_status pamc_create_dense(int32_t n, const int8_t *w, int w_on_device, int c
     const size_t total = (size_t)n * n;
     unsigned long long *d_sum = nullptr;
     int *d_err = nullptr;
-    if (!alloc_n(h, h->d_J, total, h->inst_bufs) || !alloc_n(h, d_sum, 1, h->inst_bufs) ||
+    if (!alloc_n(h, h->d_J, total, h->inst_bufs) ||
+        !alloc_n(h, h->d_Jb, (size_t)n * dense_bits_pitch(n), h->inst_bufs) || !alloc_n(h, d_sum, 1, h->inst_bufs) ||
         !alloc_n(h, d_err, 1, h->inst_bufs)) {
         dev_free_all(h, h->inst_bufs);
         delete h;
@@ -673,6 +657,7 @@ pamc_status pamc_create_dense(int32_t n, const int8_t *w, int w_on_device, int c
     if (e == cudaSuccess) e = launch_dense_negate_sum(total, h->d_J, d_sum, h->stream);
     if (e == cudaSuccess) e = launch_dense_validate(n, h->d_J, d_err, h->stream);
     if (e == cudaSuccess) e = launch_dense_to_e4m3(total, h->d_J, h->stream);   // stored as e4m3 bytes
+    if (e == cudaSuccess) e = launch_dense_pack_bits(n, h->d_J, h->d_Jb, h->stream);
     unsigned long long wsum = 0;
     int err = 0;
     if (e == cudaSuccess) e = cudaMemcpyAsync(&wsum, d_sum, sizeof(wsum), cudaMemcpyDeviceToHost, h->stream);
@@ -1066,10 +1051,9 @@ pamc_status pamc_shard_sweep(pamc_handle h, const int64_t *E_all, const int32_t 
         if (e == cudaSuccess) e = dense_recompute(h, src, h->d_plocal, h->d_ncm_idx + h->sh_base, -1);
         if (e == cudaSuccess) e = sweep_timer(h, false);
         if (e == cudaSuccess)
-            e = launch_dense_sweep(n, c, p.sweeps, p.rule, h->dense_Hc, (int32_t)t, p.seed, h->dense_nupd,
-                                   h->dense_rows, h->dense_grid, h->d_J, h->d_perm, h->d_tab, src, h->d_plocal,
-                                   nullptr, h->d_ncm_idx + h->sh_base, h->d_H, dst, Ed, h->d_G, h->d_T, h->d_T2,
-                                   h->d_flip, h->d_snew, h->d_bar, h->d_ctl, h->stream, h->dense_tcu, h->sh_base);
+            e = launch_dense_sweep(n, c, p.sweeps, p.rule, h->dense_Hc, (int32_t)t, p.seed, h->dense_cs, h->d_Jb,
+                                   h->d_perm, h->d_tab, src, h->d_plocal, h->d_H, dst, Ed, h->d_rowbits, h->d_ctl,
+                                   h->stream, h->sh_base);
         if (e == cudaSuccess) e = sweep_timer(h, true);
         h->launches += 4;
         if (e == cudaSuccess && E_own)

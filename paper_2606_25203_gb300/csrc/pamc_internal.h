@@ -348,17 +348,17 @@ cudaError_t launch_dense_energy(int32_t n, int32_t R, const int32_t *H, const in
 cudaError_t launch_init_spins(int kind, int32_t K, int32_t n, int32_t R, uint64_t seed, int32_t t,
                               int only_if_restart, const DevCtl *ctl, int8_t *spins, cudaStream_t st,
                               int32_t rbase = 0);
-int dense_block_positions();
-int dense_sweep_threads();
-size_t dense_sweep_smem(int32_t n, int32_t R, int32_t rows_per, bool tcu);
-cudaError_t launch_dense_sweep(int32_t n, int32_t R, int32_t S, int32_t rule, int32_t Hc, int32_t t,
-                               uint64_t seed, int32_t n_upd, int32_t rows_per, int32_t grid,
-                               const int8_t *J, const int32_t *perm, const uint64_t *tab,
-                               const int8_t *src, const int32_t *parent, const int8_t *ncm_buf,
-                               const int32_t *ncm_idx, int32_t *H, int8_t *dst, int64_t *E,
-                               int32_t *G, uint32_t *T, uint32_t *T2, unsigned long long *flip,
-                               unsigned long long *snew, void *bar, DevCtl *ctl, cudaStream_t st, bool tcu,
-                               int32_t rbase = 0);
+// Sweeps of the dense instance (dense_sweep.cu): the bit matrix (bit j of row
+// i set iff J_ij = +1, rows of dense_bits_pitch words), one cluster of cs CTAs
+// per replica (0: the fields of a replica fit no cluster); rowbits: scratch of
+// S * ceil(n / 32) words.
+int32_t dense_bits_pitch(int32_t n);
+cudaError_t launch_dense_pack_bits(int32_t n, const int8_t *J, uint32_t *Jb, cudaStream_t st);
+int dense_sweep_cluster(int32_t n, int32_t R, int sms);
+cudaError_t launch_dense_sweep(int32_t n, int32_t R, int32_t S, int32_t rule, int32_t Hc, int32_t t, uint64_t seed,
+                               int cs, const uint32_t *Jb, const int32_t *perm, const uint64_t *tab,
+                               const int8_t *src, const int32_t *parent, int32_t *H, int8_t *dst, int64_t *E,
+                               uint32_t *rowbits, DevCtl *ctl, cudaStream_t st, int32_t rbase = 0);
 cudaError_t launch_dense_to_e4m3(size_t total, int8_t *J, cudaStream_t st);
 
 // ---- dense recompute on tcgen05 (dense_tc.cu), n a multiple of 16

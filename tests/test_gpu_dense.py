@@ -83,6 +83,20 @@ def test_dense_cold_rare_flips(pg, rule):
     compare_dense(pg, 1024, 12, R=16, sweeps=2, beta0=0.5, beta1=3.0, rule=rule, seed=9, check_every=3)
 
 
+@pytest.mark.parametrize("rule", [0, 1])
+@pytest.mark.parametrize("cluster", [1, 2, 4, 8])
+@pytest.mark.parametrize("n,R,betas", [
+    (33, 3, (0.05, 2.0)),          # slices of one word, most of a cluster's CTAs empty
+    (1023, 6, (0.01, 1.0)),        # ragged words and batches, hot to cold
+    (2501, 5, (0.0005, 0.001)),    # thresholds over every field: the table stays in device memory
+])
+def test_dense_clusters(pg, monkeypatch, n, R, betas, cluster, rule):
+    """A replica's fields split over 1 to 8 CTAs, at the edges of slices,
+    row words and batches; results are the same for every split."""
+    monkeypatch.setenv("PAMC_DENSE_CLUSTER", str(cluster))
+    compare_dense(pg, n, 3, R=R, sweeps=2, beta0=betas[0], beta1=betas[1], rule=rule, seed=n)
+
+
 def test_dense_restart_and_controller(pg):
     compare_dense(pg, 320, 60, R=16, sweeps=1, beta0=0.01, beta1=0.4, stagnation=1, z_rst=45, seed=5,
                   check_every=3)
