@@ -116,14 +116,12 @@ struct pamc_handle_s {
     DevCtl *d_ctl = nullptr;
     int8_t *d_best = nullptr;
     // dense instances
-    int8_t *d_J = nullptr;               // n x n couplings (J = -w)
-    uint32_t *d_Jb = nullptr;            // the same as bits (dense_sweep.cu)
+    uint32_t *d_Jb = nullptr;            // n x n couplings J = -w, one bit each (+1 set)
     int32_t *d_H = nullptr;              // [R][n] fields
-    uint8_t *d_Sb = nullptr;             // [64][n] e4m3 population for the tcgen05 recompute
-    bool dense_tc = false;               // recompute on tcgen05 (n a multiple of 16)
-    alignas(64) unsigned char tm_J[128];  // tensor maps of J and of d_Sb
+    uint8_t *d_Sb = nullptr;             // e4m3 population for the recompute
+    alignas(64) unsigned char tm_J[128];  // tensor maps of d_Jb and of d_Sb
     alignas(64) unsigned char tm_S[128];
-    int32_t *d_perm = nullptr, *d_sidx = nullptr, *d_ident = nullptr, *d_nonc = nullptr;
+    int32_t *d_perm = nullptr, *d_sidx = nullptr, *d_ident = nullptr;
     int32_t *d_boff = nullptr;           // bucket offsets of the order sort
     uint32_t *d_pkey = nullptr;
     uint32_t *d_rowbits = nullptr;       // positions that flipped in some replica (one bit each)
@@ -410,13 +408,9 @@ SweepCfg choose_cfg(int kind, int32_t n, int32_t R, int32_t H, double avg_level,
 }
 
 // ---------------------------------------------------------------- dense runs
-// H = J S for the population given by (src, parent, ncm_idx)
-cudaError_t dense_recompute(pamc_handle h, const int8_t *src, const int32_t *parent, const int32_t *ncm_idx,
-                            int restart_t) {
-    if (h->dense_tc)
-        return launch_dense_recompute_tc(h->n, h->dense_R, h->tm_J, h->tm_S, src, parent, nullptr, ncm_idx, h->d_Sb,
-                                         h->d_H, h->d_ctl, h->stream, restart_t);
-    return launch_dense_recompute(h->n, h->dense_R, h->d_J, src, parent, nullptr, ncm_idx, h->d_H, h->d_ctl,
+// H = J S for the population whose replica r is row parent[r] of src
+cudaError_t dense_recompute(pamc_handle h, const int8_t *src, const int32_t *parent, int restart_t) {
+    return launch_dense_recompute(h->n, h->dense_R, h->tm_J, h->tm_S, src, parent, h->d_Sb, h->d_H, h->d_ctl,
                                   h->stream, restart_t);
 }
 
@@ -457,20 +451,17 @@ pamc_status init_dense(pamc_handle h, pamc_params p, int32_t base, int32_t own, 
               alloc_n(h, h->d_perm, (size_t)S * n, h->bufs) && alloc_n(h, h->d_pkey, (size_t)S * n, h->bufs) &&
               alloc_n(h, h->d_sidx, (size_t)S * n, h->bufs) &&
               alloc_n(h, h->d_rowbits, (size_t)S * ((n + 31) / 32), h->bufs) &&
-              alloc_n(h, h->d_ident, R, h->bufs) && alloc_n(h, h->d_nonc, R, h->bufs) &&
+              alloc_n(h, h->d_ident, R, h->bufs) &&
               alloc_n(h, h->d_boff, dense_perm_offsets(S), h->bufs);
     if (ok && split) ok = alloc_n(h, h->d_plocal, R, h->bufs) && alloc_n(h, h->d_rows, Rg, h->bufs);
-    const char *rc_env = getenv("PAMC_DENSE_RECOMPUTE");   // "mma": the mma.sync kernel
-    h->dense_tc = dense_tc_supported(n) && !(rc_env && strcmp(rc_env, "mma") == 0);
-    if (ok && h->dense_tc) {
-        ok = alloc_n(h, h->d_Sb, (size_t)64 * n, h->bufs);
-        if (ok && (dense_tc_map(h->tm_J, h->d_J, n, n, 256) != cudaSuccess ||
-                   dense_tc_map(h->tm_S, h->d_Sb, 64, n, 64) != cudaSuccess))
-            h->dense_tc = false;
-    }
+    if (ok) ok = alloc_n(h, h->d_Sb, dense_recompute_scratch(n), h->bufs);
     if (!ok) {
         release_run(h);
         return fail(h, PAMC_ERR_OOM, "device allocation of the dense population failed");
+    }
+    if (dense_recompute_maps(n, R, h->d_Jb, h->d_Sb, h->tm_J, h->tm_S) != cudaSuccess) {
+        release_run(h);
+        return fail(h, PAMC_ERR_CUDA, "tensor maps of the dense instance");
     }
     DevCtl c;
     memset(&c, 0, sizeof(c));
@@ -488,7 +479,6 @@ pamc_status init_dense(pamc_handle h, pamc_params p, int32_t base, int32_t own, 
     if (e == cudaSuccess) e = cudaMemcpyAsync(h->d_ident, ident.data(), 4 * R, cudaMemcpyHostToDevice, h->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(h->d_count, ones.data(), 4 * Rg, cudaMemcpyHostToDevice, h->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(h->d_ncm_idx, minus.data(), 4 * Rg, cudaMemcpyHostToDevice, h->stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(h->d_nonc, minus.data(), 4 * R, cudaMemcpyHostToDevice, h->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(h->d_best, 0, n, h->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(h->d_E[0], 0, 64 * 8, h->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(h->d_E[1], 0, 64 * 8, h->stream);
@@ -496,7 +486,7 @@ pamc_status init_dense(pamc_handle h, pamc_params p, int32_t base, int32_t own, 
     if (e == cudaSuccess)
         e = launch_init_spins(0, 0, n, R, p.seed, 0, 0, h->d_ctl, h->d_spins[0], h->stream, base);
     if (e == cudaSuccess)
-        e = dense_recompute(h, h->d_spins[0], h->d_ident, h->d_nonc, -1);
+        e = dense_recompute(h, h->d_spins[0], h->d_ident, -1);
     if (e == cudaSuccess)
         e = launch_dense_energy(n, R, h->d_H, h->d_spins[0], h->d_E[0], h->d_ctl, h->stream, -1);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
@@ -526,7 +516,7 @@ pamc_status step_dense(pamc_handle h, int32_t nsteps) {
                             nullptr, h->stream);
         if (e == cudaSuccess) e = launch_dense_tables(p.rule, h->dense_Hc, n, h->d_ctl, h->d_tab, h->stream);
         if (e == cudaSuccess)
-            e = dense_recompute(h, src, h->d_parent, h->d_ncm_idx, -1);
+            e = dense_recompute(h, src, h->d_parent, -1);
         if (e == cudaSuccess) e = sweep_timer(h, false);
         if (e == cudaSuccess)
             e = launch_dense_sweep(n, R, p.sweeps, p.rule, h->dense_Hc, (int32_t)t, p.seed, h->dense_cs, h->d_Jb,
@@ -539,7 +529,7 @@ pamc_status step_dense(pamc_handle h, int32_t nsteps) {
             const int32_t tk = (int32_t)(t + 1);
             e = launch_init_spins(0, 0, n, R, p.seed, tk, 1, h->d_ctl, dst, h->stream);
             if (e == cudaSuccess)
-                e = dense_recompute(h, dst, h->d_ident, h->d_nonc, tk);
+                e = dense_recompute(h, dst, h->d_ident, tk);
             if (e == cudaSuccess) e = launch_dense_energy(n, R, h->d_H, dst, Ed, h->d_ctl, h->stream, tk);
             h->launches += 3;
         }
@@ -640,30 +630,40 @@ pamc_status pamc_create_dense(int32_t n, const int8_t *w, int w_on_device, int c
     h->dense = 1;
     h->nnz = 0;
     h->H = 0;
-    const size_t total = (size_t)n * n;
+    // weights on the device are read in place, host ones through a staging
+    // buffer of as many rows as fit 256 MB
+    const int32_t chunk = w_on_device ? n : (int32_t)std::max<int64_t>(1, std::min<int64_t>(n, (256ll << 20) / n));
     unsigned long long *d_sum = nullptr;
     int *d_err = nullptr;
-    if (!alloc_n(h, h->d_J, total, h->inst_bufs) ||
-        !alloc_n(h, h->d_Jb, (size_t)n * dense_bits_pitch(n), h->inst_bufs) || !alloc_n(h, d_sum, 1, h->inst_bufs) ||
-        !alloc_n(h, d_err, 1, h->inst_bufs)) {
+    int8_t *d_stage = nullptr;
+    std::vector<DevBuf> tmp;
+    if (!alloc_n(h, h->d_Jb, (size_t)n * dense_bits_pitch(n), h->inst_bufs) || !alloc_n(h, d_sum, 1, tmp) ||
+        !alloc_n(h, d_err, 1, tmp) || (!w_on_device && !alloc_n(h, d_stage, (size_t)chunk * n, tmp))) {
+        dev_free_all(h, tmp);
         dev_free_all(h, h->inst_bufs);
         delete h;
         return fail(nullptr, PAMC_ERR_OOM, "device allocation of the dense instance failed");
     }
-    e = cudaMemcpyAsync(h->d_J, w, total, w_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
-                        h->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(d_sum, 0, sizeof(*d_sum), h->stream);
+    e = cudaMemsetAsync(d_sum, 0, sizeof(*d_sum), h->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(d_err, 0, sizeof(*d_err), h->stream);
-    if (e == cudaSuccess) e = launch_dense_negate_sum(total, h->d_J, d_sum, h->stream);
-    if (e == cudaSuccess) e = launch_dense_validate(n, h->d_J, d_err, h->stream);
-    if (e == cudaSuccess) e = launch_dense_to_e4m3(total, h->d_J, h->stream);   // stored as e4m3 bytes
-    if (e == cudaSuccess) e = launch_dense_pack_bits(n, h->d_J, h->d_Jb, h->stream);
+    for (int32_t i0 = 0; e == cudaSuccess && i0 < n; i0 += chunk) {
+        const int32_t rows = std::min(chunk, n - i0);
+        const int8_t *src = w;
+        if (!w_on_device) {
+            e = cudaMemcpyAsync(d_stage, w + (size_t)i0 * n, (size_t)rows * n, cudaMemcpyHostToDevice, h->stream);
+            src = d_stage;
+        }
+        if (e == cudaSuccess) e = launch_dense_pack(n, i0, rows, src, h->d_Jb, d_sum, d_err, h->stream);
+        h->launches += 1;
+    }
+    if (e == cudaSuccess) e = launch_dense_symmetric(n, h->d_Jb, d_err, h->stream);
     unsigned long long wsum = 0;
     int err = 0;
     if (e == cudaSuccess) e = cudaMemcpyAsync(&wsum, d_sum, sizeof(wsum), cudaMemcpyDeviceToHost, h->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(&err, d_err, sizeof(err), cudaMemcpyDeviceToHost, h->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-    h->launches += 2;
+    h->launches += 1;
+    dev_free_all(h, tmp);
     if (e != cudaSuccess || err != 0) {
         dev_free_all(h, h->inst_bufs);
         delete h;
@@ -672,7 +672,7 @@ pamc_status pamc_create_dense(int32_t n, const int8_t *w, int w_on_device, int c
                     err == PAMC_ERR_ASYM ? "not symmetric" : err == PAMC_ERR_DIAG ? "nonzero diagonal"
                                                                             : "entries must be +-1 off the diagonal");
     }
-    h->W = (int64_t)wsum / 2;   // sum over ordered pairs counts each edge twice
+    h->W = ((int64_t)n * (n - 1) - 2 * (int64_t)wsum) / 2;   // every edge counted twice; wsum: the negative entries
     *out = h;
     return PAMC_OK;
 }
@@ -1048,7 +1048,7 @@ pamc_status pamc_shard_sweep(pamc_handle h, const int64_t *E_all, const int32_t 
     if (e == cudaSuccess && nimports > 0)
         e = cudaMemcpyAsync(src + (size_t)c * n, imports, (size_t)nimports * n, cudaMemcpyDeviceToDevice, h->stream);
     if (h->dense) {   // the fields of the own slots' parents, then the sweeps
-        if (e == cudaSuccess) e = dense_recompute(h, src, h->d_plocal, h->d_ncm_idx + h->sh_base, -1);
+        if (e == cudaSuccess) e = dense_recompute(h, src, h->d_plocal, -1);
         if (e == cudaSuccess) e = sweep_timer(h, false);
         if (e == cudaSuccess)
             e = launch_dense_sweep(n, c, p.sweeps, p.rule, h->dense_Hc, (int32_t)t, p.seed, h->dense_cs, h->d_Jb,
@@ -1101,7 +1101,7 @@ pamc_status pamc_shard_control(pamc_handle h, const int64_t *E_all, int64_t *E_o
         if (h->dense) {
             const int32_t tk = (int32_t)(t + 1);
             e = launch_init_spins(0, 0, n, c, p.seed, tk, 1, h->d_ctl, dst, h->stream, h->sh_base);
-            if (e == cudaSuccess) e = dense_recompute(h, dst, h->d_ident, h->d_nonc, tk);
+            if (e == cudaSuccess) e = dense_recompute(h, dst, h->d_ident, tk);
             if (e == cudaSuccess) e = launch_dense_energy(n, c, h->d_H, dst, Ed, h->d_ctl, h->stream, tk);
             h->launches += 3;
         } else {
@@ -1309,7 +1309,7 @@ pamc_status pamc_load(pamc_handle h, const void *buf, size_t size) {
     in += (size_t)R * 8;
     if (e == cudaSuccess) e = cudaMemcpyAsync(h->d_best, in, (size_t)n, cudaMemcpyHostToDevice, h->stream);
     // dense runs keep the fields of the population: recompute them exactly
-    if (e == cudaSuccess && h->dense) e = dense_recompute(h, h->d_spins[cur], h->d_ident, h->d_nonc, -1);
+    if (e == cudaSuccess && h->dense) e = dense_recompute(h, h->d_spins[cur], h->d_ident, -1);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);   // the host buffer may go after return
     if (e != cudaSuccess) return cuda_fail(h, e, "pamc_load upload");
     h->host_t = c.t;
@@ -1338,7 +1338,7 @@ pamc_status pamc_set_population(pamc_handle h, const int8_t *spins) {
     cudaError_t e = cudaMemcpyAsync(h->d_spins[cur], spins, total, cudaMemcpyHostToDevice, h->stream);
     if (h->dense) {
         if (e == cudaSuccess)
-            e = dense_recompute(h, h->d_spins[cur], h->d_ident, h->d_nonc, -1);
+            e = dense_recompute(h, h->d_spins[cur], h->d_ident, -1);
         if (e == cudaSuccess)
             e = launch_dense_energy(n, R, h->d_H, h->d_spins[cur], h->d_E[cur], h->d_ctl, h->stream, -1);
     } else if (e == cudaSuccess) {

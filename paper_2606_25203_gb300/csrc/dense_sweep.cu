@@ -481,19 +481,6 @@ __global__ void __launch_bounds__(kDsThreads, 1) k_dense_sweep(DenseSweepArgs a,
     }
 }
 
-// bit (i, j) of the bit matrix from the e4m3 couplings: J_ij = +1 (0x38);
-// a warp packs the 32 columns of a word
-__global__ void __launch_bounds__(256)
-k_dense_pack_bits(int32_t n, int32_t pitch, const uint8_t *__restrict__ J, uint32_t *__restrict__ Jb) {
-    const int lane = threadIdx.x & 31;
-    const int32_t i = blockIdx.y;
-    for (int32_t w = blockIdx.x * 8 + (threadIdx.x >> 5); w < pitch; w += gridDim.x * 8) {
-        const int32_t j = 32 * w + lane;
-        const uint32_t b = __ballot_sync(0xffffffffu, j < n && J[(size_t)i * n + min(j, n - 1)] == 0x38);
-        if (lane == 0) Jb[(size_t)i * pitch + w] = b;
-    }
-}
-
 size_t ds_smem(int32_t n, int cs) {
     const int32_t per = ((n + cs - 1) / cs + 31) & ~31, nW = per >> 5, nWp = nW | 1;
     return ((sizeof(DsSmem) + 15) & ~(size_t)15) + (size_t)32 * nWp * 4 + (size_t)nW * 4;
@@ -501,17 +488,8 @@ size_t ds_smem(int32_t n, int cs) {
 
 }  // namespace
 
-int32_t dense_bits_pitch(int32_t n) { return ((n + 127) / 128) * 4; }
-
-cudaError_t launch_dense_pack_bits(int32_t n, const int8_t *J, uint32_t *Jb, cudaStream_t st) {
-    const int32_t pitch = dense_bits_pitch(n);
-    for (int32_t i0 = 0; i0 < n; i0 += 65535) {
-        const int32_t rows = n - i0 < 65535 ? n - i0 : 65535;
-        k_dense_pack_bits<<<dim3((pitch + 63) / 64, rows), 256, 0, st>>>(
-            n, pitch, reinterpret_cast<const uint8_t *>(J) + (size_t)i0 * n, Jb + (size_t)i0 * pitch);
-    }
-    return cudaGetLastError();
-}
+// words of a row: whole 128-byte lines (the recompute copies 1,024 couplings of a row at a time)
+int32_t dense_bits_pitch(int32_t n) { return ((n + 1023) / 1024) * 32; }
 
 // The smallest cluster whose slices fit; from n = 32,000 on twice or four times
 // as many CTAs a replica where every cluster still gets its own SMs: a slice's

@@ -255,7 +255,7 @@ size_t hamming_tc_scratch(int32_t n, int32_t R) {
 bool hamming_tc_enabled(int32_t n, int32_t R) {
     const char *env = getenv("PAMC_HAMMING");
     if (env && strcmp(env, "cuda") == 0) return false;
-    return R >= 2 && n >= 1 && dense_tc_supported(16);
+    return R >= 2 && n >= 1 && dense_tc_supported();
 }
 
 cudaError_t launch_hamming_tc(int32_t n, int32_t R, const int8_t *spins, uint8_t *Sb, unsigned long long *hist,

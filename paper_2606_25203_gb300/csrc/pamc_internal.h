@@ -331,18 +331,16 @@ cudaError_t launch_hamming_tc(int32_t n, int32_t R, const int8_t *spins, uint8_t
                               unsigned long long *sum, int *err, cudaStream_t st);
 
 // ---- dense instances (dense.cu)
-cudaError_t launch_dense_validate(int32_t n, const int8_t *J, int *err, cudaStream_t st);
-cudaError_t launch_dense_negate_sum(size_t total, int8_t *J, unsigned long long *wsum, cudaStream_t st);
+// int8 weights -> bit matrix (rows i0 .. of w, whose first row is row i0);
+// *neg += the negative entries, *err the first error found (pamc_status)
+cudaError_t launch_dense_pack(int32_t n, int32_t i0, int32_t rows, const int8_t *w, uint32_t *Jb,
+                              unsigned long long *neg, int *err, cudaStream_t st);
+cudaError_t launch_dense_symmetric(int32_t n, const uint32_t *Jb, int *err, cudaStream_t st);
 cudaError_t launch_dense_perm(int32_t n, uint64_t seed, int32_t t, int32_t S, int32_t *perm,
                               uint32_t *skey, int32_t *sidx, int32_t *boff, const DevCtl *ctl, cudaStream_t st);
 size_t dense_perm_offsets(int32_t S);   // int32 bucket offsets launch_dense_perm needs
 cudaError_t launch_dense_tables(int rule, int32_t Hc, int32_t n, DevCtl *ctl, uint64_t *tab,
                                 cudaStream_t st);
-size_t dense_recompute_smem();
-cudaError_t launch_dense_recompute(int32_t n, int32_t R, const int8_t *J, const int8_t *src,
-                                   const int32_t *parent, const int8_t *ncm_buf,
-                                   const int32_t *ncm_idx, int32_t *H, const DevCtl *ctl,
-                                   cudaStream_t st, int restart_t);
 cudaError_t launch_dense_energy(int32_t n, int32_t R, const int32_t *H, const int8_t *spins, int64_t *E,
                                 const DevCtl *ctl, cudaStream_t st, int restart_t);
 cudaError_t launch_init_spins(int kind, int32_t K, int32_t n, int32_t R, uint64_t seed, int32_t t,
@@ -353,22 +351,22 @@ cudaError_t launch_init_spins(int kind, int32_t K, int32_t n, int32_t R, uint64_
 // per replica (0: the fields of a replica fit no cluster); rowbits: scratch of
 // S * ceil(n / 32) words.
 int32_t dense_bits_pitch(int32_t n);
-cudaError_t launch_dense_pack_bits(int32_t n, const int8_t *J, uint32_t *Jb, cudaStream_t st);
 int dense_sweep_cluster(int32_t n, int32_t R, int sms);
 cudaError_t launch_dense_sweep(int32_t n, int32_t R, int32_t S, int32_t rule, int32_t Hc, int32_t t, uint64_t seed,
                                int cs, const uint32_t *Jb, const int32_t *perm, const uint64_t *tab,
                                const int8_t *src, const int32_t *parent, int32_t *H, int8_t *dst, int64_t *E,
                                uint32_t *rowbits, DevCtl *ctl, cudaStream_t st, int32_t rbase = 0);
-cudaError_t launch_dense_to_e4m3(size_t total, int8_t *J, cudaStream_t st);
 
-// ---- dense recompute on tcgen05 (dense_tc.cu), n a multiple of 16
-bool dense_tc_supported(int32_t n);
-size_t dense_tc_smem();
-// map: 128-byte CUtensorMap storage (64-byte aligned)
+// ---- dense recompute H = J S on tcgen05 (dense_tc.cu); Sb: scratch of
+// dense_recompute_scratch bytes; maps: 128-byte CUtensorMap storage each
+// (64-byte aligned), of the bit matrix and of Sb
+bool dense_tc_supported();
+size_t dense_recompute_scratch(int32_t n);
 cudaError_t dense_tc_map(void *map, const void *base, int32_t rows, int32_t cols, int32_t box_rows);
-cudaError_t launch_dense_recompute_tc(int32_t n, int32_t R, const void *mapJ, const void *mapS,
-                                      const int8_t *src, const int32_t *parent, const int8_t *ncm_buf,
-                                      const int32_t *ncm_idx, uint8_t *Sb, int32_t *H, DevCtl *ctl,
-                                      cudaStream_t st, int restart_t);
+cudaError_t dense_recompute_maps(int32_t n, int32_t R, const uint32_t *Jb, const uint8_t *Sb, void *mapJ,
+                                 void *mapS);
+cudaError_t launch_dense_recompute(int32_t n, int32_t R, const void *mapJ, const void *mapS, const int8_t *src,
+                                   const int32_t *parent, uint8_t *Sb, int32_t *H, DevCtl *ctl, cudaStream_t st,
+                                   int restart_t);
 
 }  // namespace pamc
