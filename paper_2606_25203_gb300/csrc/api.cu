@@ -83,7 +83,7 @@ struct pamc_handle_s {
     // instance
     int32_t *d_rp = nullptr;
     uint32_t *d_adj = nullptr;
-    int4 *d_nibc = nullptr;      // per-vertex constants of the biased 4-bit lanes, or nullptr
+    int nib_halves = 0;        // half-rows of the 4-bit lanes (0: they do not apply)
     // run
     pamc_params p{};
     int initialized = 0;
@@ -315,8 +315,11 @@ SweepCfg choose_cfg(int kind, int32_t n, int32_t R, int32_t H, double avg_level,
     const int32_t groups = (R + 3) / 4;   // every sweep kind groups four replicas
     const bool lpv_ok = kind == 0 && ell_w > 4;
     if (const char *env = getenv("PAMC_SWEEP_CFG")) {
-        int a = 0, b = 0, v = 1;
-        const int got = sscanf(env, "%d,%d,%d", &a, &b, &v);
+        int a = 0, b = 0, v = 1, staged = 0;
+        const int got = sscanf(env, "%d,%d,%d,%d", &a, &b, &v, &staged);
+        if (got == 4 && staged && kind == 0 && ell_w > 0 && a == 1 && b >= 1 && b <= 8 && v >= 1 && v <= 8 &&
+            (v & (v - 1)) == 0 && sweep_staged_ring(n, H, ell_w, SweepCfg{1, b, v, 1}) > 0)
+            return SweepCfg{1, b, v, 1};
         if (got >= 2 && a >= 1 && a <= 15 && b >= 1 && a * b * 32 <= 1024 &&
             v >= 1 && v <= 32 && (v & (v - 1)) == 0) {
             // Ising: lanes per vertex on ELL rows; the cascaded Potts sweep:
@@ -405,6 +408,25 @@ SweepCfg choose_cfg(int kind, int32_t n, int32_t R, int32_t H, double avg_level,
             best.lanes_per_vertex *= 2;
     }
     return best;
+}
+
+// The staged sweep (sweep_staged.cu) where every group of four has an SM to
+// itself and a launch is bound by its levels: byte lanes up to an average level
+// of 125 vertices (wider ones have the lanes of the plain sweep busy), 16-bit
+// lanes up to 400.  A pass of a set covers an average level with a little room;
+// rows of more than five couplings take two lanes a vertex, beyond 32 four.
+// us per launch, plain against staged sweep: N=800 degree 48 R=128 329 / 214,
+// N=3,000 degree 20 R=64 279 / 231 (levels of 59), N=2,000 R=256 187 / 189
+// (39), N=4,000 degree 14 R=100 534 / 450 (105), N=10,007 R=509 895 / 954 (196);
+// 16-bit lanes N=2,500 degree 12 R=250 (83) 464 / 179.
+SweepCfg staged_cfg(int32_t n, int32_t R, int32_t H, double avg_level, double avg_deg, int sms, int32_t ell_w) {
+    const bool wide = H > kByteLaneMaxH;
+    SweepCfg c{1, 2, avg_deg > 32.0 ? 4 : avg_deg > 5.0 ? 2 : 1, 0};
+    if ((R + 3) / 4 > sms || avg_level > (wide ? 400.0 : 125.0)) return c;
+    const double warps = 1.15 * avg_level * c.lanes_per_vertex / 32.0;
+    c.warps_per_group = warps <= 2.0 ? 2 : warps <= 4.0 ? 4 : warps <= 6.0 ? 6 : 8;
+    c.staged = sweep_staged_ring(n, H, ell_w, c) > 0 ? 1 : 0;
+    return c;
 }
 
 // ---------------------------------------------------------------- dense runs
@@ -586,14 +608,9 @@ pamc_status pamc_create_csr(int32_t n, const int32_t *row_ptr, const int32_t *co
     // (the schedule's position record holds the degree in 8 bits)
     const int64_t ell_entries = (int64_t)((n + 31) / 32) * 32 * ((maxdeg + 3) & ~3);
     h->ell_w = (maxdeg > 0 && maxdeg < 256 && ell_entries <= 4 * (int64_t)h->nnz + 4096) ? ((maxdeg + 3) & ~3) : 0;
-    // field ranges beyond the fixed 4-bit bias (7) but within 15 a half-row:
-    // the biased 4-bit lanes' per-vertex constants
-    std::vector<int4> nibc;
-    const bool biased = h->ell_w > 0 && !(H <= kNibbleMaxH && (h->ell_w == 4 || h->ell_w == 8)) &&
-                        nibble_biased_constants(n, row_ptr, adj.data(), H, h->ell_w, nibc);
+    h->nib_halves = h->ell_w > 0 ? nibble_halves(n, row_ptr, adj.data(), H, h->ell_w) : 0;
     if (!alloc_n(h, h->d_rp, (size_t)n + 1, h->inst_bufs) ||
-        !alloc_n(h, h->d_adj, (size_t)std::max(h->nnz, 1), h->inst_bufs) ||
-        (biased && !alloc_n(h, h->d_nibc, (size_t)n, h->inst_bufs))) {
+        !alloc_n(h, h->d_adj, (size_t)std::max(h->nnz, 1), h->inst_bufs)) {
         dev_free_all(h, h->inst_bufs);
         delete h;
         return fail(nullptr, PAMC_ERR_OOM, "device allocation of the instance failed");
@@ -602,8 +619,6 @@ pamc_status pamc_create_csr(int32_t n, const int32_t *row_ptr, const int32_t *co
     if (e == cudaSuccess && h->nnz > 0)
         e = cudaMemcpyAsync(h->d_adj, adj.data(), sizeof(uint32_t) * h->nnz, cudaMemcpyHostToDevice,
                             h->stream);
-    if (e == cudaSuccess && biased)
-        e = cudaMemcpyAsync(h->d_nibc, nibc.data(), sizeof(int4) * n, cudaMemcpyHostToDevice, h->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     if (e != cudaSuccess) {
         dev_free_all(h, h->inst_bufs);
@@ -806,13 +821,20 @@ static pamc_status init_run(pamc_handle h, const pamc_params *pp, int32_t rank, 
     int sms = 152;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
     h->cfg = choose_cfg(sweep_kind(p), n, own, h->H, avg_level, (double)h->nnz / std::max(n, 1), sms, h->ell_w);
+    const char *genv = getenv("PAMC_SWEEP_GLOBAL");
+    const bool nib_ok = p.kind == 0 && sweep_nibble_ok(h->nib_halves, p.sweeps, 1, false) && !sweep_push_enabled();
+    if (p.kind == 0 && p.sweeps > 0 && h->ell_w > 0 && !nib_ok && !sweep_push_enabled() &&
+        !(genv && genv[0] == '1') && !getenv("PAMC_SWEEP_CFG")) {
+        const SweepCfg c = staged_cfg(n, own, h->H, avg_level, (double)h->nnz / std::max(n, 1), sms, h->ell_w);
+        if (c.staged) h->cfg = c;
+    }
     // Ising groups whose spin words do not fit shared memory (or all of them
     // with PAMC_SWEEP_GLOBAL=1) keep the words in device memory: one lane per
     // vertex, one group per CTA
-    const char *genv = getenv("PAMC_SWEEP_GLOBAL");
     const bool wide = p.kind == 0 && h->H > kByteLaneMaxH;   // 16-bit field lanes, one lane per vertex
-    if (wide) h->cfg.lanes_per_vertex = 1;
-    if (p.kind == 0 && ((genv && genv[0] == '1') || sweep_smem_bytes(0, n, h->H, h->cfg) > kSmemMax)) {
+    if (wide && !h->cfg.staged) h->cfg.lanes_per_vertex = 1;
+    if (p.kind == 0 && !h->cfg.staged &&
+        ((genv && genv[0] == '1') || sweep_smem_bytes(0, n, h->H, h->cfg) > kSmemMax)) {
         if (!getenv("PAMC_SWEEP_CFG")) h->cfg = SweepCfg{1, 16, 1};
         h->cfg.lanes_per_vertex = 1;
         if (!alloc_n(h, h->d_gsp, gsp_words(n, own) * (wide ? 2 : 1), h->bufs)) {
@@ -824,8 +846,7 @@ static pamc_status init_run(pamc_handle h, const pamc_params *pp, int32_t rank, 
     // field ranges of at most 7 on ELL rows of width 4 or 8, or of 15 a
     // half-row on rows up to 16 wide: eight replicas a word (groups of eight,
     // shaped like a population of half the size)
-    if (p.kind == 0 && !h->gsp && sweep_nibble_ok(h->H, p.sweeps, h->ell_w, 1, false, h->d_nibc != nullptr) &&
-        !sweep_push_enabled()) {
+    if (nib_ok && !h->gsp && !h->cfg.staged) {
         SweepCfg c = choose_cfg(0, n, 4 * ((own + 7) / 8), h->H, avg_level, (double)h->nnz / std::max(n, 1), sms,
                                 h->ell_w);
         c.lanes_per_vertex = 1;
@@ -898,7 +919,7 @@ pamc_status pamc_step(pamc_handle h, int32_t nsteps) {
                            h->d_nkey, h->d_ctl, h->stream);
             h->launches += 1;
         }
-        SchedView sv{h->d_order, h->d_lvl, h->d_nlev, h->d_ell, h->d_pos, h->ell_w, h->d_nibc};
+        SchedView sv{h->d_order, h->d_lvl, h->d_nlev, h->d_ell, h->d_pos, h->ell_w, h->nib_halves};
         if (e == cudaSuccess) e = sweep_timer(h, false);
         if (e == cudaSuccess)
             e = launch_sweep(sweep_kind(p), p.rule, n, h->d_rp, h->d_adj, h->H, p, (int32_t)t,
@@ -1069,7 +1090,7 @@ pamc_status pamc_shard_sweep(pamc_handle h, const int64_t *E_all, const int32_t 
     }
     pamc_params pl = p;   // the sweep sees the own slots only
     pl.R = c;
-    SchedView sv{h->d_order, h->d_lvl, h->d_nlev, h->d_ell, h->d_pos, h->ell_w, h->d_nibc};
+    SchedView sv{h->d_order, h->d_lvl, h->d_nlev, h->d_ell, h->d_pos, h->ell_w, h->nib_halves};
     if (e == cudaSuccess) e = sweep_timer(h, false);
     if (e == cudaSuccess)
         e = launch_sweep(sweep_kind(p), p.rule, n, h->d_rp, h->d_adj, h->H, pl, (int32_t)t,
@@ -1620,7 +1641,7 @@ pamc_status rebuild(pamc_batch b) {
     std::vector<int2> swi[2][2][kClasses];   // Ising, spin words on chip [ell][rule][class]
     std::vector<int2> gswi[2][2][kClasses];  // Ising, spin words in device memory
     std::vector<int2> pswi[2][kClasses];     // Potts (cascaded sampler) [ell][class]
-    std::vector<int2> nswi[2][2][kClasses];  // Ising, 4-bit lanes (ELL rows) [biased][rule][class]
+    std::vector<int2> nswi[2][2][kClasses];  // Ising, 4-bit lanes (ELL rows) [two halves][rule][class]
     std::vector<NcmDesc> ncm;
     std::vector<int2> ncmi;
     std::vector<RedrawDesc> rds;
@@ -1632,7 +1653,7 @@ pamc_status rebuild(pamc_batch b) {
     // members whose field ranges fit 4-bit lanes take eight replicas a word, as alone
     auto member_nib = [&](pamc_handle h) {
         return h->p.kind == 0 && !member_global(h) &&
-               sweep_nibble_ok(h->H, h->p.sweeps, h->ell_w, 1, false, h->d_nibc != nullptr) && !sweep_push_enabled();
+               sweep_nibble_ok(h->nib_halves, h->p.sweeps, 1, false) && !sweep_push_enabled();
     };
     for (pamc_handle h : b->members)
         if (h->host_t < h->p.steps) {
@@ -1645,7 +1666,7 @@ pamc_status rebuild(pamc_batch b) {
     SweepCfg eff[kClasses], peff[kClasses], geff[kClasses], neff[kClasses];
     for (int c = 0; c < kClasses; ++c) {
         neff[c] = SweepCfg{b->shape[c].groups_per_cta, b->shape[c].warps_per_group, 1};
-        while (neff[c].groups_per_cta > 1 && sweep_nibble_smem_bytes(nnmax[c], kNibbleBiasedMaxH, neff[c]) > kSmemMax)
+        while (neff[c].groups_per_cta > 1 && sweep_nibble_smem_bytes(nnmax[c], kNibbleTwoMaxH, neff[c]) > kSmemMax)
             neff[c].groups_per_cta -= 1;
         geff[c] = SweepCfg{b->shape[c].groups_per_cta, b->shape[c].warps_per_group, 1};
         eff[c] = b->shape[c];
@@ -1706,7 +1727,6 @@ pamc_status rebuild(pamc_batch b) {
             return bfail(b, PAMC_ERR_OOM, "device allocation of a member's group spin words failed");
         d.gsp = gl ? h->d_gsp : nullptr;
         const bool nb = member_nib(h);
-        d.nibc = nb ? h->d_nibc : nullptr;
         const SweepCfg cfg = p.kind != 0 ? peff[cls] : gl ? geff[cls] : nb ? neff[cls] : eff[cls];
         d.push = p.kind == 0 && !gl && !nb && sweep_push_ok(h->H, p.sweeps, h->d_ell != nullptr, cfg.lanes_per_vertex)
                      ? 1 : 0;
@@ -1716,7 +1736,7 @@ pamc_status rebuild(pamc_batch b) {
         const int32_t ctas = (groups + cfg.groups_per_cta - 1) / cfg.groups_per_cta;
         // with sweeps = 0 the launch still copies the resampled population and its energies
         auto &items = p.kind != 0 ? pswi[h->d_ell != nullptr][cls]
-                                  : nb ? nswi[h->d_nibc != nullptr][p.rule][cls]
+                                  : nb ? nswi[h->nib_halves == 2][p.rule][cls]
                                        : (gl ? gswi : swi)[h->d_ell != nullptr][p.rule][cls];
         for (int32_t x = 0; x < ctas; ++x) items.push_back(make_int2(idx, x));
         Rmax = std::max(Rmax, p.R);

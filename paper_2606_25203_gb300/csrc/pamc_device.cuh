@@ -66,6 +66,33 @@ __device__ __forceinline__ u32x4 philox_rk(uint32_t c0, uint32_t c1, uint32_t c2
 }
 
 // ---------------------------------------------------------------------------
+// Position-indexed ELL rows of a schedule (width W, a multiple of 4): the
+// couplings of position i in 16-byte groups of four slots.  Group v of the 32
+// positions of a block lies in 512 contiguous bytes, so that a warp reads the
+// group of 32 consecutive positions with one coalesced 16-byte load a lane;
+// within the block the positions are permuted by v, so that the groups of one
+// position sit in different shared-memory banks when a block is staged there.
+// 32-bit offsets: n W < 2^32 (n < 2^24, W < 256).
+// ---------------------------------------------------------------------------
+__host__ __device__ __forceinline__ uint32_t ell_rot(uint32_t v) {
+    return ((v & 1u) << 2) | (v & 2u) | ((v >> 2) & 1u);
+}
+__host__ __device__ __forceinline__ uint32_t ell_word(uint32_t i, uint32_t W, uint32_t v) {
+    return (i & ~31u) * W + v * 128u + (((i & 31u) ^ ell_rot(v)) << 2);
+}
+__device__ __forceinline__ uint4 ell4(const uint32_t *es, int32_t i, int32_t W, uint32_t v) {
+    return *reinterpret_cast<const uint4 *>(es + ell_word((uint32_t)i, (uint32_t)W, v));
+}
+
+// A position's row sums in one word: sum_j J_kj (16 bits, signed), the weights
+// of the negative couplings in the slots 0..7 and 8..15 (4 bits each; exact
+// where the 4-bit lanes apply) and sum_j |J_kj| (8 bits; exact up to 127).
+__host__ __device__ __forceinline__ int32_t pos_sums(int32_t jsum, uint32_t neg0, uint32_t neg1, uint32_t habs) {
+    return (int32_t)(((uint32_t)jsum & 0xFFFFu) | (neg0 & 15u) << 16 | (neg1 & 15u) << 20 | (habs & 0xFFu) << 24);
+}
+__device__ __forceinline__ int32_t pos_jsum(int32_t y) { return (int32_t)(int16_t)(uint16_t)y; }
+
+// ---------------------------------------------------------------------------
 // Deterministic exp: x = k ln2 + r (Cody & Waite, with ln2 split into a
 // 32-significant-bit head and a tail), e^r by the degree-13 Taylor series in
 // Horner form with fused multiply-adds, result scaled by 2^k.  Constants are

@@ -130,28 +130,41 @@ schedule_body(int32_t n, const int32_t *__restrict__ rp, const uint32_t *__restr
     }
     // Position-indexed neighbour lists: order[i] becomes k | deg << 24 (deg =
     // nonzero couplings).  With an ELL buffer (width W, a multiple of 4) the
-    // couplings of position i go to ell[(i/32)*32*W + s*32 + i%32], s < deg,
-    // and the slots deg..W-1 hold 0 (vertex 0, coupling 0), so that a warp's
-    // lanes read consecutive words, the first four slots can be read before
-    // deg is known, and pos[i] = {k | deg << 24, sum_j J_kj}.
+    // couplings of position i go to the slots s < deg of its row (ell_word),
+    // and the slots deg..W-1 hold 0 (vertex 0, coupling 0), so that whole
+    // 16-byte groups can be read before deg is known, and pos[i] = {k | deg <<
+    // 24, row sums (pos_sums)}.
     uint32_t *es = ell ? ell + base * (size_t)(((n + 31) >> 5) << 5) * W : nullptr;
     int2 *ps = pos ? pos + base * (size_t)n : nullptr;
     for (int32_t i = threadIdx.x; i < n; i += blockDim.x) {
         const int32_t k = ord[i];
         int32_t d = 0, jsum = 0;
-        uint32_t *ep = es ? es + (size_t)(i >> 5) * 32 * W + (i & 31) : nullptr;
+        uint32_t habs = 0u, neg = 0u;   // sum |J|; negative weight of the slots 0..7 and 8..15 (4 bits each)
+        uint32_t g4[4] = {0u, 0u, 0u, 0u};
+        auto put = [&](int32_t v) {
+            *reinterpret_cast<uint4 *>(es + ell_word((uint32_t)i, (uint32_t)W, (uint32_t)v)) =
+                make_uint4(g4[0], g4[1], g4[2], g4[3]);
+            g4[0] = g4[1] = g4[2] = g4[3] = 0u;
+        };
         for (int32_t e = rp[k]; e < rp[k + 1]; ++e) {
             const uint32_t a = adj[e];
             const int32_t J = (int32_t)a >> 24;
             if (J == 0) continue;
-            if (ep) ep[(size_t)d * 32] = a;
+            const int32_t x = d & 3;
+            g4[0] = x == 0 ? a : g4[0];
+            g4[1] = x == 1 ? a : g4[1];
+            g4[2] = x == 2 ? a : g4[2];
+            g4[3] = x == 3 ? a : g4[3];
+            if (x == 3 && es) put(d >> 2);
+            habs += (uint32_t)(J < 0 ? -J : J);
+            if (J < 0 && d < 16) neg += (uint32_t)(-J) << (d < 8 ? 0 : 16);
             ++d;
             jsum += J;
         }
-        if (ep)
-            for (int32_t s2 = d; s2 < W; ++s2) ep[(size_t)s2 * 32] = 0u;
+        if (es)
+            for (int32_t v = d >> 2; v < W >> 2; ++v) put(v);   // the last couplings, then zeros
         ord[i] = k | (d << 24);
-        if (ps) ps[i] = make_int2(k | (d << 24), jsum);
+        if (ps) ps[i] = make_int2(k | (d << 24), pos_sums(jsum, neg & 0xFFFFu, neg >> 16, habs));
     }
 }
 

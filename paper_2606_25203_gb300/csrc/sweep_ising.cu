@@ -205,9 +205,8 @@ sweep_ising_push_body(int32_t n, int32_t n_pad, const int32_t *__restrict__ rp,
             uint32_t e4[4] = {0u, 0u, 0u, 0u};
             auto fetch = [&](int32_t i, int2 &r, uint32_t (&e)[4]) {
                 r = pos[i];
-                const uint32_t *ep = es + (size_t)(i >> 5) * 32 * W + (i & 31);
-#pragma unroll
-                for (int q = 0; q < 4; ++q) e[q] = ep[q * 32];
+                const uint4 v = ell4(es, i, W, 0);
+                e[0] = v.x; e[1] = v.y; e[2] = v.z; e[3] = v.w;
             };
             if (L > 0) fetch(min(li, n - 1), pr, e4);
             for (int32_t lev = 0; lev < L; ++lev) {
@@ -222,7 +221,7 @@ sweep_ising_push_body(int32_t n, int32_t n_pad, const int32_t *__restrict__ rp,
                     const uint32_t F = sp[k];
                     const u32x4 u = draw((uint32_t)k, (uint32_t)sw, (uint32_t)t, ctr3);
                     const uint32_t old = (F >> 7) & 0x01010101u;
-                    const uint32_t nw = ising_decide_push<RULE>(F, H - 128 - pr.y, u, tab_s, H);
+                    const uint32_t nw = ising_decide_push<RULE>(F, H - 128 - pos_jsum(pr.y), u, tab_s, H);
                     const uint32_t fl = nw ^ old;
                     if (fl != 0u) {
                         sp[k] = F ^ (fl << 7);
@@ -234,9 +233,8 @@ sweep_ising_push_body(int32_t n, int32_t n_pad, const int32_t *__restrict__ rp,
                         for (int q = 0; q < 4; ++q)   // padding slots: vertex 0, coupling 0
                             if (q < deg) atomicAdd(&sp[e4[q] & 0xFFFFFFu], delta * (uint32_t)((int32_t)e4[q] >> 24));
                         if (deg > 4) {
-                            const uint32_t *ep = es + (size_t)(i >> 5) * 32 * W + (i & 31);
                             for (int32_t sl = 4; sl < deg; ++sl) {
-                                const uint32_t e = ep[(size_t)sl * 32];
+                                const uint32_t e = es[ell_word((uint32_t)i, (uint32_t)W, (uint32_t)sl >> 2) + (sl & 3)];
                                 atomicAdd(&sp[e & 0xFFFFFFu], delta * (uint32_t)((int32_t)e >> 24));
                             }
                         }
@@ -261,7 +259,7 @@ sweep_ising_push_body(int32_t n, int32_t n_pad, const int32_t *__restrict__ rp,
             const uint32_t F = sp[p0.x & 0xFFFFFF];
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                const int32_t h = 2 * ((int32_t)((F >> (8 * q)) & 0x7Fu) - 64) - p0.y;
+                const int32_t h = 2 * ((int32_t)((F >> (8 * q)) & 0x7Fu) - 64) - pos_jsum(p0.y);
                 acc[q] += ((F >> (8 * q + 7)) & 1u) ? h : -h;
             }
         }
@@ -282,17 +280,18 @@ sweep_ising_push_body(int32_t n, int32_t n_pad, const int32_t *__restrict__ rp,
     if (active && li < 4 && r0 + li < R) E_dst[r0 + li] = -((long long)red[gl * 4 + li] / 2);
 }
 
-// Row i of a position-indexed ELL block of width W: lanes of a warp read
-// consecutive words (slot s of position i at (i & ~31) * W + 32 s + (i & 31)),
-// with 32-bit offset arithmetic (n W < 2^32: n < 2^24, W < 256).
-__device__ __forceinline__ const uint32_t *ell_row(const uint32_t *es, int32_t i, int32_t W) {
-    return es + ((uint32_t)(i & ~31) * (uint32_t)W + (uint32_t)(i & 31));
+// four couplings of a row on the neighbours' spin words
+__device__ __forceinline__ uint32_t add4(uint32_t A, const uint4 &e, const uint32_t *sp) {
+    A += sp[e.x & 0xFFFFFFu] * (uint32_t)((int32_t)e.x >> 24);
+    A += sp[e.y & 0xFFFFFFu] * (uint32_t)((int32_t)e.y >> 24);
+    A += sp[e.z & 0xFFFFFFu] * (uint32_t)((int32_t)e.z >> 24);
+    return A + sp[e.w & 0xFFFFFFu] * (uint32_t)((int32_t)e.w >> 24);
 }
 
 // The sweep of one CTA's replica groups (groups bid*gpc .. bid*gpc+gpc-1 of
 // the instance), shared by the single-instance and the batched kernels.  With
 // LPV > 1 (position-indexed ELL only; LPV a power of two up to 32) LPV lanes share a vertex: lane sub takes
-// the coupling slots sub, sub + LPV, ...; the byte-lane partial sums add up
+// the groups of four couplings sub, sub + LPV, ...; the byte-lane partial sums add up
 // exactly under XOR shuffles (plain 32-bit addition), and every lane of the
 // group runs the same iterations so that the shuffles always converge.
 template <bool ELLP, int RULE, int LPV, class KeyT, bool GSP = false, int WC = 0>
@@ -365,21 +364,19 @@ sweep_ising_body(int32_t n, int32_t n_pad, const int32_t *__restrict__ rp,
             const int2 *pos = ELLP ? spos + sb * (size_t)n : nullptr;
             const int32_t L = snlev[sb];
             if constexpr (ELLP && LPV > 1) {
-                // lane sub of a vertex takes the slots sub + LPV q; the record
-                // and the first eight slots of a pass are loaded ahead, for a
-                // level's first pass before the previous level's barrier
-                // (from a clamped position: they do not depend on spins)
-                const int32_t vl = li / LPV, sub = li % LPV, vpi = tpg / LPV;
+                // lane sub of a vertex takes the groups of four couplings sub +
+                // LPV q; the record and the first two groups of a pass are
+                // loaded ahead, for a level's first pass before the previous
+                // level's barrier (from a clamped position: they do not depend
+                // on spins)
+                const int32_t vl = li / LPV, sub = li % LPV, vpi = tpg / LPV, V = W >> 2;
+                const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
                 int2 pr;
-                uint32_t e8[8];
+                uint4 e0, e1;
                 auto fetch = [&](int32_t i) {
                     pr = pos[i];
-                    const uint32_t *ep = ell_row(es, i, W);
-#pragma unroll
-                    for (int q = 0; q < 8; ++q) {
-                        const int32_t sl = sub + q * LPV;   // slots >= deg hold coupling 0
-                        e8[q] = sl < W ? ep[(size_t)sl * 32] : 0u;
-                    }
+                    e0 = sub < V ? ell4(es, i, W, sub) : zero;   // slots >= deg hold coupling 0
+                    e1 = sub + LPV < V ? ell4(es, i, W, sub + LPV) : zero;
                 };
                 if (L > 0) fetch(min(vl, n - 1));
                 for (int32_t lev = 0; lev < L; ++lev) {
@@ -393,27 +390,19 @@ sweep_ising_body(int32_t n, int32_t n_pad, const int32_t *__restrict__ rp,
                         const int32_t k = pr.x & 0xFFFFFF;
                         const int32_t deg = (int32_t)((uint32_t)pr.x >> 24);
                         const u32x4 u = draw((uint32_t)k, (uint32_t)sw, (uint32_t)t, ctr3);
-                        uint32_t Ap = 0u;
-#pragma unroll
-                        for (int q = 0; q < 8; ++q) Ap += sp[e8[q] & 0xFFFFFFu] * (uint32_t)((int32_t)e8[q] >> 24);
-                        if (8 * LPV < deg) {
-                            const uint32_t *ep = ell_row(es, ic, W);
-                            for (int32_t s0 = sub + 8 * LPV; s0 < deg; s0 += 8 * LPV) {
-                                uint32_t ev[8];
-#pragma unroll
-                                for (int q = 0; q < 8; ++q) {
-                                    const int32_t sl = s0 + q * LPV;
-                                    ev[q] = sl < W ? ep[(size_t)sl * 32] : 0u;
-                                }
-#pragma unroll
-                                for (int q = 0; q < 8; ++q)
-                                    Ap += sp[ev[q] & 0xFFFFFFu] * (uint32_t)((int32_t)ev[q] >> 24);
-                            }
+                        uint32_t Ap = add4(0u, e0, sp);
+                        if (4 * (sub + LPV) < deg) Ap = add4(Ap, e1, sp);
+                        for (int32_t v = sub + 2 * LPV; 4 * v < deg; v += 2 * LPV) {
+                            const uint4 f0 = ell4(es, ic, W, v);
+                            uint4 f1 = zero;
+                            if (4 * (v + LPV) < deg) f1 = ell4(es, ic, W, v + LPV);
+                            Ap = add4(Ap, f0, sp);
+                            if (4 * (v + LPV) < deg) Ap = add4(Ap, f1, sp);
                         }
 #pragma unroll
                         for (int o = 1; o < LPV; o <<= 1) Ap += __shfl_xor_sync(0xffffffffu, Ap, o);
                         const uint32_t old = sp[k];
-                        const uint32_t nw = ising_decide<RULE>(0x80808080u + Ap, H - 256 - pr.y, u, old, tab_s, H);
+                        const uint32_t nw = ising_decide<RULE>(0x80808080u + Ap, H - 256 - pos_jsum(pr.y), u, old, tab_s, H);
                         // every lane has read sp[k] before any lane of the group writes it
                         __syncwarp();
                         if (act && sub == 0 && nw != old) {
@@ -431,30 +420,32 @@ sweep_ising_body(int32_t n, int32_t n_pad, const int32_t *__restrict__ rp,
             // position before the previous level's barrier (they do not
             // depend on spins), so the wait overlaps the barrier
             int2 pr = make_int2(0, 0);
-            uint32_t e4[4] = {0u, 0u, 0u, 0u};
+            uint4 e4 = make_uint4(0u, 0u, 0u, 0u);
             int32_t end = 0;
             if (ELLP && L > 0) {
                 // unconditional, from a clamped position: whether it is used is
                 // decided once the level's bounds are known
                 const int32_t i0 = min(li, n - 1);
                 pr = pos[i0];
-                const uint32_t *ep = ell_row(es, i0, W);
-#pragma unroll
-                for (int q = 0; q < 4; ++q) e4[q] = ep[q * 32];
+                e4 = ell4(es, i0, W, 0);
             }
             for (int32_t lev = 0; lev < L; ++lev) {
                 const int32_t beg = lp[lev];
                 end = lp[lev + 1];
                 int32_t i = beg + li;
+                int32_t kc = 0, re0 = 0, re1 = 0;   // CSR rows: the position's vertex and its row
+                if (!ELLP && i < end) {
+                    kc = ord[i] & 0xFFFFFF;
+                    re0 = rp[kc];
+                    re1 = rp[kc + 1];
+                }
                 while (i < end) {
                     const int32_t inext = i + tpg;
                     int2 prn = make_int2(0, 0);
-                    uint32_t e4n[4] = {0u, 0u, 0u, 0u};
+                    uint4 e4n = make_uint4(0u, 0u, 0u, 0u);
                     if (ELLP && inext < end) {
                         prn = pos[inext];
-                        const uint32_t *epn = ell_row(es, inext, W);
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) e4n[q] = epn[q * 32];
+                        e4n = ell4(es, inext, W, 0);
                     }
                     // A: byte q = 128 + sum_j J_kj [s_j = +1] of replica q
                     uint32_t A = 0x80808080u;
@@ -464,99 +455,68 @@ sweep_ising_body(int32_t n, int32_t n_pad, const int32_t *__restrict__ rp,
                         const uint32_t a0 = (uint32_t)pr.x;
                         k = (int32_t)(a0 & 0xFFFFFFu);
                         const int32_t deg = (int32_t)(a0 >> 24);
-                        jsum = pr.y;
+                        jsum = pos_jsum(pr.y);
                         // the next neighbour words are requested before the draw is
                         // computed, so that the Philox rounds overlap their latency
                         if (W <= 4) {   // every neighbour word is already in registers
-#pragma unroll
-                            for (int q = 0; q < 4; ++q)   // padding slots: coupling 0
-                                A += sp[e4[q] & 0xFFFFFFu] * (uint32_t)((int32_t)e4[q] >> 24);
+                            A = add4(A, e4, sp);   // padding slots: coupling 0
                             u = draw((uint32_t)k, (uint32_t)sw, (uint32_t)t, ctr3);
                         } else if constexpr (WC > 0 && WC <= 16) {
-                        const uint32_t *ep = ell_row(es, i, W) + 4 * 32;
-                        // rows of at most sixteen slots (compile-time width):
-                        // the words beyond the first four in blocks of four,
-                        // all in flight before the draw (a level's positions
-                        // are grouped by degree, so a warp's lanes mostly
-                        // agree on how many blocks they need)
-                        uint32_t ev[4], ew[4], ex[4];
-                        if (deg > 4) {
-#pragma unroll
-                            for (int q = 0; q < 4; ++q) ev[q] = (4 + q < W) ? ep[q * 32] : 0u;
-                        }
-                        if (deg > 8) {
-#pragma unroll
-                            for (int q = 0; q < 4; ++q) ew[q] = (8 + q < W) ? ep[(4 + q) * 32] : 0u;
-                        }
-                        if (deg > 12) {
-#pragma unroll
-                            for (int q = 0; q < 4; ++q) ex[q] = (12 + q < W) ? ep[(8 + q) * 32] : 0u;
-                        }
-                        u = draw((uint32_t)k, (uint32_t)sw, (uint32_t)t, ctr3);
-#pragma unroll
-                        for (int q = 0; q < 4; ++q)   // padding slots: coupling 0
-                            A += sp[e4[q] & 0xFFFFFFu] * (uint32_t)((int32_t)e4[q] >> 24);
-                        if (deg > 4) {
-#pragma unroll
-                            for (int q = 0; q < 4; ++q)
-                                A += sp[ev[q] & 0xFFFFFFu] * (uint32_t)((int32_t)ev[q] >> 24);
-                        }
-                        if (deg > 8) {
-#pragma unroll
-                            for (int q = 0; q < 4; ++q)
-                                A += sp[ew[q] & 0xFFFFFFu] * (uint32_t)((int32_t)ew[q] >> 24);
-                        }
-                        if (deg > 12) {
-#pragma unroll
-                            for (int q = 0; q < 4; ++q)
-                                A += sp[ex[q] & 0xFFFFFFu] * (uint32_t)((int32_t)ex[q] >> 24);
-                        }
+                            // rows of at most sixteen slots (compile-time width):
+                            // the groups beyond the first all in flight before
+                            // the draw (a level's positions are grouped by
+                            // degree, so a warp's lanes mostly agree on how many
+                            // they need)
+                            uint4 ev, ew, ex;
+                            if (deg > 4) ev = ell4(es, i, W, 1);
+                            if (WC > 8 && deg > 8) ew = ell4(es, i, W, 2);
+                            if (WC > 12 && deg > 12) ex = ell4(es, i, W, 3);
+                            u = draw((uint32_t)k, (uint32_t)sw, (uint32_t)t, ctr3);
+                            A = add4(A, e4, sp);
+                            if (deg > 4) A = add4(A, ev, sp);
+                            if (WC > 8 && deg > 8) A = add4(A, ew, sp);
+                            if (WC > 12 && deg > 12) A = add4(A, ex, sp);
                         } else {
-                        const uint32_t *ep = ell_row(es, i, W) + 4 * 32;
-                        // up to sixteen more neighbour words in flight before the draw
-                        uint32_t ev[8], ew[8];
-                        if (deg > 4) {
+                            // up to sixteen more neighbour words in flight before
+                            // the draw, in groups of four as the degree asks
+                            // (levels are grouped by degree, so a warp's lanes
+                            // mostly agree on how many they need)
+                            uint4 ev[4];
 #pragma unroll
-                            for (int q = 0; q < 8; ++q) ev[q] = (4 + q < W) ? ep[q * 32] : 0u;
-                        }
-                        if (deg > 12) {
+                            for (int q = 0; q < 4; ++q)
+                                if (deg > 4 + 4 * q) ev[q] = ell4(es, i, W, 1 + q);
+                            u = draw((uint32_t)k, (uint32_t)sw, (uint32_t)t, ctr3);
+                            A = add4(A, e4, sp);
 #pragma unroll
-                            for (int q = 0; q < 8; ++q) ew[q] = (12 + q < W) ? ep[(8 + q) * 32] : 0u;
-                        }
-                        u = draw((uint32_t)k, (uint32_t)sw, (uint32_t)t, ctr3);
-#pragma unroll
-                        for (int q = 0; q < 4; ++q)   // padding slots: coupling 0
-                            A += sp[e4[q] & 0xFFFFFFu] * (uint32_t)((int32_t)e4[q] >> 24);
-                        if (deg > 4) {
-#pragma unroll
-                            for (int q = 0; q < 8; ++q)
-                                A += sp[ev[q] & 0xFFFFFFu] * (uint32_t)((int32_t)ev[q] >> 24);
-                        }
-                        if (deg > 12) {
-#pragma unroll
-                            for (int q = 0; q < 8; ++q)
-                                A += sp[ew[q] & 0xFFFFFFu] * (uint32_t)((int32_t)ew[q] >> 24);
-                        }
-                        for (int32_t b0 = 20; b0 < deg; b0 += 8) {
-                            ep += (b0 == 20 ? 16 : 8) * 32;
-#pragma unroll
-                            for (int q = 0; q < 8; ++q) ev[q] = (b0 + q < W) ? ep[q * 32] : 0u;
-#pragma unroll
-                            for (int q = 0; q < 8; ++q)
-                                A += sp[ev[q] & 0xFFFFFFu] * (uint32_t)((int32_t)ev[q] >> 24);
-                        }
+                            for (int q = 0; q < 4; ++q)
+                                if (deg > 4 + 4 * q) A = add4(A, ev[q], sp);
+                            for (int32_t v = 5; 4 * v < deg; ++v) A = add4(A, ell4(es, i, W, v), sp);
                         }
                     } else {
-                        k = ord[i] & 0xFFFFFF;
+                        // CSR rows, eight couplings in flight; the next position's
+                        // vertex and row bounds are on their way
+                        k = kc;
                         jsum = 0;
-                        for (int32_t e = rp[k]; e < rp[k + 1]; ++e) {
-                            const uint32_t a = adj[e];
-                            const int32_t J = (int32_t)a >> 24;
-                            A += sp[a & 0xFFFFFFu] * (uint32_t)J;
-                            jsum += J;
+                        const int32_t e1 = re1;
+                        int32_t e = re0;
+                        if (inext < end) {
+                            kc = ord[inext] & 0xFFFFFF;
+                            re0 = rp[kc];
+                            re1 = rp[kc + 1];
+                        }
+                        u = draw((uint32_t)k, (uint32_t)sw, (uint32_t)t, ctr3);
+                        for (; e < e1; e += 8) {
+                            uint32_t a[8];
+#pragma unroll
+                            for (int q = 0; q < 8; ++q) a[q] = e + q < e1 ? adj[e + q] : 0u;
+#pragma unroll
+                            for (int q = 0; q < 8; ++q) {
+                                const int32_t J = (int32_t)a[q] >> 24;
+                                A += sp[a[q] & 0xFFFFFFu] * (uint32_t)J;
+                                jsum += J;
+                            }
                         }
                     }
-                    if (!ELLP) u = draw((uint32_t)k, (uint32_t)sw, (uint32_t)t, ctr3);
                     const uint32_t old = sp[k];
                     const uint32_t nw = ising_decide<RULE>(A, H - 256 - jsum, u, old, tab_s, H);
                     if (nw != old) {
@@ -565,15 +525,12 @@ sweep_ising_body(int32_t n, int32_t n_pad, const int32_t *__restrict__ rp,
                     }
                     i = inext;
                     pr = prn;
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) e4[q] = e4n[q];
+                    e4 = e4n;
                 }
                 if (ELLP && lev + 1 < L) {   // the next level's first position (clamped, see above)
                     const int32_t i2 = min(end + li, n - 1);
                     pr = pos[i2];
-                    const uint32_t *ep = ell_row(es, i2, W);
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) e4[q] = ep[q * 32];
+                    e4 = ell4(es, i2, W, 0);
                 }
                 group_barrier(1 + gl, tpg, gpc);
             }
@@ -590,32 +547,22 @@ sweep_ising_body(int32_t n, int32_t n_pad, const int32_t *__restrict__ rp,
             const uint32_t *es = sell + sb * ell_stride;
             const int2 *pos = spos + sb * (size_t)n;
             int2 pr = make_int2(0, 0);
-            uint32_t e4[4] = {0u, 0u, 0u, 0u};
+            uint4 e4 = make_uint4(0u, 0u, 0u, 0u);
             auto fetch = [&](int32_t i) {
                 pr = pos[i];
-                const uint32_t *ep = ell_row(es, i, W);
-#pragma unroll
-                for (int q = 0; q < 4; ++q) e4[q] = q < W ? ep[q * 32] : 0u;
+                e4 = ell4(es, i, W, 0);
             };
             if (li < n) fetch(li);
             for (int32_t i = li; i < n; i += tpg) {
                 const int2 p0 = pr;
-                uint32_t A = 0x80808080u;
-#pragma unroll
-                for (int q = 0; q < 4; ++q) A += sp[e4[q] & 0xFFFFFFu] * (uint32_t)((int32_t)e4[q] >> 24);
+                uint32_t A = add4(0x80808080u, e4, sp);
                 if (i + tpg < n) fetch(i + tpg);
                 const int32_t deg = (int32_t)((uint32_t)p0.x >> 24);
-                if (deg > 4) {
-                    const uint32_t *ep = ell_row(es, i, W);
-                    for (int32_t sl = 4; sl < deg; ++sl) {
-                        const uint32_t e = ep[(size_t)sl * 32];
-                        A += sp[e & 0xFFFFFFu] * (uint32_t)((int32_t)e >> 24);
-                    }
-                }
+                for (int32_t v = 1; 4 * v < deg; ++v) A = add4(A, ell4(es, i, W, v), sp);
                 const uint32_t w = sp[p0.x & 0xFFFFFF];
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
-                    const int32_t h = 2 * ((int32_t)((A >> (8 * q)) & 0xFFu) - 128) - p0.y;   // p0.y = sum_j J_kj
+                    const int32_t h = 2 * ((int32_t)((A >> (8 * q)) & 0xFFu) - 128) - pos_jsum(p0.y);
                     acc[q] += ((w >> (8 * q)) & 1u) ? h : -h;
                 }
             }

@@ -7,23 +7,31 @@
 // group's words take the same 4n bytes of shared memory for twice the
 // replicas.
 //
-// Fixed bias (sum_j |J_kj| <= 7 for every vertex: the +-1 torus, graphs of
-// degree <= 7; ELL width 4 or 8).  A = 0x88888888 + sum_j J_kj word_j has
-// nibble q = 8 + sum_j J_kj [s_j = +1] in [1, 15]: no nibble carries or
-// borrows, so h_q + H = 2 nibble_q(A) + c0, c0 = H - 16 - sum_j J_kj, indexes
-// the threshold table as in the byte-lane kernel.
+// Satisfied weight.  With M the weight of the negative couplings of a half-row
+// (ELL slots 0..7 or 8..15), A = M 0x11111111 + sum_{j in half} J_kj word_j has
+// nibble q = N_q = sum_{J > 0} J [s_j = +1] + sum_{J < 0} |J| [s_j = -1], in
+// [0, 15] wherever the half's sum |J| <= 15 (every partial sum stays in range,
+// so the word sums exactly), and h_q = 2 N_q - D, D = sum_j |J_kj|.  One half
+// (D <= 7 on rows of at most eight slots: the +-1 torus, graphs of degree <= 7)
+// keeps the nibbles; two halves are added in byte lanes (sums <= 30).  M, M'
+// and D come with the position's record (pos_sums).
 //
-// Biased lanes (ELL width up to 16; sum |J| <= 15 over the slots 0..7 and
-// over the slots 8..15 of every vertex: +-1 graphs of degree <= 16, such as
-// sparse random graphs of mean degree 6).  With M the weight of the negative
-// couplings of a half, A_half = M 0x11111111 + sum_{j in half} J_kj word_j
-// has nibble q = N_q = sum_{J > 0} J [s_j = +1] + sum_{J < 0} |J| [s_j = -1]
-// in [0, 15] (the satisfied weight of the half; every partial sum stays in
-// range, so the word sums exactly), and h_q = 2 (N1_q + N2_q) - sum_j |J_kj|.
-// The two halves are added in byte lanes (even and odd nibbles apart, sums
-// <= 30), and h_q + H = 2 (N1_q + N2_q) + c0 with c0 = H - sum_j |J_kj|.  The
-// per-vertex constants (M1 0x11111111, M2 0x11111111, c0) are computed once
-// per instance.
+// Decision.  For a vertex of weight D the new spin depends on the draw and an
+// index x in [0, D], the threshold rising with x: heat-bath x = N (s = +1 iff
+// u < T(2x - D)), Metropolis x = the unsatisfied weight D - N for s = +1, N for
+// s = -1 (flip iff u < T_M(D - 2x)).  Shared memory holds a row of 32-bit
+// thresholds for each D, 256 bytes apart, so that the address of a replica's
+// entry is the row address with its lowest byte replaced by 4 x: one byte
+// permute.  A threshold of 2^32 (always) does not fit 32 bits: those entries
+// hold 2^32 - 1, and the replicas with x at or beyond the first such entry are
+// set by one addition over the word (nibble or byte x + 8 - x_f, + 128 - x_f:
+// the top bit).  A decision then takes a permute, a shared load, a compare and
+// a predicated addition.
+//
+// Bound: the integer pipe (half the issue rate), Philox about a third of it:
+// 247 instructions a visit of eight replicas (260 with biased field lanes and
+// 64-bit thresholds, whose launches took 1,247 us against 1,138 on the
+// 141 x 141 torus, R = 4,096, 10 sweeps).
 //
 // Draws.  Replica r uses word r mod 4 of Philox(k, sweep, t, FLIP<<24 | r/4)
 // as everywhere else: the eight replicas of a word take two calls, of the
@@ -65,63 +73,71 @@ __device__ __forceinline__ void nib_barrier(int id, int nthreads, int groups) {
     }
 }
 
-__device__ __forceinline__ const uint32_t *nib_ell_row(const uint32_t *es, int32_t i, int32_t W) {
-    return es + ((uint32_t)(i & ~31) * (uint32_t)W + (uint32_t)(i & 31));
+// four couplings of a row on the neighbours' spin words
+__device__ __forceinline__ uint32_t nib_add4(uint32_t A, const uint4 &e, const uint32_t *sp) {
+    A += sp[e.x & 0xFFFFFFu] * (uint32_t)((int32_t)e.x >> 24);
+    A += sp[e.y & 0xFFFFFFu] * (uint32_t)((int32_t)e.y >> 24);
+    A += sp[e.z & 0xFFFFFFu] * (uint32_t)((int32_t)e.z >> 24);
+    return A + sp[e.w & 0xFFFFFFu] * (uint32_t)((int32_t)e.w >> 24);
 }
 
-// New eight-replica word from the nibble accumulator A, c0 = H - 16 -
-// sum_j J_kj, the draws of the two four-replica groups and the old word.
-template <int RULE>
-__device__ __forceinline__ uint32_t ising_decide8(uint32_t A, int32_t c0, const u32x4 &ua, const u32x4 &ub,
-                                                  uint32_t old, const uint64_t *tab_s, int32_t H) {
-    const uint32_t uw[8] = {ua.x, ua.y, ua.z, ua.w, ub.x, ub.y, ub.z, ub.w};
-    uint32_t nw = 0;
-    // heat-bath: entry h + H = 2 nibble + c0 sits 16 * nibble bytes past
-    // tab_s + c0, and 16 * nibble is nibble q of A moved to bits 4..7
-    const char *tp = reinterpret_cast<const char *>(tab_s + c0);
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-        const int32_t idx = 2 * (int32_t)((A >> (4 * q)) & 0xFu) + c0;   // h + H
-        if (RULE == 0) {
-            const uint32_t off = q == 0 ? (A << 4) & 0xF0u : (A >> (4 * q - 4)) & 0xF0u;
-            const uint64_t T = *reinterpret_cast<const uint64_t *>(tp + off);
-            nw |= ((uint64_t)uw[q] < T ? 1u : 0u) << (4 * q);
-        } else {
-            const uint32_t s = (old >> (4 * q)) & 1u;
-            const int32_t ix = s ? idx : 2 * H - idx;              // s*h + H
-            nw |= (((uint64_t)uw[q] < tab_s[ix]) ? (s ^ 1u) : s) << (4 * q);
-        }
-    }
-    return nw;
+__device__ __forceinline__ uint32_t lds_u32(uint32_t addr) {
+    uint32_t v;
+    asm("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr));
+    return v;
+}
+// w + bit where u < T
+__device__ __forceinline__ void add_if_below(uint32_t &w, uint32_t u, uint32_t T, uint32_t bit) {
+    asm("{\n .reg .pred p;\n setp.lt.u32 p, %1, %2;\n @p add.u32 %0, %0, %3;\n}" : "+r"(w) : "r"(u), "r"(T), "r"(bit));
 }
 
-// Biased lanes: the same from the byte-lane sums E (even nibbles: replica
-// 2b in byte b) and O (odd nibbles: replica 2b + 1), each N1_q + N2_q in
-// [0, 30], and c0 = H - sum_j |J_kj|.
-template <int RULE>
-__device__ __forceinline__ uint32_t ising_decide8b(uint32_t E, uint32_t O, int32_t c0, const u32x4 &ua,
-                                                   const u32x4 &ub, uint32_t old, const uint64_t *tab_s,
-                                                   int32_t H) {
-    const uint32_t uw[8] = {ua.x, ua.y, ua.z, ua.w, ub.x, ub.y, ub.z, ub.w};
-    uint32_t nw = 0;
-    // heat-bath: entry h + H = 2 N + c0 sits 16 N bytes past tab_s + c0
-    const char *tp = reinterpret_cast<const char *>(tab_s + c0);
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-        const uint32_t src = (q & 1) ? O : E;
-        const int b = q >> 1;
-        if (RULE == 0) {
-            const uint32_t off = b == 0 ? (src << 4) & 0x1F0u : (src >> (8 * b - 4)) & 0x1F0u;
-            const uint64_t T = *reinterpret_cast<const uint64_t *>(tp + off);
-            nw |= ((uint64_t)uw[q] < T ? 1u : 0u) << (4 * q);
+// bytes of the threshold rows and, per row, the word that marks the entries of
+// 2^32: rows D = 0..H, 256 bytes apart (the row address has a clear low byte)
+constexpr int32_t kNibRow = 64;
+__host__ __device__ constexpr size_t nib_table_bytes(int32_t H) { return (size_t)(H + 1) * (kNibRow * 4 + 4) + 12 + 256; }
+
+// The decisions of eight replicas: E, O the index of the even and the odd
+// replicas in bytes, row the address of the vertex's thresholds, force its
+// mark word, X the index nibbles (one half only).
+template <int RULE, bool TWO>
+__device__ __forceinline__ uint32_t nib_decide(uint32_t X, uint32_t E, uint32_t O, uint32_t D, uint32_t row,
+                                               uint32_t force, const u32x4 &ua, const u32x4 &ub, uint32_t old) {
+    if constexpr (RULE == 1) {   // the unsatisfied weight of the replicas with s = +1
+        if constexpr (TWO) {
+            const uint32_t me = (old & 0x01010101u) * 0xFFu, mo = ((old >> 4) & 0x01010101u) * 0xFFu;
+            const uint32_t D4 = D * 0x01010101u;
+            E = (E & ~me) | ((D4 - E) & me);
+            O = (O & ~mo) | ((D4 - O) & mo);
         } else {
-            const int32_t idx = 2 * (int32_t)((src >> (8 * b)) & 0xFFu) + c0;   // h + H
-            const uint32_t s = (old >> (4 * q)) & 1u;
-            const int32_t ix = s ? idx : 2 * H - idx;                         // s*h + H
-            nw |= (((uint64_t)uw[q] < tab_s[ix]) ? (s ^ 1u) : s) << (4 * q);
+            const uint32_t m = old * 0xFu;
+            X = (X & ~m) | ((D * 0x11111111u - X) & m);
         }
     }
-    return nw;
+    uint32_t e4, o4;   // 4 x of the even and the odd replicas, in bytes
+    if constexpr (TWO) {
+        e4 = E << 2;
+        o4 = O << 2;
+    } else {
+        e4 = (X << 2) & 0x3C3C3C3Cu;
+        o4 = (X >> 2) & 0x3C3C3C3Cu;
+    }
+    const uint32_t uw[8] = {ua.x, ua.y, ua.z, ua.w, ub.x, ub.y, ub.z, ub.w};
+    uint32_t n0 = 0u, n1 = 0u;
+#pragma unroll
+    for (int q = 0; q < 8; q += 2) {
+        const uint32_t te = lds_u32(__byte_perm(e4, row, 0x7650u + (q >> 1)));
+        const uint32_t to = lds_u32(__byte_perm(o4, row, 0x7650u + (q >> 1)));
+        add_if_below(n0, uw[q], te, 1u << (4 * q));
+        add_if_below(n1, uw[q + 1], to, 16u << (4 * q));
+    }
+    uint32_t nw = n0 | n1;
+    if constexpr (TWO) {
+        nw |= ((E + force) >> 7) & 0x01010101u;
+        nw |= ((O + force) >> 3) & 0x10101010u;
+    } else {
+        nw |= ((X + force) >> 3) & 0x11111111u;
+    }
+    return RULE == 1 ? nw ^ old : nw;
 }
 
 __device__ __forceinline__ void nib_halves(uint32_t A1, uint32_t A2, uint32_t &E, uint32_t &O) {
@@ -131,9 +147,9 @@ __device__ __forceinline__ void nib_halves(uint32_t A1, uint32_t A2, uint32_t &E
 
 // The sweeps of one CTA's groups of eight (groups bid*gpc .. bid*gpc+gpc-1
 // of the instance), shared by the single-instance and the batched kernels;
-// WC = 0: the ELL width read at run time; BIASED: the biased lanes (width 4
-// to 16, per-vertex constants d.nibc), else the fixed bias (width 4 or 8).
-template <int RULE, int WC, bool BIASED, class KeyT>
+// WC = 0: the ELL width read at run time; TWO: both halves of the rows (width 4
+// to 16), else one (width 4 or 8).
+template <int RULE, int WC, bool TWO, class KeyT>
 __device__ __forceinline__ void
 nib_body(const SweepDesc &d, const KeyT &draw, int32_t t, int32_t slot, const int8_t *__restrict__ src,
          int8_t *__restrict__ dst, int64_t *__restrict__ E_dst, int gpc, int tpg, int32_t bid) {
@@ -142,11 +158,26 @@ nib_body(const SweepDesc &d, const KeyT &draw, int32_t t, int32_t slot, const in
     if (ctl->done) return;
     const int32_t n = d.n, n_pad = d.n_pad, H = d.H, R = d.R, S = d.S;
     const int32_t W = WC > 0 ? WC : d.W;
-    const int tabn = 2 * H + 1;
-    uint64_t *tab_s = reinterpret_cast<uint64_t *>(smem);
-    uint32_t *spins_all = reinterpret_cast<uint32_t *>(smem + (((size_t)tabn * 8 + 15) & ~(size_t)15));
+    // threshold rows at the first 256-byte boundary, the marks behind them
+    const uint32_t smem0 = (uint32_t)__cvta_generic_to_shared(smem);
+    const uint32_t rows0 = (smem0 + 255u) & ~255u;
+    uint32_t *tab_s = reinterpret_cast<uint32_t *>(smem + (rows0 - smem0));
+    uint32_t *mark_s = tab_s + (H + 1) * kNibRow;
+    const uint32_t marks0 = rows0 + (uint32_t)(H + 1) * (kNibRow * 4);
+    uint32_t *spins_all = reinterpret_cast<uint32_t *>(smem + ((nib_table_bytes(H) + 15) & ~(size_t)15));
     unsigned long long *red = reinterpret_cast<unsigned long long *>(spins_all + (size_t)gpc * n_pad);
-    for (int i = threadIdx.x; i < tabn; i += blockDim.x) tab_s[i] = d.tab[i];
+    for (int i = threadIdx.x; i < (H + 1) * (H + 1); i += blockDim.x) {
+        const int32_t D = i / (H + 1), x = i % (H + 1);
+        if (x > D) continue;
+        // tab[h + H] (heat-bath), tab[s h + H] (Metropolis): h = 2x - D, s h = D - 2x
+        const uint64_t T = d.tab[RULE == 0 ? 2 * x - D + H : D - 2 * x + H];
+        tab_s[D * kNibRow + x] = T > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)T;
+    }
+    for (int32_t D = threadIdx.x; D <= H; D += blockDim.x) {
+        int32_t xf = 0;   // first entry of 2^32 (D + 1: none)
+        while (xf <= D && d.tab[RULE == 0 ? 2 * xf - D + H : D - 2 * xf + H] <= 0xFFFFFFFFull) ++xf;
+        mark_s[D] = TWO ? (uint32_t)(128 - xf) * 0x01010101u : (uint32_t)(8 - xf) * 0x11111111u;
+    }
     for (int i = threadIdx.x; i < gpc * 8; i += blockDim.x) red[i] = 0ull;
 
     const int gl = threadIdx.x / tpg, li = threadIdx.x % tpg;
@@ -192,21 +223,18 @@ nib_body(const SweepDesc &d, const KeyT &draw, int32_t t, int32_t slot, const in
             const uint32_t *es = d.sell + sb * ell_stride;
             const int2 *pos = d.spos + sb * (size_t)n;
             const int32_t L = d.snlev[sb];
-            // the record and the first four neighbour words of a position are
-            // loaded one iteration ahead -- for a level's first position before
-            // the previous level's barrier (they do not depend on spins)
-            // (biased lanes: and the vertex's constants)
+            // the record and the first four couplings of a position (the first
+            // eight where the rows have more) are loaded one iteration ahead --
+            // for a level's first position before the previous level's barrier
+            // (they do not depend on spins)
             int2 pr = make_int2(0, 0);
-            uint32_t e4[4] = {0u, 0u, 0u, 0u};
-            int4 nc = make_int4(0, 0, 0, 0);
+            uint4 e4 = make_uint4(0u, 0u, 0u, 0u), f4 = e4;
             int32_t end = 0;
             if (L > 0) {
                 const int32_t i0 = min(li, n - 1);
                 pr = pos[i0];
-                const uint32_t *ep = nib_ell_row(es, i0, W);
-#pragma unroll
-                for (int q = 0; q < 4; ++q) e4[q] = ep[q * 32];
-                if constexpr (BIASED) nc = d.nibc[pr.x & 0xFFFFFF];
+                e4 = ell4(es, i0, W, 0);
+                if (W > 4) f4 = ell4(es, i0, W, 1);
             }
             for (int32_t lev = 0; lev < L; ++lev) {
                 const int32_t beg = lp[lev];
@@ -215,80 +243,51 @@ nib_body(const SweepDesc &d, const KeyT &draw, int32_t t, int32_t slot, const in
                 while (i < end) {
                     const int32_t inext = i + tpg;
                     int2 prn = make_int2(0, 0);
-                    uint32_t e4n[4] = {0u, 0u, 0u, 0u};
-                    int4 ncn = make_int4(0, 0, 0, 0);
+                    uint4 e4n = make_uint4(0u, 0u, 0u, 0u), f4n = e4n;
                     if (inext < end) {
                         prn = pos[inext];
-                        const uint32_t *epn = nib_ell_row(es, inext, W);
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) e4n[q] = epn[q * 32];
-                        if constexpr (BIASED) ncn = d.nibc[prn.x & 0xFFFFFF];
+                        e4n = ell4(es, inext, W, 0);
+                        if (W > 4) f4n = ell4(es, inext, W, 1);
                     }
                     const uint32_t a0 = (uint32_t)pr.x;
                     const int32_t k = (int32_t)(a0 & 0xFFFFFFu);
-                    uint32_t A = BIASED ? (uint32_t)nc.x : 0x88888888u;
-                    if (W > 4) {   // slots 4..7 (padding slots hold coupling 0)
-                        const uint32_t *ep = nib_ell_row(es, i, W) + 4 * 32;
-                        uint32_t ev[4];
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) ev[q] = ep[q * 32];
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) A += sp[ev[q] & 0xFFFFFFu] * (uint32_t)((int32_t)ev[q] >> 24);
-                    }
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) A += sp[e4[q] & 0xFFFFFFu] * (uint32_t)((int32_t)e4[q] >> 24);
-                    uint32_t A2 = 0u;
-                    if constexpr (BIASED) {
-                        // slots 8..15 into the second half, in blocks of four
+                    const uint32_t ys = (uint32_t)pr.y;
+                    uint32_t A = ((ys >> 16) & 15u) * 0x11111111u, A2 = 0u;
+                    A = nib_add4(A, e4, sp);   // (padding slots: coupling 0)
+                    if (W > 4) A = nib_add4(A, f4, sp);
+                    if constexpr (TWO) {
+                        // slots 8..15 into the second half, in groups of four
                         // while the degree asks for them (levels are grouped
                         // by degree, so a warp's lanes mostly agree)
-                        A2 = (uint32_t)nc.y;
+                        A2 = ((ys >> 20) & 15u) * 0x11111111u;
                         const int32_t deg = (int32_t)(a0 >> 24);
                         if (W > 8 && deg > 8) {
-                            const uint32_t *ep = nib_ell_row(es, i, W) + 8 * 32;
-                            uint32_t ev[4];
-#pragma unroll
-                            for (int q = 0; q < 4; ++q) ev[q] = ep[q * 32];
-#pragma unroll
-                            for (int q = 0; q < 4; ++q)
-                                A2 += sp[ev[q] & 0xFFFFFFu] * (uint32_t)((int32_t)ev[q] >> 24);
-                            if (W > 12 && deg > 12) {
-#pragma unroll
-                                for (int q = 0; q < 4; ++q) ev[q] = ep[(4 + q) * 32];
-#pragma unroll
-                                for (int q = 0; q < 4; ++q)
-                                    A2 += sp[ev[q] & 0xFFFFFFu] * (uint32_t)((int32_t)ev[q] >> 24);
-                            }
+                            A2 = nib_add4(A2, ell4(es, i, W, 2), sp);
+                            if (W > 12 && deg > 12) A2 = nib_add4(A2, ell4(es, i, W, 3), sp);
                         }
                     }
                     const u32x4 ua = draw((uint32_t)k, (uint32_t)sw, (uint32_t)t, ctrA);
                     const u32x4 ub = draw((uint32_t)k, (uint32_t)sw, (uint32_t)t, ctrB);
                     const uint32_t old = sp[k];
-                    uint32_t nw;
-                    if constexpr (BIASED) {
-                        uint32_t E, O;
-                        nib_halves(A, A2, E, O);
-                        nw = ising_decide8b<RULE>(E, O, nc.z, ua, ub, old, tab_s, H);
-                    } else {
-                        nw = ising_decide8<RULE>(A, H - 16 - pr.y, ua, ub, old, tab_s, H);
-                    }
+                    const uint32_t D = ys >> 24;
+                    const uint32_t row = rows0 + (D << 8), force = lds_u32(marks0 + (D << 2));
+                    uint32_t E = 0u, O = 0u;
+                    if constexpr (TWO) nib_halves(A, A2, E, O);
+                    const uint32_t nw = nib_decide<RULE, TWO>(A, E, O, D, row, force, ua, ub, old);
                     if (nw != old) {
                         sp[k] = nw;
                         nflip += __popc((nw ^ old) & live);
                     }
                     i = inext;
                     pr = prn;
-                    nc = ncn;
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) e4[q] = e4n[q];
+                    e4 = e4n;
+                    f4 = f4n;
                 }
                 if (lev + 1 < L) {   // the next level's first position (clamped, see above)
                     const int32_t i2 = min(end + li, n - 1);
                     pr = pos[i2];
-                    const uint32_t *ep = nib_ell_row(es, i2, W);
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) e4[q] = ep[q * 32];
-                    if constexpr (BIASED) nc = d.nibc[pr.x & 0xFFFFFF];
+                    e4 = ell4(es, i2, W, 0);
+                    if (W > 4) f4 = ell4(es, i2, W, 1);
                 }
                 nib_barrier(1 + gl, tpg, gpc);
             }
@@ -308,35 +307,20 @@ nib_body(const SweepDesc &d, const KeyT &draw, int32_t t, int32_t slot, const in
         const int2 *pos = d.spos + sb * (size_t)n;
         for (int32_t i = li; i < n; i += tpg) {
             const int2 p0 = pos[i];
-            const uint32_t *ep = nib_ell_row(es, i, W);
             const uint32_t w = sp[p0.x & 0xFFFFFF];
-            if constexpr (BIASED) {
-                const int4 c = d.nibc[p0.x & 0xFFFFFF];
-                uint32_t A = (uint32_t)c.x, A2 = (uint32_t)c.y;
-                for (int q = 0; q < W; ++q) {
-                    const uint32_t e = ep[q * 32];
-                    const uint32_t v = sp[e & 0xFFFFFFu] * (uint32_t)((int32_t)e >> 24);
-                    if (q < 8) A += v;
-                    else A2 += v;
-                }
+            const uint32_t ys = (uint32_t)p0.y;
+            const int32_t D = (int32_t)(ys >> 24);
+            uint32_t A = ((ys >> 16) & 15u) * 0x11111111u, A2 = TWO ? ((ys >> 20) & 15u) * 0x11111111u : 0u;
 #pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                    const int32_t nq = (int32_t)((A >> (4 * q)) & 0xFu) + (int32_t)((A2 >> (4 * q)) & 0xFu);
-                    const int32_t h = 2 * nq + c.z - H;   // c.z = H - sum_j |J_kj|
-                    acc[q] += ((w >> (4 * q)) & 1u) ? h : -h;
-                }
-            } else {
-                uint32_t A = 0x88888888u;
+            for (int v = 0; v < (TWO ? 4 : 2); ++v) {
+                if (4 * v >= W) break;
+                if (v < 2) A = nib_add4(A, ell4(es, i, W, v), sp);
+                else A2 = nib_add4(A2, ell4(es, i, W, v), sp);
+            }
 #pragma unroll
-                for (int q = 0; q < W; ++q) {
-                    const uint32_t e = ep[q * 32];
-                    A += sp[e & 0xFFFFFFu] * (uint32_t)((int32_t)e >> 24);
-                }
-#pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                    const int32_t h = 2 * ((int32_t)((A >> (4 * q)) & 0xFu) - 8) - p0.y;   // p0.y = sum_j J_kj
-                    acc[q] += ((w >> (4 * q)) & 1u) ? h : -h;
-                }
+            for (int q = 0; q < 8; ++q) {
+                const int32_t h = 2 * (int32_t)(((A >> (4 * q)) & 0xFu) + ((A2 >> (4 * q)) & 0xFu)) - D;
+                acc[q] += ((w >> (4 * q)) & 1u) ? h : -h;
             }
         }
         for (int32_t k = li; k < n; k += tpg) {
@@ -356,21 +340,21 @@ nib_body(const SweepDesc &d, const KeyT &draw, int32_t t, int32_t slot, const in
     if (active && li < 8 && r0 + li < R) E_dst[r0 + li] = -((long long)red[gl * 8 + li] / 2);
 }
 
-template <int RULE, int WC, bool BIASED>
+template <int RULE, int WC, bool TWO>
 __global__ void __launch_bounds__(1024) k_sweep_ising_nib(SweepDesc d, int gpc, int tpg) {
-    nib_body<RULE, WC, BIASED>(d, NibKeys{d.K}, d.t, d.slot, d.src, d.dst, d.E_dst, gpc, tpg, blockIdx.x);
+    nib_body<RULE, WC, TWO>(d, NibKeys{d.K}, d.t, d.slot, d.src, d.dst, d.E_dst, gpc, tpg, blockIdx.x);
 }
 
 // Many instances in one launch: CTA b works on member items[b].x, its block
 // of groups items[b].y; the step index comes from the member's controller.
-template <int RULE, bool BIASED>
+template <int RULE, bool TWO>
 __global__ void __launch_bounds__(1024)
 k_sweep_ising_nib_batched(const SweepDesc *__restrict__ descs, const int2 *__restrict__ items, int gpc, int tpg) {
     const int2 it = items[blockIdx.x];
     const SweepDesc &d = descs[it.x];
     const int32_t t = d.ctl->t;
     if (t >= d.t_end) return;
-    nib_body<RULE, 0, BIASED>(d, NibKeysSeed{d.K.k0[0], d.K.k1[0]}, t, t % d.slots, d.sp[t & 1],
+    nib_body<RULE, 0, TWO>(d, NibKeysSeed{d.K.k0[0], d.K.k1[0]}, t, t % d.slots, d.sp[t & 1],
                               d.sp[(t + 1) & 1], d.en[(t + 1) & 1], gpc, tpg, it.y);
 }
 
@@ -381,36 +365,29 @@ bool sweep_nibble_enabled() {
     return !(env && env[0] == '0');
 }
 
-bool sweep_nibble_ok(int32_t H, int32_t S, int32_t ell_w, int lanes_per_vertex, bool global_spins,
-                     bool biased_ok) {
-    const bool fixed = H <= kNibbleMaxH && (ell_w == 4 || ell_w == 8);
-    return (fixed || biased_ok) && S > 0 && lanes_per_vertex == 1 && !global_spins && sweep_nibble_enabled();
-}
-
-bool nibble_biased_constants(int32_t n, const int32_t *rp, const uint32_t *adj, int32_t H, int32_t ell_w,
-                             std::vector<int4> &out) {
-    if (!(ell_w == 4 || ell_w == 8 || ell_w == 12 || ell_w == 16) || H > kNibbleBiasedMaxH) return false;
-    out.assign((size_t)n, make_int4(0, 0, 0, 0));
+int nibble_halves(int32_t n, const int32_t *rp, const uint32_t *adj, int32_t H, int32_t ell_w) {
+    if (H <= kNibbleMaxH && (ell_w == 4 || ell_w == 8)) return 1;
+    if (!(ell_w == 4 || ell_w == 8 || ell_w == 12 || ell_w == 16) || H > kNibbleTwoMaxH) return 0;
     for (int32_t k = 0; k < n; ++k) {
-        int32_t slot = 0, half[2] = {0, 0}, neg[2] = {0, 0};
+        int32_t slot = 0, half[2] = {0, 0};
         for (int32_t e = rp[k]; e < rp[k + 1]; ++e) {
             const int32_t J = (int32_t)adj[e] >> 24;
             if (J == 0) continue;   // the ELL rows hold the nonzero couplings only
-            const int hf = slot < 8 ? 0 : 1;
-            half[hf] += J < 0 ? -J : J;
-            neg[hf] += J < 0 ? -J : 0;
+            half[slot < 8 ? 0 : 1] += J < 0 ? -J : J;
             ++slot;
         }
-        if (slot > ell_w || half[0] > kNibbleHalfMaxH || half[1] > kNibbleHalfMaxH) return false;
-        out[k] = make_int4((int32_t)((uint32_t)neg[0] * 0x11111111u), (int32_t)((uint32_t)neg[1] * 0x11111111u),
-                           H - half[0] - half[1], 0);
+        if (slot > ell_w || half[0] > kNibbleHalfMaxH || half[1] > kNibbleHalfMaxH) return 0;
     }
-    return true;
+    return 2;
+}
+
+bool sweep_nibble_ok(int halves, int32_t S, int lanes_per_vertex, bool global_spins) {
+    return halves > 0 && S > 0 && lanes_per_vertex == 1 && !global_spins && sweep_nibble_enabled();
 }
 
 size_t sweep_nibble_smem_bytes(int32_t n, int32_t H, SweepCfg cfg) {
     const int32_t n_pad = (n + 3) & ~3;
-    return (((size_t)(2 * H + 1) * 8 + 15) & ~(size_t)15) + (size_t)cfg.groups_per_cta * n_pad * 4 +
+    return ((nib_table_bytes(H) + 15) & ~(size_t)15) + (size_t)cfg.groups_per_cta * n_pad * 4 +
            (size_t)cfg.groups_per_cta * 8 * 8;
 }
 
@@ -418,10 +395,10 @@ cudaError_t launch_sweep_ising_nib(int rule, int32_t n, int32_t H, const pamc_pa
                                    SchedView sv, const uint64_t *tab, const int8_t *src, const int32_t *parent,
                                    const int8_t *ncm_buf, const int32_t *ncm_idx, int8_t *dst, int64_t *E_dst,
                                    const DevCtl *ctl, SweepCfg cfg, cudaStream_t st, int32_t rbase) {
-    const bool biased = sv.nibc != nullptr;
+    const bool two = sv.halves == 2;
     if (!(sv.ell != nullptr && p.sweeps > 0 &&
-          (biased ? (sv.W % 4 == 0 && sv.W >= 4 && sv.W <= 16 && H <= kNibbleBiasedMaxH)
-                  : ((sv.W == 4 || sv.W == 8) && H <= kNibbleMaxH))))
+          (two ? (sv.W % 4 == 0 && sv.W >= 4 && sv.W <= 16 && H <= kNibbleTwoMaxH)
+               : (sv.halves == 1 && (sv.W == 4 || sv.W == 8) && H <= kNibbleMaxH))))
         return cudaErrorInvalidValue;
     const int32_t groups = (p.R + 7) / 8;
     const int gpc = cfg.groups_per_cta, tpg = cfg.warps_per_group * 32;
@@ -432,7 +409,6 @@ cudaError_t launch_sweep_ising_nib(int rule, int32_t n, int32_t H, const pamc_pa
     d.dst = dst; d.E_dst = E_dst; d.ctl = ctl; d.n = n; d.n_pad = (n + 3) & ~3; d.H = H; d.R = p.R;
     d.S = p.sweeps; d.t = t; d.slot = slot; d.W = sv.W; d.K = make_philox_keys(p.seed);
     d.gbase = rbase / 4;
-    d.nibc = sv.nibc;
     const size_t smem = sweep_nibble_smem_bytes(n, H, cfg);
     const int grid = (groups + gpc - 1) / gpc;
     cudaError_t err = cudaSuccess;
@@ -444,7 +420,7 @@ cudaError_t launch_sweep_ising_nib(int rule, int32_t n, int32_t H, const pamc_pa
     } while (0)
 #define PAMC_NIB_W(RU)                                                                       \
     do {                                                                                     \
-        if (!biased) {                                                                       \
+        if (!two) {                                                                       \
             if (sv.W == 4) PAMC_NIB(RU, 4, false);                                           \
             else PAMC_NIB(RU, 8, false);                                                     \
         } else if (sv.W == 4) PAMC_NIB(RU, 4, true);                                         \
@@ -459,11 +435,11 @@ cudaError_t launch_sweep_ising_nib(int rule, int32_t n, int32_t H, const pamc_pa
     return cudaGetLastError();
 }
 
-cudaError_t launch_sweep_ising_nib_batched(int rule, bool biased, const SweepDesc *descs, const int2 *items,
+cudaError_t launch_sweep_ising_nib_batched(int rule, bool two, const SweepDesc *descs, const int2 *items,
                                            int32_t nitems, int32_t n_max, SweepCfg cfg, cudaStream_t st) {
     if (nitems <= 0) return cudaSuccess;
     const int gpc = cfg.groups_per_cta, tpg = cfg.warps_per_group * 32;
-    const size_t smem = sweep_nibble_smem_bytes(n_max, biased ? kNibbleBiasedMaxH : kNibbleMaxH, cfg);
+    const size_t smem = sweep_nibble_smem_bytes(n_max, two ? kNibbleTwoMaxH : kNibbleMaxH, cfg);
     cudaError_t err;
 #define PAMC_NIBB(RU, BI)                                                                    \
     do {                                                                                     \
@@ -472,10 +448,10 @@ cudaError_t launch_sweep_ising_nib_batched(int rule, bool biased, const SweepDes
         k_sweep_ising_nib_batched<RU, BI><<<nitems, gpc * tpg, smem, st>>>(descs, items, gpc, tpg); \
     } while (0)
     if (rule == 0) {
-        if (biased) PAMC_NIBB(0, true);
+        if (two) PAMC_NIBB(0, true);
         else PAMC_NIBB(0, false);
     } else {
-        if (biased) PAMC_NIBB(1, true);
+        if (two) PAMC_NIBB(1, true);
         else PAMC_NIBB(1, false);
     }
 #undef PAMC_NIBB

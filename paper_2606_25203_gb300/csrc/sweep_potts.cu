@@ -14,8 +14,8 @@
 // from the position-indexed ELL of the schedule when it exists, else from CSR.
 //
 // Lane pairs (PAIR, ELL rows): two lanes share a position.  Lane s runs the
-// Philox call of replicas 2s and 2s + 1 and sums the coupling slots of its
-// parity; one shuffle adds the two partial byte-lane sums (one of them
+// Philox call of replicas 2s and 2s + 1 and sums every second group of
+// four couplings; one shuffle adds the two partial byte-lane sums (one of them
 // carries the bias) and one more ORs the two halves of the new label word.
 // The draws and decisions are those of the one-lane body.
 #include "pamc_device.cuh"
@@ -36,6 +36,18 @@ __device__ __forceinline__ void potts_barrier(int id, int nthreads, int groups) 
 // one-hot words of four byte labels (0..2)
 __device__ __forceinline__ uint2 onehot(uint32_t labels) {
     return make_uint2(__vcmpeq4(labels, 0u) & 0x01010101u, __vcmpeq4(labels, 0x01010101u) & 0x01010101u);
+}
+
+// four couplings of a row on the neighbours' one-hot words
+__device__ __forceinline__ void potts_add4(uint32_t &A0, uint32_t &A1, const uint4 &e, const uint2 *oh) {
+    const uint32_t w[4] = {e.x, e.y, e.z, e.w};
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const uint2 o = oh[w[q] & 0xFFFFFFu];
+        const uint32_t J = (uint32_t)((int32_t)w[q] >> 24);
+        A0 += o.x * J;
+        A1 += o.y * J;
+    }
 }
 
 // The sweeps of one CTA's replica groups (groups bid*gpc .. bid*gpc+gpc-1 of
@@ -104,30 +116,20 @@ potts_body(int32_t n, int32_t n_pad, const int32_t *__restrict__ rp, const uint3
                         const bool valid = iv < end;
                         const int32_t i = valid ? iv : end - 1;
                         const int2 pr = pos[i];
-                        const uint32_t *ep = es + (size_t)(i >> 5) * 32 * W + (i & 31);
-                        uint32_t ev[8];
+                        // groups of four couplings sl and sl + 2
+                        uint4 ev[2];
 #pragma unroll
-                        for (int q = 0; q < 8; ++q) ev[q] = 2 * q + sl < W ? ep[(2 * q + sl) * 32] : 0u;
+                        for (int q = 0; q < 2; ++q)
+                            ev[q] = 4 * (2 * q + sl) < W ? ell4(es, i, W, 2 * q + sl) : make_uint4(0u, 0u, 0u, 0u);
                         const int32_t k = pr.x & 0xFFFFFF;
                         const int32_t deg = (int32_t)((uint32_t)pr.x >> 24);
-                        const int32_t jsum = pr.y;
+                        const int32_t jsum = pos_jsum(pr.y);
                         const u32x4 u = philox((uint32_t)k, (uint32_t)sw, (uint32_t)t,
                                                (kTagFlip << 24) | (uint32_t)(2 * gk + sl), key0, key1);
                         uint32_t A0 = sl ? 0u : 0x80808080u, A1 = sl ? 0u : 0x80808080u;
-#pragma unroll
-                        for (int q = 0; q < 8; ++q) {
-                            const uint2 o = oh[ev[q] & 0xFFFFFFu];
-                            const uint32_t J = (uint32_t)((int32_t)ev[q] >> 24);
-                            A0 += o.x * J;
-                            A1 += o.y * J;
-                        }
-                        for (int32_t b0 = 16; b0 < deg; b0 += 4) {   // W >= deg rounded up to 4
-                            const uint32_t ew0 = ep[(b0 + sl) * 32], ew1 = ep[(b0 + 2 + sl) * 32];
-                            const uint2 o0 = oh[ew0 & 0xFFFFFFu], o1 = oh[ew1 & 0xFFFFFFu];
-                            const uint32_t J0 = (uint32_t)((int32_t)ew0 >> 24), J1 = (uint32_t)((int32_t)ew1 >> 24);
-                            A0 += o0.x * J0 + o1.x * J1;
-                            A1 += o0.y * J0 + o1.y * J1;
-                        }
+                        potts_add4(A0, A1, ev[0], oh);
+                        potts_add4(A0, A1, ev[1], oh);
+                        for (int32_t v = 4 + sl; 4 * v < deg; v += 2) potts_add4(A0, A1, ell4(es, i, W, v), oh);
                         A0 += __shfl_xor_sync(0xffffffffu, A0, 1);
                         A1 += __shfl_xor_sync(0xffffffffu, A1, 1);
                         uint32_t lab = 0u;
@@ -162,36 +164,20 @@ potts_body(int32_t n, int32_t n_pad, const int32_t *__restrict__ rp, const uint3
                         // the record, then up to sixteen coupling words in flight while
                         // the two Philox calls run (padding slots: coupling 0)
                         const int2 pr = pos[i];
-                        const uint32_t *ep = es + (size_t)(i >> 5) * 32 * W + (i & 31);
-                        uint32_t ev[16];
+                        uint4 ev[4];
 #pragma unroll
-                        for (int q = 0; q < 16; ++q) ev[q] = q < W ? ep[q * 32] : 0u;
+                        for (int q = 0; q < 4; ++q)
+                            ev[q] = 4 * q < W ? ell4(es, i, W, q) : make_uint4(0u, 0u, 0u, 0u);
                         k = pr.x & 0xFFFFFF;
                         const int32_t deg = (int32_t)((uint32_t)pr.x >> 24);
-                        jsum = pr.y;
+                        jsum = pos_jsum(pr.y);
                         ua = philox((uint32_t)k, (uint32_t)sw, (uint32_t)t, (kTagFlip << 24) | (uint32_t)(2 * gk),
                                     key0, key1);
                         ub = philox((uint32_t)k, (uint32_t)sw, (uint32_t)t, (kTagFlip << 24) | (uint32_t)(2 * gk + 1),
                                     key0, key1);
 #pragma unroll
-                        for (int q = 0; q < 16; ++q) {
-                            const uint2 o = oh[ev[q] & 0xFFFFFFu];
-                            const uint32_t J = (uint32_t)((int32_t)ev[q] >> 24);
-                            A0 += o.x * J;
-                            A1 += o.y * J;
-                        }
-                        for (int32_t b0 = 16; b0 < deg; b0 += 4) {
-                            uint32_t ew[4];
-#pragma unroll
-                            for (int q = 0; q < 4; ++q) ew[q] = ep[(b0 + q) * 32];
-#pragma unroll
-                            for (int q = 0; q < 4; ++q) {
-                                const uint2 o = oh[ew[q] & 0xFFFFFFu];
-                                const uint32_t J = (uint32_t)((int32_t)ew[q] >> 24);
-                                A0 += o.x * J;
-                                A1 += o.y * J;
-                            }
-                        }
+                        for (int q = 0; q < 4; ++q) potts_add4(A0, A1, ev[q], oh);
+                        for (int32_t v = 4; 4 * v < deg; ++v) potts_add4(A0, A1, ell4(es, i, W, v), oh);
                     } else {
                         k = ord[i] & 0xFFFFFF;
                         jsum = 0;

@@ -126,14 +126,17 @@ __global__ void __launch_bounds__(1024) k_sweep_ising_wide(SweepDesc d, int gpc,
                         const int2 pr = pos[i];
                         k = pr.x & 0xFFFFFF;
                         const int32_t deg = (int32_t)((uint32_t)pr.x >> 24);
-                        jsum = pr.y;
-                        const uint32_t *ep = es + (size_t)(i >> 5) * 32 * W + (i & 31);
-                        for (int32_t s = 0; s < deg; ++s) {
-                            const uint32_t e = ep[(size_t)s * 32];
-                            const uint2 w = sp[e & 0xFFFFFFu];
-                            const uint32_t J = (uint32_t)((int32_t)e >> 24);
-                            A.x += w.x * J;
-                            A.y += w.y * J;
+                        jsum = pos_jsum(pr.y);
+                        for (int32_t v = 0; 4 * v < deg; ++v) {
+                            const uint4 e4 = ell4(es, i, W, v);
+                            const uint32_t e[4] = {e4.x, e4.y, e4.z, e4.w};
+#pragma unroll
+                            for (int s = 0; s < 4; ++s) {   // padding slots: coupling 0
+                                const uint2 w = sp[e[s] & 0xFFFFFFu];
+                                const uint32_t J = (uint32_t)((int32_t)e[s] >> 24);
+                                A.x += w.x * J;
+                                A.y += w.y * J;
+                            }
                         }
                     } else {
                         k = ord[i] & 0xFFFFFF;

@@ -186,6 +186,36 @@ def test_lanes_per_vertex_default_choice(pg, monkeypatch):
         assert (lpv > 1) == want_many, (inst.name, lpv)
 
 
+@pytest.mark.parametrize("cfg", ["1,1,1,1", "1,2,2,1", "1,3,8,1", "1,8,4,1"])
+def test_staged_sweep(pg, monkeypatch, cfg):
+    """The staged sweep (rows and draws through a ring in shared memory, two
+    sets of warps taking the passes in turn) at its edges, against the oracle:
+    levels shorter and longer than a pass, a last block of one position, a
+    ring that wraps, rows beyond what a lane reads ahead, a ragged group, byte
+    and 16-bit fields, thresholds in shared and in global memory, both rules;
+    and by default for small populations."""
+    wide = W.gnm(257, 900, signed=True, seed=3)
+    e = np.repeat(np.arange(wide.n), np.diff(wide.row_ptr))
+    wide.w = (wide.w * (1 + (np.minimum(e, wide.col) * 7 + np.maximum(e, wide.col)) % 127)).astype(np.int32)
+    dense = W.csr_from_edges(41, *np.triu_indices(41, 1), np.full(41 * 20, 99), "k41w99")
+    cases = [(W.gnm(33, 60, seed=5), 5, 0), (W.torus(20, 20, seed=2), 4, 1), (W.erdos_renyi(300, 0.2, seed=1), 13, 0),
+             (wide, 6, 1), (dense, 3, 0)]   # (H = 3,960: its thresholds are read from global memory)
+    for inst, R, rule in cases:
+        p = dict(R=R, sweeps=3, beta0=0.2, beta1=2.0, rule=rule, seed=9)
+        monkeypatch.setenv("PAMC_SWEEP_CFG", cfg)
+        s = pg.Solver(inst.row_ptr, inst.col, inst.w)
+        s.init(steps=4, **p)
+        assert tuple(pg.pamc_sweep_shape(s.h)[:3]) == tuple(int(x) for x in cfg.split(",")[:3])
+        s.step(4)
+        ref = oracle.OracleRun(inst.row_ptr, inst.col, inst.w, steps=4, **p)
+        ref.step(4)
+        assert pg.pamc_sweep_stats(s.h)["flips"] == ref.sweep_flips(), inst.name
+        s.close()
+        compare_run(pg, inst, 4, **p)
+        monkeypatch.delenv("PAMC_SWEEP_CFG")
+        compare_run(pg, inst, 3, **p)
+
+
 def test_independent_chains_baseline(pg):
     inst = W.gnm(400, 1100, signed=True, seed=6)
     compare_run(pg, inst, 6, R=9, sweeps=2, resample=0, seed=1)
