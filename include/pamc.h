@@ -159,14 +159,17 @@ pamc_status pamc_control_history(pamc_handle h, int64_t *hist, int32_t *hist_len
 int64_t pamc_launch_count(pamc_handle h);
 
 /* Launch shape the sparse sweep of an initialised run uses: replica groups
- * per CTA (four replicas each; eight on 4-bit lanes, see pamc_sweep_mode),
+ * per CTA (four replicas each; eight on 4-bit lanes, up to 32 with one bit a
+ * replica, see pamc_sweep_mode),
  * warps per group, and lanes that share one position: Ising runs on ELL
  * schedules split a vertex's couplings over 1-32 lanes; Max-3-Cut runs take
  * lane pairs with the cascaded sampler on ELL schedules (each lane one
  * Philox call, half the couplings and two replicas' decisions) and quads
  * with the softmax sampler (one replica each); 1 otherwise.  Set by
  * pamc_init from the schedule's level widths, or by the environment variable
- * PAMC_SWEEP_CFG="gpc,wpg[,lpv]".  The shape changes speed only, never
+ * PAMC_SWEEP_CFG="gpc,wpg[,lpv]" (on ELL rows also "1,wpg,lpv,1", the staged
+ * sweep of small populations, wpg its consumer warps, and "1,wpg,lpv,0,q", one
+ * bit a replica, 4q replicas a group).  The shape changes speed only, never
  * results.  PAMC_ERR_STATE before pamc_init or for dense runs. */
 pamc_status pamc_sweep_shape(pamc_handle h, int *groups_per_cta, int *warps_per_group, int *lanes_per_vertex);
 
@@ -183,7 +186,10 @@ pamc_status pamc_sweep_shape(pamc_handle h, int *groups_per_cta, int *warps_per_
  * words in shared memory, at least one sweep, and either sum_j |w_ij| <= 7
  * per vertex on rows of width 4 or 8, or at most 15 over each vertex's first
  * eight nonzero couplings in CSR order and over the rest, on rows up to 16
- * wide; off with PAMC_SWEEP_NIBBLE=0).  Speed only, never results.
+ * wide; off with PAMC_SWEEP_NIBBLE=0), plus 32 when a word holds one bit a
+ * replica (couplings +-1, at most 63 neighbours, ELL rows, spin words in
+ * shared memory, at least one sweep, and a population large enough; off with
+ * PAMC_SWEEP_NIBBLE=0).  Speed only, never results.
  * PAMC_ERR_STATE before pamc_init or for dense or Potts runs. */
 pamc_status pamc_sweep_mode(pamc_handle h, int *mode);
 
@@ -286,8 +292,9 @@ int pamc_size_class(int32_t n);
 /* Launch shape of the batched sweep for one size class: replica groups (of
  * four replicas) per CTA and warps per group, groups * warps <= 32.  Where the
  * class's largest member needs it, fewer groups per CTA are used so that the
- * spins fit shared memory.  The shape changes speed only, never results.
- * Takes effect at the next pamc_batch_step.  PAMC_ERR_ARG when out of range. */
+ * spins fit shared memory.  Members that could take one bit a replica have a
+ * shape of their own unless the class's was set here (or by PAMC_BATCH_CFG).
+ * The shape changes speed only, never results.  Takes effect at the next pamc_batch_step.  PAMC_ERR_ARG when out of range. */
 pamc_status pamc_batch_set_shape(pamc_batch b, int size_class, int groups_per_cta, int warps_per_group);
 pamc_status pamc_batch_get_shape(pamc_batch b, int size_class, int *groups_per_cta, int *warps_per_group);
 /* Lanes that share one vertex's couplings in the batched Ising sweep of a size

@@ -372,7 +372,8 @@ def pamc_sweep_shape(h) -> tuple:
 
 
 def pamc_sweep_mode(h) -> int:
-    """0 pull over CSR rows, 1 pull over ELL rows, 2 push (fields kept and updated on flips)."""
+    """0 pull over CSR rows, 1 pull over ELL rows, 2 push (fields kept and updated on flips);
+    plus 4 spin words in device memory, 8 16-bit lanes, 16 4-bit lanes, 32 one bit a replica."""
     v = ctypes.c_int(0)
     _check(_lib.pamc_sweep_mode(h, ctypes.byref(v)), h)
     return v.value

@@ -6,12 +6,14 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <array>
 #include <climits>
 #include <cstdarg>
 #include <cstdio>
 #include <cmath>
 #include <cstdlib>
 #include <cstring>
+#include <map>
 #include <new>
 #include <string>
 #include <tuple>
@@ -83,6 +85,8 @@ struct pamc_handle_s {
     // instance
     int32_t *d_rp = nullptr;
     uint32_t *d_adj = nullptr;
+    double avg_level = 1.0;    // vertices in an average dependency level of the run's schedules
+    bool bits_ok = false;      // couplings +-1 on ELL rows: one bit a replica applies
     int nib_halves = 0;        // half-rows of the 4-bit lanes (0: they do not apply)
     // run
     pamc_params p{};
@@ -436,6 +440,44 @@ cudaError_t dense_recompute(pamc_handle h, const int8_t *src, const int32_t *par
                                   h->stream, restart_t);
 }
 
+// Lanes a vertex and warps of a group on one bit a replica (sweep_bits.cu): one
+// lane where an average level has 256 vertices or more, else four, which also
+// share the long rows' sums; warps for a level's lanes, 16 (two CTAs an SM) at
+// most where the SMs hold several groups.  us per launch of 10 sweeps, 1 lane / 2 / 4:
+// N=7,000 degree 5.7 R=4,096 (levels of 350) 510 / 589 / 780, N=10,007 degree 20
+// R=2,048 (196) 1,645 / 1,250 / 1,150, N=2,000 degree 20 R=4,096 (40) 1,309 / 865 / 481.
+SweepCfg bits_shape(double avg_level, int nc, bool one_group) {
+    SweepCfg c{1, 4, avg_level >= 256.0 ? 1 : 4, 0, nc};
+    const double lanes = avg_level * c.lanes_per_vertex;
+    c.warps_per_group = lanes >= 1024.0 && one_group ? 32 : lanes >= 256.0 ? 16 : lanes >= 128.0 ? 8 : 4;
+    return c;
+}
+
+// One bit a replica in a single run: as many groups as SMs (or a multiple), so
+// that a word holds the replicas an SM has to sweep anyway.  A word of few
+// replicas spends its time on the sum and the planes: from two quads on it
+// beats the byte lanes, from three on (and wide levels) the 4-bit lanes.  us per
+// launch of 10 sweeps, 4-bit lanes / bits: 141 x 141 torus R=1,024 (two quads) 323 /
+// 396, R=1,500 (three) 585 / 478, R=4,096 (seven) 1,139 / 820; byte lanes /
+// bits: N=2,000 degree 20 R=1,024 (two) 456 / 413, N=10,007 degree 20 R=1,100
+// (two) 1,136 / 1,138, R=4,096 (seven) 2,962 / 1,335.  Narrow levels stay with the
+// 4-bit lanes where these apply (N=1,024 torus, R=2,700: 106 / 122).
+bool bits_pay(int nc, double avg_level, bool nib) { return nib ? nc >= 3 && avg_level >= 256.0 : nc >= 2; }
+SweepCfg bits_cfg(int32_t n, int32_t R, int32_t H, double avg_level, int sms, bool nib) {
+    SweepCfg c{1, 1, 1, 0, 0};
+    if (const char *env = getenv("PAMC_SWEEP_CFG")) {   // "1,warps,lanes,0,quads" forces it
+        int a = 0, b = 0, v = 0, st = 0, nc = 0;
+        if (sscanf(env, "%d,%d,%d,%d,%d", &a, &b, &v, &st, &nc) == 5 && !st && nc >= 1 && nc <= 8 && a == 1 && b >= 1 &&
+            b <= 32 && (v == 1 || v == 2 || v == 4) && sweep_bits_smem_bytes(n, H) <= kSmemMax)
+            c = SweepCfg{a, b, v, 0, nc};
+        return c;
+    }
+    const int32_t per_sm = (R + 32 * sms - 1) / (32 * sms);
+    const int nc = (R + 4 * sms * per_sm - 1) / (4 * sms * per_sm);
+    if (!bits_pay(nc, avg_level, nib) || sweep_bits_smem_bytes(n, H) > kSmemMax) return c;
+    return bits_shape(avg_level, nc, per_sm == 1);
+}
+
 // own: the replicas this handle sweeps (base: the first one's index in the
 // whole population of p.R); own = p.R unless the population is split.
 pamc_status init_dense(pamc_handle h, pamc_params p, int32_t base, int32_t own, bool split) {
@@ -608,6 +650,7 @@ pamc_status pamc_create_csr(int32_t n, const int32_t *row_ptr, const int32_t *co
     // (the schedule's position record holds the degree in 8 bits)
     const int64_t ell_entries = (int64_t)((n + 31) / 32) * 32 * ((maxdeg + 3) & ~3);
     h->ell_w = (maxdeg > 0 && maxdeg < 256 && ell_entries <= 4 * (int64_t)h->nnz + 4096) ? ((maxdeg + 3) & ~3) : 0;
+    h->bits_ok = bits_apply(n, row_ptr, adj.data(), H, h->ell_w);
     h->nib_halves = h->ell_w > 0 ? nibble_halves(n, row_ptr, adj.data(), H, h->ell_w) : 0;
     if (!alloc_n(h, h->d_rp, (size_t)n + 1, h->inst_bufs) ||
         !alloc_n(h, h->d_adj, (size_t)std::max(h->nnz, 1), h->inst_bufs)) {
@@ -818,6 +861,7 @@ static pamc_status init_run(pamc_handle h, const pamc_params *pp, int32_t rank, 
         if (e != cudaSuccess) return cuda_fail(h, e, "schedule depth readback");
         avg_level = (double)n / std::max(depth, 1);
     }
+    h->avg_level = avg_level;
     int sms = 152;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
     h->cfg = choose_cfg(sweep_kind(p), n, own, h->H, avg_level, (double)h->nnz / std::max(n, 1), sms, h->ell_w);
@@ -843,10 +887,15 @@ static pamc_status init_run(pamc_handle h, const pamc_params *pp, int32_t rank, 
         }
         h->gsp = true;
     }
+    if (p.kind == 0 && p.sweeps > 0 && h->bits_ok && !h->gsp && !h->cfg.staged && sweep_nibble_enabled() &&
+        !sweep_push_enabled() && !(genv && genv[0] == '1')) {
+        const SweepCfg c = bits_cfg(n, own, h->H, avg_level, sms, nib_ok);
+        if (c.bits) h->cfg = c;
+    }
     // field ranges of at most 7 on ELL rows of width 4 or 8, or of 15 a
     // half-row on rows up to 16 wide: eight replicas a word (groups of eight,
     // shaped like a population of half the size)
-    if (nib_ok && !h->gsp && !h->cfg.staged) {
+    if (nib_ok && !h->gsp && !h->cfg.staged && !h->cfg.bits) {
         SweepCfg c = choose_cfg(0, n, 4 * ((own + 7) / 8), h->H, avg_level, (double)h->nnz / std::max(n, 1), sms,
                                 h->ell_w);
         c.lanes_per_vertex = 1;
@@ -861,7 +910,7 @@ static pamc_status init_run(pamc_handle h, const pamc_params *pp, int32_t rank, 
             h->nib = true;
         }
     }
-    if (!h->gsp && sweep_smem_bytes(sweep_kind(p), n, h->H, h->cfg) > kSmemMax) {
+    if (!h->gsp && !h->cfg.bits && sweep_smem_bytes(sweep_kind(p), n, h->H, h->cfg) > kSmemMax) {
         release_run(h);
         return fail(h, PAMC_ERR_RANGE, "n = %d: one replica group's labels exceed shared memory", n);
     }
@@ -1520,6 +1569,7 @@ pamc_status pamc_sweep_mode(pamc_handle h, int *mode) {
         return fail(h, PAMC_ERR_STATE, "no sparse Ising run initialised");
     const bool ell = h->d_ell != nullptr;
     if (h->gsp) *mode = (ell ? 1 : 0) | 4;
+    else if (h->cfg.bits) *mode = 1 | 32;
     else if (h->nib) *mode = 1 | 16;
     else *mode = sweep_push_ok(h->H, h->p.sweeps, ell, h->cfg.lanes_per_vertex) ? 2 : ell ? 1 : 0;
     if (h->H > kByteLaneMaxH) *mode |= 8;
@@ -1565,6 +1615,8 @@ struct pamc_batch_s {
     int64_t launches = 0;
     int64_t rebuilds = 0;
     SweepCfg shape[3];            // batched sweep launch shape per size class
+    bool shaped[3] = {false, false, false};   // the caller chose it
+    cudaStream_t side[4] = {nullptr, nullptr, nullptr, nullptr};   // branches of the captured step
     bool global[3] = {false, false, false};   // Ising members' spin words in device memory
     char err[256] = "";
 };
@@ -1655,8 +1707,29 @@ pamc_status rebuild(pamc_batch b) {
         return h->p.kind == 0 && !member_global(h) &&
                sweep_nibble_ok(h->nib_halves, h->p.sweeps, 1, false) && !sweep_push_enabled();
     };
+    // members on one bit a replica: quads a group so that the batch has about
+    // two groups an SM (the largest members' groups bound the step)
+    int sms = 152;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->device);
+    auto bits_can = [&](pamc_handle h) {
+        return h->p.kind == 0 && h->p.sweeps > 0 && h->bits_ok && !member_global(h) && !b->shaped[batch_class(h->n)] &&
+               sweep_nibble_enabled() && !sweep_push_enabled() && sweep_bits_smem_bytes(h->n, h->H) <= kSmemMax;
+    };
+    int64_t bits_R = 0;
     for (pamc_handle h : b->members)
-        if (h->host_t < h->p.steps) {
+        if (h->host_t < h->p.steps && bits_can(h)) bits_R += h->p.R;
+    const int bits_nc = (int)std::min<int64_t>(8, (bits_R + 4 * sms) / (8 * sms));
+    auto member_bits = [&](pamc_handle h) { return bits_can(h) && bits_pay(bits_nc, h->avg_level, member_nib(h)); };
+    struct BitsLaunch {
+        std::vector<int2> items;
+        size_t smem = 0;
+    };
+    std::map<std::array<int, 4>, BitsLaunch> bits;   // by rule, planes, lanes a vertex, warps
+    // the largest members first: their groups bound the step
+    std::vector<pamc_handle> members = b->members;
+    std::stable_sort(members.begin(), members.end(), [](pamc_handle x, pamc_handle y) { return x->n > y->n; });
+    for (pamc_handle h : members)
+        if (h->host_t < h->p.steps && !member_bits(h)) {
             int32_t &m = (h->p.kind != 0 ? pnmax : member_global(h) ? gnmax : member_nib(h) ? nnmax
                                                                                             : nmax)[batch_class(h->n)];
             m = std::max(m, h->n);
@@ -1676,7 +1749,7 @@ pamc_status rebuild(pamc_batch b) {
         while (peff[c].groups_per_cta > 1 && sweep_potts_smem_bytes(pnmax[c], 127, peff[c]) > kSmemMax)
             peff[c].groups_per_cta -= 1;
     }
-    for (pamc_handle h : b->members) {
+    for (pamc_handle h : members) {
         const pamc_params &p = h->p;
         if (h->host_t >= p.steps) continue;
         const uint32_t k0 = (uint32_t)p.seed, k1 = (uint32_t)(p.seed >> 32);
@@ -1727,15 +1800,22 @@ pamc_status rebuild(pamc_batch b) {
             return bfail(b, PAMC_ERR_OOM, "device allocation of a member's group spin words failed");
         d.gsp = gl ? h->d_gsp : nullptr;
         const bool nb = member_nib(h);
-        const SweepCfg cfg = p.kind != 0 ? peff[cls] : gl ? geff[cls] : nb ? neff[cls] : eff[cls];
-        d.push = p.kind == 0 && !gl && !nb && sweep_push_ok(h->H, p.sweeps, h->d_ell != nullptr, cfg.lanes_per_vertex)
+        const bool bt = member_bits(h);
+        const SweepCfg cfg = bt ? bits_shape(h->avg_level, bits_nc, false) : p.kind != 0 ? peff[cls] : gl ? geff[cls] : nb ? neff[cls] : eff[cls];
+        d.push = p.kind == 0 && !gl && !nb && !bt && sweep_push_ok(h->H, p.sweeps, h->d_ell != nullptr, cfg.lanes_per_vertex)
                      ? 1 : 0;
         const int idx = (int)sw.size();
         sw.push_back(d);
-        const int32_t groups = nb ? (p.R + 7) / 8 : (p.R + 3) / 4;
+        const int32_t groups = bt ? (p.R + 4 * bits_nc - 1) / (4 * bits_nc) : nb ? (p.R + 7) / 8 : (p.R + 3) / 4;
         const int32_t ctas = (groups + cfg.groups_per_cta - 1) / cfg.groups_per_cta;
         // with sweeps = 0 the launch still copies the resampled population and its energies
-        auto &items = p.kind != 0 ? pswi[h->d_ell != nullptr][cls]
+        BitsLaunch *bl = nullptr;
+        if (bt) {
+            bl = &bits[{p.rule, sweep_bits_planes(h->H), cfg.lanes_per_vertex, cfg.warps_per_group}];
+            bl->smem = std::max(bl->smem, sweep_bits_smem_bytes(h->n, h->H));
+        }
+        auto &items = bt ? bl->items
+                      : p.kind != 0 ? pswi[h->d_ell != nullptr][cls]
                                   : nb ? nswi[h->nib_halves == 2][p.rule][cls]
                                        : (gl ? gswi : swi)[h->d_ell != nullptr][p.rule][cls];
         for (int32_t x = 0; x < ctas; ++x) items.push_back(make_int2(idx, x));
@@ -1757,6 +1837,7 @@ pamc_status rebuild(pamc_batch b) {
     for (auto &a : nswi)
         for (auto &c : a)
             for (auto &v : c) all_items.insert(all_items.end(), v.begin(), v.end());
+    for (auto &[key, v] : bits) all_items.insert(all_items.end(), v.items.begin(), v.items.end());
     const size_t n_rdsi = rdsi.size();
     rdsi.insert(rdsi.end(), rdei.begin(), rdei.end());   // one upload: spin items, then energy items
     const bool ok = upload(b, b->sd, sd) && upload(b, b->sdi, sdi) && upload(b, b->prep, prep) &&
@@ -1779,47 +1860,68 @@ pamc_status rebuild(pamc_batch b) {
                                b->stream);
         nl += 1;
     }
+    // The sweeps of the different layouts and the next schedule are branches of
+    // the step: none fills the device alone, and none reads what another writes.
+    for (cudaStream_t &x : b->side)
+        if (e == cudaSuccess && !x) e = cudaStreamCreateWithFlags(&x, cudaStreamNonBlocking);
+    std::vector<cudaEvent_t> events;
+    auto mark = [&](cudaStream_t from, cudaStream_t to) {   // to waits for what from holds so far
+        cudaEvent_t ev = nullptr;
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
+        if (ev) events.push_back(ev);
+        if (e == cudaSuccess) e = cudaEventRecord(ev, from);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(to, ev, 0);
+    };
+    constexpr int kSides = 4;
+    int branch = 0;
+    bool forked[kSides] = {false, false, false, false};
+    auto next_branch = [&]() {   // the batch's own stream, then the side streams in turn
+        const int x = branch++ % (kSides + 1);
+        if (x == 0) return b->stream;
+        return b->side[x - 1];
+    };
+    for (int x = 0; x < kSides && e == cudaSuccess; ++x) mark(b->stream, b->side[x]), forked[x] = e == cudaSuccess;
     size_t off = 0;
-    for (int el = 0; el < 2 && e == cudaSuccess; ++el)
-        for (int ru = 0; ru < 2 && e == cudaSuccess; ++ru)
-            for (int c = 0; c < kClasses && e == cudaSuccess; ++c) {
-                const auto &items = swi[el][ru][c];
-                if (items.empty()) continue;
-                e = launch_sweep_ising_batched(ru, el != 0, (const SweepDesc *)b->sw.p, (const int2 *)b->swi.p + off,
-                                               (int32_t)items.size(), nmax[c], eff[c], b->stream);
-                off += items.size();
-                nl += 1;
-            }
-    for (int el = 0; el < 2 && e == cudaSuccess; ++el)
-        for (int ru = 0; ru < 2 && e == cudaSuccess; ++ru)
-            for (int c = 0; c < kClasses && e == cudaSuccess; ++c) {
-                const auto &items = gswi[el][ru][c];
-                if (items.empty()) continue;
-                e = launch_sweep_ising_batched(ru, el != 0, (const SweepDesc *)b->sw.p, (const int2 *)b->swi.p + off,
-                                               (int32_t)items.size(), gnmax[c], geff[c], b->stream, true);
-                off += items.size();
-                nl += 1;
-            }
-    for (int el = 0; el < 2 && e == cudaSuccess; ++el)
-        for (int c = 0; c < kClasses && e == cudaSuccess; ++c) {
-            const auto &items = pswi[el][c];
-            if (items.empty()) continue;
-            e = launch_sweep_potts_batched(el != 0, (const SweepDesc *)b->sw.p, (const int2 *)b->swi.p + off,
-                                           (int32_t)items.size(), pnmax[c], peff[c], b->stream);
-            off += items.size();
-            nl += 1;
-        }
-    for (int bi = 0; bi < 2 && e == cudaSuccess; ++bi)
-        for (int ru = 0; ru < 2 && e == cudaSuccess; ++ru)
-            for (int c = 0; c < kClasses && e == cudaSuccess; ++c) {
-                const auto &items = nswi[bi][ru][c];
-                if (items.empty()) continue;
-                e = launch_sweep_ising_nib_batched(ru, bi != 0, (const SweepDesc *)b->sw.p,
-                                                   (const int2 *)b->swi.p + off, (int32_t)items.size(), nnmax[c],
-                                                   neff[c], b->stream);
-                off += items.size();
-                nl += 1;
-            }
+    auto sweep = [&](size_t count, auto &&launch) {   // one branch: the items off .. off + count - 1
+        if (count == 0 || e != cudaSuccess) return;
+        e = launch((const int2 *)b->swi.p + off, (int32_t)count, next_branch());
+        off += count;
+        nl += 1;
+    };
+    const SweepDesc *descs = (const SweepDesc *)b->sw.p;
+    for (int gl = 0; gl < 2; ++gl)
+        for (int el = 0; el < 2; ++el)
+            for (int ru = 0; ru < 2; ++ru)
+                for (int c = 0; c < kClasses; ++c)
+                    sweep((gl ? gswi : swi)[el][ru][c].size(), [&](const int2 *it, int32_t m, cudaStream_t st) {
+                        return launch_sweep_ising_batched(ru, el != 0, descs, it, m, gl ? gnmax[c] : nmax[c],
+                                                          gl ? geff[c] : eff[c], st, gl != 0);
+                    });
+    for (int el = 0; el < 2; ++el)
+        for (int c = 0; c < kClasses; ++c)
+            sweep(pswi[el][c].size(), [&](const int2 *it, int32_t m, cudaStream_t st) {
+                return launch_sweep_potts_batched(el != 0, descs, it, m, pnmax[c], peff[c], st);
+            });
+    for (int bi = 0; bi < 2; ++bi)
+        for (int ru = 0; ru < 2; ++ru)
+            for (int c = 0; c < kClasses; ++c)
+                sweep(nswi[bi][ru][c].size(), [&](const int2 *it, int32_t m, cudaStream_t st) {
+                    return launch_sweep_ising_nib_batched(ru, bi != 0, descs, it, m, nnmax[c], neff[c], st);
+                });
+    for (auto &[key, v] : bits)
+        sweep(v.items.size(), [&, &key = key, &v = v](const int2 *it, int32_t m, cudaStream_t st) {
+            return launch_sweep_ising_bits_batched(key[0], key[1], key[2], key[3], bits_nc, v.smem, descs, it, m, st);
+        });
+    if (e == cudaSuccess && !sdi.empty()) {
+        int32_t sched_nmax = 1;
+        for (const SchedDesc &d : sd) sched_nmax = std::max(sched_nmax, d.n);
+        launch_schedule_batched((const SchedDesc *)b->sd.p, (const int2 *)b->sdi.p, (int32_t)sdi.size(), sched_nmax,
+                                next_branch());
+        e = cudaGetLastError();
+        nl += 1;
+    }
+    for (int x = 0; x < kSides; ++x)
+        if (forked[x]) mark(b->side[x], b->stream);
     if (e == cudaSuccess) e = launch_control_batched((const CtlDesc *)b->ctl.p, (int32_t)ctls.size(), b->stream);
     nl += 1;
     if (e == cudaSuccess && !rds.empty()) {
@@ -1827,16 +1929,9 @@ pamc_status rebuild(pamc_batch b) {
                                   (int32_t)n_rdsi, (const int2 *)b->rdi.p + n_rdsi, (int32_t)rdei.size(), b->stream);
         nl += 3;
     }
-    if (e == cudaSuccess && !sdi.empty()) {
-        int32_t sched_nmax = 1;
-        for (const SchedDesc &d : sd) sched_nmax = std::max(sched_nmax, d.n);
-        launch_schedule_batched((const SchedDesc *)b->sd.p, (const int2 *)b->sdi.p, (int32_t)sdi.size(), sched_nmax,
-                                b->stream);
-        e = cudaGetLastError();
-        nl += 1;
-    }
     cudaGraph_t g = nullptr;
     const cudaError_t e2 = cudaStreamEndCapture(b->stream, &g);
+    for (cudaEvent_t ev : events) cudaEventDestroy(ev);
     if (e == cudaSuccess) e = e2;
     if (e != cudaSuccess) {
         if (g) cudaGraphDestroy(g);
@@ -1881,7 +1976,10 @@ pamc_status pamc_batch_create(int cuda_device, void *stream, pamc_batch *out) {
     if (!b) return bfail(nullptr, PAMC_ERR_OOM, "host allocation failed");
     b->device = cuda_device;
     b->stream = (cudaStream_t)stream;
-    for (int c = 0; c < kClasses; ++c) b->shape[c] = batch_cfg(c);
+    for (int c = 0; c < kClasses; ++c) {
+        b->shape[c] = batch_cfg(c);
+        b->shaped[c] = getenv("PAMC_BATCH_CFG") != nullptr;
+    }
     if (!b->stream) {   // graph capture needs a stream other than the legacy default one
         if (cudaStreamCreateWithFlags(&b->stream, cudaStreamNonBlocking) != cudaSuccess) {
             delete b;
@@ -1908,11 +2006,12 @@ pamc_status pamc_batch_add(pamc_batch b, pamc_handle h) {
     for (pamc_handle m : b->members)
         if (m == h) return bfail(b, PAMC_ERR_ARG, "handle already in the batch");
     if (cudaSetDevice(b->device) != cudaSuccess) return bfail(b, PAMC_ERR_CUDA, "cudaSetDevice failed");
-    // Inside the batch the schedule ring is refilled one step at a time: after
-    // step t it holds steps t+1 .. t+16.  Fill the slots of the steps up to
-    // host_t + 15 that the member's own stepping has not built yet.
+    // Inside the batch the schedule ring is refilled one step at a time: step t
+    // builds step t+15 beside its sweeps (the slot of step t-1), so that after
+    // it the ring holds steps t+1 .. t+15.  Fill the slots of the steps up to
+    // host_t + 14 that the member's own stepping has not built yet.
     const pamc_params &p = h->p;
-    const int64_t want = std::min<int64_t>(h->host_t + kSchedSlots, p.steps);
+    const int64_t want = std::min<int64_t>(h->host_t + kSchedSlots - 1, p.steps);
     if (p.sweeps > 0 && h->sched_end < want) {
         launch_schedule(h->n, h->d_rp, h->d_adj, p.seed, (int32_t)h->sched_end, (int32_t)(want - h->sched_end),
                         p.sweeps, 0, kSchedSlots, h->d_order, h->d_lvl, h->d_nlev, h->d_skey, h->d_scnt,
@@ -1948,7 +2047,7 @@ pamc_status pamc_batch_step(pamc_batch b, int32_t nsteps) {
         for (pamc_handle h : b->members) {
             if (h->host_t >= h->p.steps) continue;
             h->host_t += 1;
-            h->sched_end = std::min<int64_t>(h->host_t + kSchedSlots, h->p.steps);
+            h->sched_end = std::min<int64_t>(h->host_t + kSchedSlots - 1, h->p.steps);
             h->launches += b->graph_launches;
             finished |= h->host_t >= h->p.steps;
         }
@@ -1987,6 +2086,7 @@ pamc_status pamc_batch_set_shape(pamc_batch b, int size_class, int groups_per_ct
         return bfail(b, PAMC_ERR_ARG, "need groups >= 1, warps >= 1 and groups * warps <= 32");
     b->shape[size_class].groups_per_cta = groups_per_cta;
     b->shape[size_class].warps_per_group = warps_per_group;
+    b->shaped[size_class] = true;
     b->dirty = true;
     return PAMC_OK;
 }
@@ -1996,6 +2096,7 @@ pamc_status pamc_batch_set_lanes(pamc_batch b, int size_class, int lanes_per_ver
     if (size_class < 0 || size_class >= kClasses) return bfail(b, PAMC_ERR_ARG, "size class must be 0, 1 or 2");
     if (!batch_lanes_ok(lanes_per_vertex)) return bfail(b, PAMC_ERR_ARG, "lanes per vertex must be 1, 2 or 4");
     b->shape[size_class].lanes_per_vertex = lanes_per_vertex;
+    b->shaped[size_class] = true;
     b->dirty = true;
     return PAMC_OK;
 }
@@ -2064,6 +2165,8 @@ void pamc_batch_destroy(pamc_batch b) {
     for (DevBuf *d : {&b->sw, &b->swi, &b->sd, &b->sdi, &b->prep, &b->tabs, &b->ctl, &b->ncm, &b->ncmi, &b->rd,
                       &b->rdi})
         if (d->p) cudaFree(d->p);
+    for (cudaStream_t x : b->side)
+        if (x) cudaStreamDestroy(x);
     if (b->own_stream) cudaStreamDestroy(b->stream);
     delete b;
 }

@@ -192,6 +192,7 @@ struct SweepCfg {
     int warps_per_group;  // warps cooperating on one group's level
     int lanes_per_vertex = 1;  // Ising, ELL: lanes sharing one vertex's couplings (1, 2, 4, .., 32)
     int staged = 0;            // Ising, ELL: the staged sweep (one group per CTA)
+    int bits = 0;              // Ising, ELL: one bit a replica, groups of 4 bits replicas (1..8; 0: not)
 };
 
 // Builds the (t, sweep) schedules of nt steps starting at t0 into ring slots
@@ -269,6 +270,23 @@ cudaError_t launch_sweep_ising_nib(int rule, int32_t n, int32_t H, const pamc_pa
 // eight).
 cudaError_t launch_sweep_ising_nib_batched(int rule, bool two, const SweepDesc *descs, const int2 *items,
                                            int32_t nitems, int32_t n_max, SweepCfg cfg, cudaStream_t st);
+
+// Ising sweeps with one bit a replica, up to 32 replicas a word
+// (sweep_bits.cu): couplings +-1, at most kBitLaneMaxH neighbours, ELL rows,
+// S >= 1, words in shared memory; cfg.bits replica quads a group, 1, 2 or 4
+// lanes a vertex.
+constexpr int32_t kBitLaneMaxH = 63;
+bool bits_apply(int32_t n, const int32_t *rp, const uint32_t *adj, int32_t H, int32_t ell_w);
+size_t sweep_bits_smem_bytes(int32_t n, int32_t H);
+cudaError_t launch_sweep_ising_bits(int rule, int32_t n, int32_t H, const pamc_params &p, int32_t t, int32_t slot,
+                                    SchedView sv, const uint64_t *tab, const int8_t *src, const int32_t *parent,
+                                    const int8_t *ncm_buf, const int32_t *ncm_idx, int8_t *dst, int64_t *E_dst,
+                                    const DevCtl *ctl, SweepCfg cfg, cudaStream_t st, int32_t rbase);
+
+int sweep_bits_planes(int32_t H);   // bit planes of the sum (3, 5 or 6)
+// Batched (a launch: members of one rule, plane count, lanes a vertex and block size).
+cudaError_t launch_sweep_ising_bits_batched(int rule, int planes, int lanes, int warps, int nc, size_t smem,
+                                            const SweepDesc *descs, const int2 *items, int32_t nitems, cudaStream_t st);
 
 // Ising sweeps of small populations (sweep_staged.cu): one CTA per group of
 // four, ELL rows and draws staged in shared memory by producer warps; byte or

@@ -91,6 +91,9 @@ cudaError_t launch_sweep(int kind, int rule, int32_t n, const int32_t *rp, const
     if (kind == 0 && cfg.staged)
         return launch_sweep_ising_staged(rule, n, H, p, t, slot, sv, tab, src, parent, ncm_buf, ncm_idx, dst, E_dst, ctl,
                                          cfg, st, rbase);
+    if (kind == 0 && cfg.bits)
+        return launch_sweep_ising_bits(rule, n, H, p, t, slot, sv, tab, src, parent, ncm_buf, ncm_idx, dst, E_dst, ctl,
+                                       cfg, st, rbase);
     if (kind == 0 && nib)
         return launch_sweep_ising_nib(rule, n, H, p, t, slot, sv, tab, src, parent, ncm_buf, ncm_idx, dst, E_dst,
                                       ctl, cfg, st, rbase);

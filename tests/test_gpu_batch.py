@@ -389,6 +389,36 @@ def test_served_stream_requests_match_oracle(pg):
         np.testing.assert_array_equal(got[req.rid].spins, spins, err_msg=f"request {req.rid}")
 
 
+def test_batch_bit_lane_members(pg):
+    """A batch of enough replicas keeps its +-1 members on one bit a replica
+    (sums of three, five and six planes, both rules, wide and narrow levels,
+    restarts); beside them the other layouts and the schedules run as branches
+    of the step: every member equals its run alone."""
+    cases = [(W.torus(60, 60, signed=True, seed=1), dict(R=500, sweeps=2, steps=20, seed=1)),
+             (W.er_avg_degree(400, 20, signed=True, seed=2), dict(R=501, sweeps=2, steps=20, seed=2, rule=1)),
+             (W.er_avg_degree(900, 42, signed=False, seed=3), dict(R=403, sweeps=1, steps=19, seed=3)),
+             (W.gnm(5000, 14000, signed=True, seed=4), dict(R=700, sweeps=2, steps=18, seed=4, stagnation=1, z_rst=5,
+                                                           cooldown_tau=1, win_short=2, win_long=3)),
+             (W.gnm(300, 900, signed=True, seed=5), dict(R=64, sweeps=2, steps=20, seed=5, kind=1))]
+    ref = [alone(pg, inst, p) for inst, p in cases]
+    b = pg.pamc_batch_create(0)
+    hs = []
+    try:
+        for inst, p in cases:
+            h = pg.pamc_create_csr(inst.n, inst.row_ptr, inst.col, inst.w)
+            pg.pamc_init(h, **p)
+            pg.pamc_batch_add(b, h)
+            hs.append(h)
+        pg.pamc_batch_step(b, 20)
+        pg.pamc_batch_sync(b)
+        for i, (inst, p) in enumerate(cases):
+            assert_same(snapshot(pg, hs[i], inst.n, p["R"]), ref[i], f"member {i}")
+    finally:
+        pg.pamc_batch_destroy(b)
+        for h in hs:
+            pg.pamc_destroy(h)
+
+
 def test_shapes_change_speed_not_results(pg):
     """Every launch shape of every size class gives the same members' results,
     and the autotuner sets one of the candidates."""

@@ -216,6 +216,47 @@ def test_staged_sweep(pg, monkeypatch, cfg):
         compare_run(pg, inst, 3, **p)
 
 
+@pytest.mark.parametrize("cfg", ["1,1,1,0,8", "1,2,2,0,3", "1,4,4,0,7", "1,3,4,0,1", "1,32,1,0,5"])
+def test_bit_lanes(pg, monkeypatch, cfg):
+    """One bit a replica: words of 1 to 8 quads, one to four lanes a vertex,
+    sums of three, five and six planes up to their largest values, rows whose
+    last group is ragged, a last word of one replica, both rules, cluster moves
+    and restarts, against the oracle; weights beyond +-1 and rows beyond 63 keep
+    the other lanes; by default where the population gives an SM's word two
+    quads or more."""
+    k64 = W.csr_from_edges(64, *np.triu_indices(64, 1), np.resize([1, -1, 1, 1, 1], 64 * 63 // 2), "k64")
+    two = W.csr_from_edges(8, np.array([0, 1]), np.array([1, 2]), np.array([1, 2]), "two")
+    k65 = W.csr_from_edges(65, *np.triu_indices(65, 1), np.ones(65 * 32), "k65")
+    cases = [(W.torus(18, 18, seed=3), 37, 0), (_max_degree_graph(300, 900, 7, 6), 33, 1), (W.gnm(500, 700, seed=4), 29, 1),
+             (_max_degree_graph(300, 2600, 31, 7), 65, 0), (W.erdos_renyi(97, 0.4, signed=True, seed=4), 13, 1), (k64, 9, 0)]
+    monkeypatch.setenv("PAMC_SWEEP_CFG", cfg)
+    for inst, R, rule in cases:
+        p = dict(R=R, sweeps=3, beta0=0.2, beta1=3.0, rule=rule, stagnation=1, z_rst=4, cooldown_tau=1, win_short=2,
+                 win_long=3, seed=4)
+        s = pg.Solver(inst.row_ptr, inst.col, inst.w)
+        s.init(steps=3, **p)
+        assert pg.pamc_sweep_mode(s.h) == 33, inst.name
+        s.step(3)
+        ref = oracle.OracleRun(inst.row_ptr, inst.col, inst.w, steps=3, **p)
+        ref.step(3)
+        assert pg.pamc_sweep_stats(s.h)["flips"] == ref.sweep_flips(), inst.name
+        s.close()
+        compare_run(pg, inst, 6, **p)
+    for inst in (two, k65):
+        s = pg.Solver(inst.row_ptr, inst.col, inst.w)
+        s.init(R=16, sweeps=1, steps=2, seed=1)
+        assert not pg.pamc_sweep_mode(s.h) & 32, inst.name
+        s.close()
+    monkeypatch.delenv("PAMC_SWEEP_CFG")
+    inst = W.erdos_renyi(97, 0.4, signed=True, seed=4)
+    s = pg.Solver(inst.row_ptr, inst.col, inst.w)
+    for R, mode in ((608, 1), (1300, 33)):
+        s.init(R=R, sweeps=1, steps=2, seed=1)
+        assert pg.pamc_sweep_mode(s.h) == mode, R
+    s.close()
+    compare_run(pg, inst, 2, R=1300, sweeps=2, beta0=0.2, beta1=2.0, seed=3)
+
+
 def test_independent_chains_baseline(pg):
     inst = W.gnm(400, 1100, signed=True, seed=6)
     compare_run(pg, inst, 6, R=9, sweeps=2, resample=0, seed=1)
