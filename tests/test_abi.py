@@ -74,6 +74,38 @@ def test_host_validation_errors(lib):
     assert b"column" in buf.value
 
 
+@pytest.mark.parametrize("order", ["sorted", "shuffled"])
+def test_symmetry_check_is_the_multiset_comparison(lib, order):
+    """Parallel entries, zero weights and rows in any order: a matrix is refused
+    as asymmetric exactly where the multisets of (i, j, w) and (j, i, w) differ."""
+    seen = set()
+    for seed in range(400):
+        r = np.random.default_rng([7, seed])
+        n, m = int(r.integers(2, 7)), int(r.integers(1, 9))
+        i = r.integers(0, n, m)
+        j = (i + r.integers(1, n, m)) % n
+        w = r.integers(-2, 3, m)
+        src, dst, ww = np.concatenate([i, j]), np.concatenate([j, i]), np.concatenate([w, w])
+        x = int(r.integers(0, 2 * m))
+        if seed % 3 == 1:
+            ww[x] += 1
+        elif seed % 3 == 2:
+            dst[x] = (src[x] + r.integers(1, n)) % n
+        o = np.lexsort((ww, dst, src))
+        if order == "shuffled":
+            o = r.permutation(2 * m)
+            o = o[np.argsort(src[o], kind="stable")]
+        src, dst, ww = src[o], dst[o], ww[o]
+        rp = np.concatenate([[0], np.cumsum(np.bincount(src, minlength=n))])
+        rc, h = _create(lib, rp, dst, ww)
+        same = sorted(zip(src, dst, ww)) == sorted(zip(dst, src, ww))
+        assert (rc != 2) == same, seed
+        seen.add(same)
+        if rc == 0:
+            lib.pamc_destroy(h)
+    assert seen == {True, False}
+
+
 def test_null_arguments(lib):
     assert lib.pamc_create_csr(4, None, None, None, 0, None, None) == 1
     assert lib.pamc_init(None, None) == 1
