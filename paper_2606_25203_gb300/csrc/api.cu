@@ -377,6 +377,20 @@ SweepCfg choose_cfg(int kind, int32_t n, int32_t R, int32_t H, double avg_level,
         const int64_t per_sm = (groups + sms - 1) / std::max(sms, 1);
         int lanes = 1024;
         while (lanes > 32 && (int64_t)lanes * per_sm > 1024) lanes >>= 1;
+        if (kind == 2 && ell_w > 0) {
+            // the softmax sampler on ELL rows, always quads: a group alone on its
+            // SM takes twice the lanes of an average level's pass (the level's
+            // chain is what counts), groups that share an SM half of them, at most
+            // their share of 1,024 lanes.  us per launch of 10 sweeps, 4 / 8 / 16
+            // warps: N=2,000 degree 12 (levels of 65) R=256 585 / 453 / 400,
+            // R=2,048 710 / 809 / 1,064; N=12,000 degree 5, R=2,048 2,740 / 2,557 /
+            // 2,548
+            SweepCfg q{1, 4, 4};
+            const double want = avg_level / (per_sm <= 1 ? 4.0 : 16.0);
+            const int most = per_sm <= 1 ? 32 : std::max(4, lanes / 32);
+            while (2 * q.warps_per_group <= most && 2 * q.warps_per_group <= want) q.warps_per_group *= 2;
+            if (sweep_smem_bytes(kind, n, H, q) <= 227 * 1024) return q;
+        }
         SweepCfg c{1, 1, 1};
         while (c.warps_per_group < 32 && 32.0 * c.warps_per_group < std::max(avg_level, 1.0)) c.warps_per_group *= 2;
         if (32 * c.warps_per_group <= lanes && sweep_smem_bytes(kind, n, H, c) <= 227 * 1024) {

@@ -174,6 +174,27 @@ def test_potts_launch_shapes_same_results(pg, monkeypatch, rule):
         compare_run(pg, inst, 4, **params)
 
 
+@pytest.mark.parametrize("K", [2, 3, 4, 5, 8])
+def test_softmax_quads_over_label_counts(pg, monkeypatch, K):
+    """The softmax sampler's quads for each way labels are told apart: rows of
+    one to seven groups of four, levels that leave quads idle, a ragged
+    population, signed and larger weights, several shapes, against the oracle."""
+    inst = W.gnm(333, 1900, signed=True, seed=8)
+    heavy = W.gnm(100, 260, signed=True, seed=9)
+    e = np.repeat(np.arange(heavy.n), np.diff(heavy.row_ptr))
+    heavy.w = (heavy.w * (1 + (np.minimum(e, heavy.col) + np.maximum(e, heavy.col)) % 7)).astype(np.int32)
+    for cfg in (None, "1,1,4", "3,2,4"):
+        if cfg:
+            monkeypatch.setenv("PAMC_SWEEP_CFG", cfg)
+        for g, R in ((inst, 11), (heavy, 6), (W.torus(9, 9, signed=True, seed=3), 5)):
+            p = dict(kind=1, rule=2, K=K, gamma=0.8, R=R, sweeps=2, beta0=0.2, beta1=2.5, seed=6)
+            s = pg.Solver(g.row_ptr, g.col, g.w)
+            s.init(steps=3, **p)
+            assert pg.pamc_sweep_shape(s.h)[2] == 4
+            s.close()
+            compare_run(pg, g, 3, **p)
+
+
 def test_lanes_per_vertex_default_choice(pg, monkeypatch):
     """Narrow-level dense-row instances get several lanes per vertex; the
     torus (rows of four) keeps one."""
