@@ -377,16 +377,20 @@ SweepCfg choose_cfg(int kind, int32_t n, int32_t R, int32_t H, double avg_level,
         const int64_t per_sm = (groups + sms - 1) / std::max(sms, 1);
         int lanes = 1024;
         while (lanes > 32 && (int64_t)lanes * per_sm > 1024) lanes >>= 1;
-        if (kind == 2 && ell_w > 0) {
-            // the softmax sampler on ELL rows, always quads: a group alone on its
-            // SM takes twice the lanes of an average level's pass (the level's
-            // chain is what counts), groups that share an SM half of them, at most
-            // their share of 1,024 lanes.  us per launch of 10 sweeps, 4 / 8 / 16
-            // warps: N=2,000 degree 12 (levels of 65) R=256 585 / 453 / 400,
-            // R=2,048 710 / 809 / 1,064; N=12,000 degree 5, R=2,048 2,740 / 2,557 /
-            // 2,548
-            SweepCfg q{1, 4, 4};
-            const double want = avg_level / (per_sm <= 1 ? 4.0 : 16.0);
+        if (ell_w > 0) {
+            // ELL rows, several lanes a position -- the cascaded sampler: pairs,
+            // the softmax sampler: quads.  A group alone on its SM takes twice
+            // the lanes of an average level's pass and more (the level's chain is
+            // what counts), groups that share an SM about half, at most their
+            // share of 1,024 lanes; the cascaded sampler takes one lane a
+            // position where a level fills that share.  us per launch of 10
+            // sweeps, 4 / 8 / 16 warps of pairs (8 warps of single lanes): N=2,000
+            // degree 12 (levels of 65) R=256 368 / 296 / 333 (414), R=2,048 473 / 518
+            // / 922 (586); N=12,000 degree 5 R=2,048 2,183 / 1,481 / 1,413 (1,379); of
+            // quads: N=2,000 R=256 585 / 453 / 400, R=2,048 710 / 809 / 1,064;
+            // N=12,000 2,740 / 2,557 / 2,548
+            SweepCfg q{1, 4, kind == 2 ? 4 : avg_level >= lanes ? 1 : 2};
+            const double want = avg_level * (kind == 2 ? 2.0 : 1.0) / (per_sm <= 1 ? 8.0 : kind == 2 ? 32.0 : 16.0);
             const int most = per_sm <= 1 ? 32 : std::max(4, lanes / 32);
             while (2 * q.warps_per_group <= most && 2 * q.warps_per_group <= want) q.warps_per_group *= 2;
             if (sweep_smem_bytes(kind, n, H, q) <= 227 * 1024) return q;
@@ -394,15 +398,11 @@ SweepCfg choose_cfg(int kind, int32_t n, int32_t R, int32_t H, double avg_level,
         SweepCfg c{1, 1, 1};
         while (c.warps_per_group < 32 && 32.0 * c.warps_per_group < std::max(avg_level, 1.0)) c.warps_per_group *= 2;
         if (32 * c.warps_per_group <= lanes && sweep_smem_bytes(kind, n, H, c) <= 227 * 1024) {
-            // several lanes a position -- the cascaded sampler on ELL rows:
-            // pairs; the softmax sampler: quads -- with twice the warps where
-            // that still fits the group's share of the SM, two groups to a
-            // CTA where the SMs hold two or more (configuration 3: cascaded
-            // 0.720 against 0.773 ms per step, softmax 1.65 against 2.08, for
-            // one group of four warps a CTA, one lane a position)
-            if (((kind == 1 && ell_w > 0) || kind == 2) && c.warps_per_group <= 16 &&
-                64 * c.warps_per_group <= lanes) {
-                SweepCfg p2{1, 2 * c.warps_per_group, kind == 2 ? 4 : 2};
+            // CSR rows, the softmax sampler: quads, with twice the warps where
+            // that still fits the group's share of the SM, two groups to a CTA
+            // where the SMs hold two or more
+            if (kind == 2 && c.warps_per_group <= 16 && 64 * c.warps_per_group <= lanes) {
+                SweepCfg p2{1, 2 * c.warps_per_group, 4};
                 if (groups >= 2 * (int64_t)sms && 2 * 32 * p2.warps_per_group <= 1024) p2.groups_per_cta = 2;
                 if (sweep_smem_bytes(kind, n, H, p2) <= 227 * 1024) return p2;
             }
@@ -1684,12 +1684,15 @@ bool upload(pamc_batch b, DevBuf &buf, const std::vector<T> &v) {
 }
 
 // Sweep launch shape per size class of n (groups of 4 replicas per CTA,
-// warps per group).  Small instances pack several groups into one CTA.
+// warps per group): few groups a CTA, so that a few members spread over the
+// SMs (bursts of ten requests of 800 to 20,000 vertices, R=512: 100 and 202 ms; with
+// eight, four and one group a CTA on 1, 2 and 16 warps 110 and 204, with one
+// group on 4, 8 and 32 warps 121 and 202).
 constexpr int kClasses = 3;
 int batch_class(int32_t n) { return n <= 2048 ? 0 : n <= 8192 ? 1 : 2; }
 bool batch_lanes_ok(int l) { return l == 1 || l == 2 || l == 4; }
 SweepCfg batch_cfg(int cls) {
-    static const SweepCfg c[kClasses] = {{8, 1, 1}, {4, 2, 1}, {1, 16, 1}};
+    static const SweepCfg c[kClasses] = {{2, 4, 1}, {2, 4, 1}, {1, 32, 1}};
     const char *env = getenv("PAMC_BATCH_CFG");   // "g0,w0;g1,w1;g2,w2"
     if (env) {
         int v[6];
@@ -1844,7 +1847,7 @@ pamc_status rebuild(pamc_batch b) {
             bl->smem = std::max(bl->smem, sweep_bits_smem_bytes(h->n, h->H));
         }
         auto &items = bt ? bl->items
-                      : p.kind != 0 ? pswi[h->d_ell != nullptr][cls]
+                      : p.kind != 0 ? pswi[h->d_ell != nullptr && p.sweeps > 0][cls]
                                   : nb ? nswi[h->nib_halves == 2][p.rule][cls]
                                        : (gl ? gswi : swi)[h->d_ell != nullptr][p.rule][cls];
         for (int32_t x = 0; x < ctas; ++x) items.push_back(make_int2(idx, x));
