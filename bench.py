@@ -86,7 +86,7 @@ PROFILED_TRAFFIC = {
     # 141x141, R=4096, 10 sweeps: one launch (42.11 MB read + 21.99 MB written)
     "sweep_torus": (64.10e6, {"paper_2606_25203_gb300/csrc/sweep_nibble.cu":
                               "69b21e268255bc135dd9ddeb4be65725178d0691"}),
-    # k_dense_sweep<TCU>, 2 sweeps: the n=30,000 capture (1.6856 GB read + 3.3 MB written, the
+    # a former k_dense_sweep on byte couplings, 2 sweeps: the n=30,000 capture (1.6856 GB read + 3.3 MB written, the
     # third step of a fresh run) scaled by n^2 to n=100,000
     "dense_sweep_100k": (1.6889e9 * (100000 / 30000) ** 2, {"paper_2606_25203_gb300/csrc/dense.cu":
                                                             "855fcc6f9ccbc2654a4c49491e4e39a2ac464c6a"}),
@@ -402,7 +402,7 @@ def run_ours(args):
     iso = sweep_roofline(insts[0], args.steps, iso0, pg.pamc_sweep_stats(solvers[0].h), sm_max)
     pg.pamc_set_sweep_timing(solvers[0].h, False)
     mode = [pg.pamc_sweep_mode(s.h) for s in solvers]
-    kname = ["k_sweep_ising_nib" if m & 16 else "k_sweep_ising_push" if m == 2 else "k_sweep_ising" for m in mode]
+    kname = ["k_sweep_ising_bits" if m & 32 else "k_sweep_ising_nib" if m & 16 else "k_sweep_ising_push" if m == 2 else "k_sweep_ising" for m in mode]
     e2e = e2e_measure(pg, torch, insts, args, local, start)
     dense = None
     if world == 1 and not args.no_dense:
@@ -823,8 +823,8 @@ def dense_measure(pg, torch, n, steps, warmup, e2e=False):
     pg.pamc_destroy(h)
     peaks, src = load_peaks()
     hbm = peaks["hbm_gbs"]
-    rc_gbs = n * n / (ms_nosweep / 1e3) / 1e9            # J bytes of the recompute
-    sw_gbs = P["sweeps"] * n * n / (ms_sweep / 1e3) / 1e9  # one read of J per sweep
+    rc_gbs = n * n / 8 / (ms_nosweep / 1e3) / 1e9            # J (one bit a coupling) of the recompute
+    sw_gbs = P["sweeps"] * n * n / 8 / (ms_sweep / 1e3) / 1e9  # one read of J per sweep
     e2e_obj = None
     if e2e:
         torch.cuda.synchronize()
@@ -847,14 +847,14 @@ def dense_measure(pg, torch, n, steps, warmup, e2e=False):
         "steps": steps, "warmup": warmup, "ms_per_step": ms / steps,
         "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "int32",
         "data": "synthetic", "config": {"workload": DENSE_WORKLOAD, "n": n, **P,
-                                        "l2": "inputs (10 GB) larger than L2"},
+                                        "l2": "inputs (1.25 GB of coupling bits) larger than L2"},
         "kernels_ms": {"step": ms / steps, "sweeps": ms_sweep, "sweep_launches_timed": sw["launches"],
                        "step_without_sweeps": ms_nosweep},
         "roofline": {"bound": "hbm", "achieved": sw_gbs, "peak": hbm, "unit": "GB/s",
                      "frac": sw_gbs / hbm,
                      "traffic": (profiled_traffic("dense_sweep_100k") * (n / 100000) ** 2
                                  if profiled_traffic("dense_sweep_100k") else None),
-                     "kernel": "k_dense_sweep (bytes = one read of J per sweep)",
+                     "kernel": "k_dense_sweep (bytes = one read of J, one bit a coupling, per sweep)",
                      "peak_source": src},
         "recompute_roofline": {"bound": "hbm", "achieved": rc_gbs, "peak": hbm, "unit": "GB/s",
                                "frac": rc_gbs / hbm},

@@ -471,14 +471,18 @@ cudaError_t dense_recompute(pamc_handle h, const int8_t *src, const int32_t *par
 
 // Lanes a vertex and warps of a group on one bit a replica (sweep_bits.cu): one
 // lane where an average level has 256 vertices or more, else four, which also
-// share the long rows' sums; warps for a level's lanes, 16 (two CTAs an SM) at
-// most where the SMs hold several groups.  us per launch of 10 sweeps, 1 lane / 2 / 4:
-// N=7,000 degree 5.7 R=4,096 (levels of 350) 510 / 589 / 780, N=10,007 degree 20
-// R=2,048 (196) 1,645 / 1,250 / 1,150, N=2,000 degree 20 R=4,096 (40) 1,309 / 865 / 481.
-SweepCfg bits_shape(double avg_level, int nc, bool one_group) {
+// share the long rows' sums; two on long rows and wide levels where a group has
+// its SM to itself (alone) and its lanes hold the rows ahead.  Warps for a
+// level's lanes, 16 (two CTAs an SM) at most otherwise.  us per launch of 10 sweeps, 1 /
+// 2 / 4 lanes: N=7,000 degree 5.7 R=4,096 (levels of 350) 510 / 565 / 643, N=10,007
+// degree 20 R=2,048 (196) 1,360 / 977 / 1,133, N=2,000 degree 20 R=4,096 (40)
+// 1,187 / 717 / 455.
+SweepCfg bits_shape(double avg_level, double avg_deg, int nc, bool alone) {
     SweepCfg c{1, 4, avg_level >= 256.0 ? 1 : 4, 0, nc};
+    const bool longrows = avg_deg > 8.0;
+    if (alone && longrows && avg_level >= 150.0) c.lanes_per_vertex = 2;
     const double lanes = avg_level * c.lanes_per_vertex;
-    c.warps_per_group = lanes >= 1024.0 && one_group ? 32 : lanes >= 256.0 ? 16 : lanes >= 128.0 ? 8 : 4;
+    c.warps_per_group = lanes >= 1024.0 && alone && !longrows ? 32 : lanes >= 256.0 ? 16 : lanes >= 128.0 ? 8 : 4;
     return c;
 }
 
@@ -492,7 +496,7 @@ SweepCfg bits_shape(double avg_level, int nc, bool one_group) {
 // (two) 1,136 / 1,138, R=4,096 (seven) 2,962 / 1,335.  Narrow levels stay with the
 // 4-bit lanes where these apply (N=1,024 torus, R=2,700: 106 / 122).
 bool bits_pay(int nc, double avg_level, bool nib) { return nib ? nc >= 3 && avg_level >= 256.0 : nc >= 2; }
-SweepCfg bits_cfg(int32_t n, int32_t R, int32_t H, double avg_level, int sms, bool nib) {
+SweepCfg bits_cfg(int32_t n, int32_t R, int32_t H, double avg_level, double avg_deg, int sms, bool nib) {
     SweepCfg c{1, 1, 1, 0, 0};
     if (const char *env = getenv("PAMC_SWEEP_CFG")) {   // "1,warps,lanes,0,quads" forces it
         int a = 0, b = 0, v = 0, st = 0, nc = 0;
@@ -504,7 +508,7 @@ SweepCfg bits_cfg(int32_t n, int32_t R, int32_t H, double avg_level, int sms, bo
     const int32_t per_sm = (R + 32 * sms - 1) / (32 * sms);
     const int nc = (R + 4 * sms * per_sm - 1) / (4 * sms * per_sm);
     if (!bits_pay(nc, avg_level, nib) || sweep_bits_smem_bytes(n, H) > kSmemMax) return c;
-    return bits_shape(avg_level, nc, per_sm == 1);
+    return bits_shape(avg_level, avg_deg, nc, per_sm == 1);
 }
 
 // own: the replicas this handle sweeps (base: the first one's index in the
@@ -918,7 +922,7 @@ static pamc_status init_run(pamc_handle h, const pamc_params *pp, int32_t rank, 
     }
     if (p.kind == 0 && p.sweeps > 0 && h->bits_ok && !h->gsp && !h->cfg.staged && sweep_nibble_enabled() &&
         !sweep_push_enabled() && !(genv && genv[0] == '1')) {
-        const SweepCfg c = bits_cfg(n, own, h->H, avg_level, sms, nib_ok);
+        const SweepCfg c = bits_cfg(n, own, h->H, avg_level, (double)h->nnz / std::max(n, 1), sms, nib_ok);
         if (c.bits) h->cfg = c;
     }
     // field ranges of at most 7 on ELL rows of width 4 or 8, or of 15 a
@@ -1833,7 +1837,7 @@ pamc_status rebuild(pamc_batch b) {
         d.gsp = gl ? h->d_gsp : nullptr;
         const bool nb = member_nib(h);
         const bool bt = member_bits(h);
-        const SweepCfg cfg = bt ? bits_shape(h->avg_level, bits_nc, false) : p.kind != 0 ? peff[cls] : gl ? geff[cls] : nb ? neff[cls] : eff[cls];
+        const SweepCfg cfg = bt ? bits_shape(h->avg_level, (double)h->nnz / std::max(h->n, 1), bits_nc, false) : p.kind != 0 ? peff[cls] : gl ? geff[cls] : nb ? neff[cls] : eff[cls];
         d.push = p.kind == 0 && !gl && !nb && !bt && sweep_push_ok(h->H, p.sweeps, h->d_ell != nullptr, cfg.lanes_per_vertex)
                      ? 1 : 0;
         const int idx = (int)sw.size();

@@ -26,8 +26,11 @@
 // collected by the floating-point adder).  On the 141 x 141 torus with 28 replicas
 // a word a visit takes 614 instructions, 473 of them integer and half of
 // those Philox: 17 a replica against 24 on 4-bit lanes.  us per launch of 10 sweeps at R =
-// 4,096, before (4-bit or byte lanes) / now: the torus 1,139 / 820, N=7,000
-// degree 5.7 751 / 510, N=10,007 degree 20 2,962 / 1,335, N=2,000 degree 20 1,097 / 481.
+// 4,096, before (4-bit or byte lanes) / now: the torus 1,139 / 818, N=7,000
+// degree 5.7 751 / 503, N=10,007 degree 20 2,962 / 1,114, N=2,000 degree 20 1,097 / 455.
+// Longer rows than 8 also waited for their couplings: with up to 24 slots loaded
+// ahead, while the draws and decisions of the pass before run, N=10,007 went from
+// 1,335 to 1,114 us, N=20,000 degree 20 R=2,048 from 2,012 to 1,567.
 //
 // QL lanes share a vertex where a level has fewer vertices than the group has
 // lanes: they split its groups of four couplings (the partial sums are added
@@ -215,42 +218,66 @@ __device__ __forceinline__ void bit4(uint32_t (&x)[4], const uint4 &e, int32_t l
     }
 }
 
-// The bit sums of a position: the lane's groups of four couplings sub, sub + QL,
-// ..., the first two given (WC = 4: one group is all there is), the rest loaded
-// as the degree asks (WC = 0).
+// Rows: WC = 4 or 8 the ELL width (P = 3); else it is read at run time, with two
+// groups of four couplings a lane loaded ahead (WC = 0), or up to 24 slots of
+// the row, 128 registers a thread, where a group has its SM to itself (kDeep).
+constexpr int kDeep = 1;
+template <int QL, int WC>
+constexpr int kAhead = WC == 4 ? 1 : WC == 8 ? (QL == 1 ? 2 : 1) : WC == 0 ? 2 : QL == 1 ? 6 : QL == 2 ? 4 : 3;
+
+// loads the lane's groups sub, sub + QL, ... of position i (beyond the row: any
+// group of it, not used)
+template <int QL, int WC>
+__device__ __forceinline__ void bit_load(uint4 (&e)[kAhead<QL, WC>], const uint32_t *es, int32_t i, int32_t W, int sub) {
+#pragma unroll
+    for (int v = 0; v < kAhead<QL, WC>; ++v) {
+        const int x = sub + v * QL;
+        if (WC == 0) e[v] = ell4(es, i, W, (uint32_t)(v == 0 && QL == 1 ? 0 : min(x, (W >> 2) - 1)));
+        else if (WC == kDeep ? 4 * x < W : (QL == 1 || 4 * x < WC)) e[v] = ell4(es, i, W, (uint32_t)x);
+    }
+}
+
+// The bit sums of a position: the lane's groups of four couplings, the first
+// given, the rest of a longer row loaded as the degree asks.
 template <int P, int QL, int WC>
-__device__ __forceinline__ void bit_sum(Planes<P> &x, const uint4 &e, const uint4 &f, const uint32_t *es, int32_t i,
+__device__ __forceinline__ void bit_sum(Planes<P> &x, const uint4 (&e)[kAhead<QL, WC>], const uint32_t *es, int32_t i,
                                         int32_t W, int32_t deg, int sub, const uint32_t *sp, uint32_t flip) {
+    constexpr int NG = kAhead<QL, WC>;
 #pragma unroll
     for (int j = 0; j < P; ++j) x.p[j] = 0u;
-    const int32_t l0 = deg - 4 * sub;
-    uint32_t a[4], b[4];
-    if constexpr (WC == 4) {
-        if (QL == 1 || sub == 0) {
-            bit4(a, e, l0, sp, flip);
-            x.add4(a[0], a[1], a[2], a[3]);
-        }
-    } else if (QL == 1 || l0 > 0) {
-        bit4(a, e, l0, sp, flip);
-        if (l0 > 4 * QL) {
-            bit4(b, f, l0 - 4 * QL, sp, flip);
+    auto pair = [&](const uint4 &g, const uint4 &h, int32_t left) {   // two groups, the first not empty
+        uint32_t a[4], b[4];
+        bit4(a, g, left, sp, flip);
+        if (left > 4 * QL) {
+            bit4(b, h, left - 4 * QL, sp, flip);
             x.add8(a, b);
         } else {
             x.add4(a[0], a[1], a[2], a[3]);
         }
-        if constexpr (WC == 0) {
-            for (int32_t v = sub + 2 * QL; 4 * v < deg; v += 2 * QL) {
-                const int32_t l = deg - 4 * v;
-                const uint4 g = ell4(es, i, W, v);
-                if (l > 4 * QL) {
-                    const uint4 h = ell4(es, i, W, v + QL);
-                    bit4(a, g, l, sp, flip);
-                    bit4(b, h, l - 4 * QL, sp, flip);
-                    x.add8(a, b);
-                } else {
-                    bit4(a, g, l, sp, flip);
-                    x.add4(a[0], a[1], a[2], a[3]);
-                }
+    };
+#pragma unroll
+    for (int v = 0; v < NG; v += 2) {
+        const int32_t left = deg - 4 * (sub + v * QL);
+        if ((QL == 1 && v == 0) || left > 0) {
+            if (v + 1 < NG) {
+                pair(e[v], e[v + 1 < NG ? v + 1 : v], left);
+            } else {
+                uint32_t a[4];
+                bit4(a, e[v], left, sp, flip);
+                x.add4(a[0], a[1], a[2], a[3]);
+            }
+        }
+    }
+    if constexpr (WC <= kDeep) {
+        for (int32_t v = sub + NG * QL; 4 * v < deg; v += 2 * QL) {
+            const int32_t left = deg - 4 * v;
+            const uint4 g = ell4(es, i, W, v);
+            if (left > 4 * QL) {
+                pair(g, ell4(es, i, W, v + QL), left);
+            } else {
+                uint32_t a[4];
+                bit4(a, g, left, sp, flip);
+                x.add4(a[0], a[1], a[2], a[3]);
             }
         }
     }
@@ -262,8 +289,7 @@ __device__ __forceinline__ void bit_sum(Planes<P> &x, const uint4 &e, const uint
 }
 
 // The sweeps of one CTA's group (group g of the instance, 4 nc replicas),
-// shared by the single-instance and the batched kernels.  WC: the ELL width 4
-// or 8 (P = 3), 0 where it is read at run time.
+// shared by the single-instance and the batched kernels.
 template <int RULE, int P, int QL, int WC, class KeyT>
 __device__ __forceinline__ void
 bits_body(const SweepDesc &d, const KeyT &key, int32_t t, int32_t slot, const int8_t *__restrict__ src,
@@ -271,7 +297,7 @@ bits_body(const SweepDesc &d, const KeyT &key, int32_t t, int32_t slot, const in
     extern __shared__ __align__(16) uint8_t smem[];
     const DevCtl *ctl = d.ctl;
     if (ctl->done) return;
-    const int32_t n = d.n, H = d.H, R = d.R, S = d.S, W = WC > 0 ? WC : d.W;
+    const int32_t n = d.n, H = d.H, R = d.R, S = d.S, W = WC > kDeep ? WC : d.W;
     const BitLayout lay = bit_layout(n, H);
     const uint32_t smem0 = (uint32_t)__cvta_generic_to_shared(smem);
     const uint32_t rows0 = (smem0 + 255u) & ~255u;
@@ -340,22 +366,22 @@ bits_body(const SweepDesc &d, const KeyT &key, int32_t t, int32_t slot, const in
         uint32_t live = 0u;   // the bits of the group's replicas
         for (int32_t q = 0; q < nrep; ++q) live |= 1u << ((q >> 2) + 8 * (q & 3));
         uint32_t nflip = 0;
-        const uint32_t V = (uint32_t)W >> 2;
-        const uint32_t v0 = QL == 1 ? 0u : min((uint32_t)sub, V - 1u);
-        const uint32_t v1 = WC == 8 && QL == 1 ? 1u : min((uint32_t)(sub + QL), V - 1u);
         for (int32_t sw = 0; sw < S; ++sw) {
             const size_t sb = (size_t)slot * S + sw;
             const int32_t *lp = d.slvl + sb * (size_t)(n + 1);
             const uint32_t *es = d.sell + sb * ell_stride;
             const int2 *pos = d.spos + sb * (size_t)n;
             const int32_t L = d.snlev[sb];
-            // the record and the lane's first two groups of couplings are loaded
-            // one pass ahead, for a level's first pass before the previous
-            // level's barrier (they do not depend on spins)
+            // the record and the first couplings of a pass are loaded one pass
+            // ahead (kDeep: the couplings once this pass's are summed, beside
+            // the draws and decisions), for a level's first pass before the
+            // previous level's barrier (they do not depend on spins)
             int32_t end = 0, ip = min(vl, n - 1);
             int2 pr = pos[ip];
-            uint4 e4 = ell4(es, ip, W, v0), f4 = make_uint4(0u, 0u, 0u, 0u);
-            if (WC != 4) f4 = ell4(es, ip, W, v1);
+            uint4 e[kAhead<QL, WC>];
+#pragma unroll
+            for (int v = 0; v < kAhead<QL, WC>; ++v) e[v] = make_uint4(0u, 0u, 0u, 0u);
+            bit_load<QL, WC>(e, es, ip, W, sub);
             for (int32_t lev = 0; lev < L; ++lev) {
                 const int32_t beg = end;
                 end = lp[lev + 1];
@@ -365,15 +391,19 @@ bits_body(const SweepDesc &d, const KeyT &key, int32_t t, int32_t slot, const in
                     const bool act = i < end;
                     const int32_t inext = min(base + vpi < end ? i + vpi : end + vl, n - 1);
                     const int2 prn = pos[inext];
-                    const uint4 e4n = ell4(es, inext, W, v0);
-                    uint4 f4n = f4;
-                    if (WC != 4) f4n = ell4(es, inext, W, v1);
-                    if (QL > 1 || act) {
-                        const uint32_t a0 = (uint32_t)pr.x;
-                        const int32_t k = (int32_t)(a0 & 0xFFFFFFu);
-                        const uint32_t old = sp[k];
-                        Planes<P> x;
-                        bit_sum<P, QL, WC>(x, e4, f4, es, ip, W, (int32_t)(a0 >> 24), sub, sp, RULE == 0 ? 0u : old);
+                    uint4 en[kAhead<QL, WC>];
+                    if constexpr (WC != kDeep) bit_load<QL, WC>(en, es, inext, W, sub);
+                    const uint32_t a0 = (uint32_t)pr.x;
+                    const int32_t k = (int32_t)(a0 & 0xFFFFFFu);
+                    const bool run = QL > 1 || act;   // (QL > 1: all lanes, for the shuffles)
+                    uint32_t old = 0u;
+                    Planes<P> x;
+                    if (run) {
+                        old = sp[k];
+                        bit_sum<P, QL, WC>(x, e, es, ip, W, (int32_t)(a0 >> 24), sub, sp, RULE == 0 ? 0u : old);
+                    }
+                    if constexpr (WC == kDeep) bit_load<QL, WC>(e, es, inext, W, sub);
+                    if (run) {
                         const uint32_t D = (uint32_t)pr.y >> 24;
                         const uint32_t row = rows0 + (D << 8);
                         // replicas beyond the first threshold of 2^32
@@ -401,12 +431,12 @@ bits_body(const SweepDesc &d, const KeyT &key, int32_t t, int32_t slot, const in
                             // (lanes of a vertex beyond the last call: bits of no replica)
                             if (m == 0 || m < ncg) {
                                 const u32x4 u = draw(ctr + (uint32_t)(m + sub), key);
-                                const uint32_t e = x.bytes4(x4[m & 3], m);
+                                const uint32_t x4b = x.bytes4(x4[m & 3], m);
                                 const float bit = (float)(1 << m);
-                                bl_add_if_below(n0, u.x, bl_lds(__byte_perm(e, row, 0x7650u)), bit);
-                                bl_add_if_below(n0, u.y, bl_lds(__byte_perm(e, row, 0x7651u)), 256.0f * bit);
-                                bl_add_if_below(n1, u.z, bl_lds(__byte_perm(e, row, 0x7652u)), bit);
-                                bl_add_if_below(n1, u.w, bl_lds(__byte_perm(e, row, 0x7653u)), 256.0f * bit);
+                                bl_add_if_below(n0, u.x, bl_lds(__byte_perm(x4b, row, 0x7650u)), bit);
+                                bl_add_if_below(n0, u.y, bl_lds(__byte_perm(x4b, row, 0x7651u)), 256.0f * bit);
+                                bl_add_if_below(n1, u.z, bl_lds(__byte_perm(x4b, row, 0x7652u)), bit);
+                                bl_add_if_below(n1, u.w, bl_lds(__byte_perm(x4b, row, 0x7653u)), 256.0f * bit);
                             }
                         }
                         uint32_t nw = __byte_perm(__float_as_uint(n0), __float_as_uint(n1), 0x5410u);
@@ -424,8 +454,10 @@ bits_body(const SweepDesc &d, const KeyT &key, int32_t t, int32_t slot, const in
                     }
                     ip = inext;
                     pr = prn;
-                    e4 = e4n;
-                    f4 = f4n;
+                    if constexpr (WC != kDeep) {
+#pragma unroll
+                        for (int v = 0; v < kAhead<QL, WC>; ++v) e[v] = en[v];
+                    }
                 }
                 __syncthreads();
             }
@@ -453,13 +485,16 @@ bits_body(const SweepDesc &d, const KeyT &key, int32_t t, int32_t slot, const in
                 const int32_t deg = (int32_t)((uint32_t)p0.x >> 24);
                 dsum += (uint32_t)p0.y >> 24;
                 Planes<P> x;
-                bit_sum<P, 1, WC>(x, ell4(es, i, W, 0), ell4(es, i, W, W > 4 ? 1u : 0u), es, i, W, deg, 0, sp,
-                                  sp[p0.x & 0xFFFFFF]);
+                uint4 e[kAhead<1, WC>];
+#pragma unroll
+                for (int v = 0; v < kAhead<1, WC>; ++v) e[v] = make_uint4(0u, 0u, 0u, 0u);
+                bit_load<1, WC>(e, es, i, W, 0);
+                bit_sum<P, 1, WC>(x, e, es, i, W, deg, 0, sp, sp[p0.x & 0xFFFFFF]);
 #pragma unroll
                 for (int m = 0; m < 8; ++m) {
-                    const uint32_t e = x.bytes4(x.nibbles(m & 3), m);
-                    acc[2 * m] += (e >> 2) & 0x003F003Fu;
-                    acc[2 * m + 1] += (e >> 10) & 0x003F003Fu;
+                    const uint32_t y = x.bytes4(x.nibbles(m & 3), m);
+                    acc[2 * m] += (y >> 2) & 0x003F003Fu;
+                    acc[2 * m + 1] += (y >> 10) & 0x003F003Fu;
                 }
             }
 #pragma unroll
@@ -492,7 +527,7 @@ bits_body(const SweepDesc &d, const KeyT &key, int32_t t, int32_t slot, const in
 }
 
 template <int RULE, int P, int QL, int WC>
-__global__ void __launch_bounds__(1024) k_sweep_ising_bits(SweepDesc d, int nc) {
+__global__ void __launch_bounds__(WC == kDeep ? 512 : 1024) k_sweep_ising_bits(SweepDesc d, int nc) {
     bits_body<RULE, P, QL, WC>(d, BitKeys{d.K}, d.t, d.slot, d.src, d.dst, d.E_dst, nc, blockIdx.x);
 }
 
@@ -530,7 +565,13 @@ cudaError_t launch_sweep_ising_bits(int rule, int32_t n, int32_t H, const pamc_p
                                     const DevCtl *ctl, SweepCfg cfg, cudaStream_t st, int32_t rbase) {
     if (sv.ell == nullptr || p.sweeps < 1 || H > kBitLaneMaxH || cfg.bits < 1 || cfg.bits > 8) return cudaErrorInvalidValue;
     const int nc = cfg.bits, groups = (p.R + 4 * nc - 1) / (4 * nc);
-    const int threads = cfg.warps_per_group * 32;
+    const int planes = sweep_bits_planes(H);
+    int dev = 0, sms = 0;
+    cudaError_t err = cudaGetDevice(&dev);
+    if (err == cudaSuccess) err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (err != cudaSuccess) return err;
+    const bool deep = planes > 3 && cfg.warps_per_group <= 16 && groups <= sms;
+    const int threads = 32 * cfg.warps_per_group;
     SweepDesc d;
     memset(&d, 0, sizeof(d));
     d.slvl = sv.lvl_ptr; d.snlev = sv.nlev; d.sell = sv.ell; d.spos = sv.pos;
@@ -539,8 +580,6 @@ cudaError_t launch_sweep_ising_bits(int rule, int32_t n, int32_t H, const pamc_p
     d.S = p.sweeps; d.t = t; d.slot = slot; d.W = sv.W; d.K = make_philox_keys(p.seed);
     d.gbase = rbase / 4;
     const size_t smem = sweep_bits_smem_bytes(n, H);
-    const int planes = sweep_bits_planes(H);
-    cudaError_t err = cudaSuccess;
 #define PAMC_BITS(RU, PL, Q, WV)                                                              \
     do {                                                                                      \
         err = allow_dynamic_smem(k_sweep_ising_bits<RU, PL, Q, WV>, smem);                    \
@@ -557,7 +596,9 @@ cudaError_t launch_sweep_ising_bits(int rule, int32_t n, int32_t H, const pamc_p
     do {                                                                                      \
         if (planes == 3 && sv.W == 4) PAMC_BITS_Q(RU, 3, 4);                                  \
         else if (planes == 3) PAMC_BITS_Q(RU, 3, 8);                                          \
-        else if (planes == 5) PAMC_BITS_Q(RU, 5, 0);                                              \
+        else if (planes == 5 && deep) PAMC_BITS_Q(RU, 5, kDeep);                              \
+        else if (planes == 5) PAMC_BITS_Q(RU, 5, 0);                                          \
+        else if (deep) PAMC_BITS_Q(RU, 6, kDeep);                                             \
         else PAMC_BITS_Q(RU, 6, 0);                                                           \
     } while (0)
     if (rule == 0) PAMC_BITS_P(0);
@@ -571,7 +612,7 @@ cudaError_t launch_sweep_ising_bits(int rule, int32_t n, int32_t H, const pamc_p
 cudaError_t launch_sweep_ising_bits_batched(int rule, int planes, int lanes, int warps, int nc, size_t smem,
                                             const SweepDesc *descs, const int2 *items, int32_t nitems, cudaStream_t st) {
     if (nitems <= 0) return cudaSuccess;
-    if (nc < 1 || nc > 8 || warps < 1 || warps > 32) return cudaErrorInvalidValue;
+    if (nc < 1 || nc > 8 || warps < 1 || warps > 16) return cudaErrorInvalidValue;
     cudaError_t err = cudaSuccess;
 #define PAMC_BITB(RU, PL, Q)                                                                  \
     do {                                                                                      \
