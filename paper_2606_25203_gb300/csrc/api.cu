@@ -319,9 +319,9 @@ size_t gsp_words(int32_t n, int32_t R) { return (size_t)((R + 3) / 4) * (size_t)
 // Launch shape of the sweep kernel: groups per CTA, warps per group and
 // lanes per vertex.  Ising runs on ELL schedules give each group a CTA of its
 // own, sized for the latency of a level, unless the SMs are shared and the
-// levels are too wide for more than one lane per vertex; Potts runs do the
-// same (one lane per vertex) where an average level fits the group's share
-// of the SM in one pass.  Otherwise every (gpc, wpg) is scored by the fraction of group slots used
+// levels are too wide for more than one lane per vertex; Potts runs on ELL
+// rows likewise (pairs, quads), on CSR rows where an average level fits the
+// group's share of the SM in one pass.  Otherwise every (gpc, wpg) is scored by the fraction of group slots used
 // over whole waves, the lane efficiency of a level (average level size over
 // the lanes of a group), and resident warps per SM; Ising runs on ELL
 // schedules then give the lanes a level leaves idle to the couplings (the

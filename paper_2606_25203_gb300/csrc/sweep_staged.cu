@@ -12,11 +12,11 @@
 // the next into registers, so that a level costs its own chain only -- barrier,
 // shared loads of the neighbours' spin words, sum, threshold, store.  (A warp
 // alone on its scheduler spends about five cycles an instruction; reading ahead
-// in the same warp doubled the chain.)  A launch of 10 sweeps at N=800, degree
+// in the same warp doubled the chain.)  A launch of 5 sweeps at N=800, degree
 // 48, R=128 went from 340 to 214 us with it, one of 5 sweeps at N=2,500, degree
 // 12, weights to 100 (16-bit lanes), R=250 from 624 to 175 us.  LPV lanes share
-// a vertex, each sums its groups of four couplings; the partial sums are added across the lanes, and
-// lane q < 4 decides replica q (two replicas a lane with LPV = 2, four with LPV
+// a vertex, each sums its groups of four couplings; the partial sums are added
+// across the lanes, and lane q < 4 decides replica q (two replicas a lane with LPV = 2, four with LPV
 // = 1) and stores its part of the word.  Draws, orders and results are those of
 // the other Ising sweeps bit for bit.
 //
