@@ -212,7 +212,19 @@ extern "C" pamc_status pamc_sweeps_noalloc(int32_t n, int32_t nnz, const int32_t
     if (sweeps > 0)
         launch_schedule(n, row_ptr, adj, seed, t, 1, sweeps, 0, 1, order, lvl, nlev, skey, scnt, s);
     e = launch_tables(0, rule, H, ctl, tab, s);
+    // warps of a group: at least by the size (the levels' width), more where few
+    // groups share an SM, up to one lane for three vertices or so.  us per call of 4
+    // sweeps, 4 / 8 / 16 / 32 warps: n = 7,000 R=256 (one group an SM) 563 / 482 /
+    // 447 / 408, R=1,024 (two) 581 / 516 / 478 / 528, R=2,048 (four) 640 / 598 / 661 /
+    // 745; n = 2,000 R=1,024 248 / 234 / 224 / 275; n = 20,000 R=100 1,214 / 942 /
+    // 845 / 807; n = 300 the same at any.
     SweepCfg cfg{1, n >= 16384 ? 8 : n >= 4096 ? 4 : n >= 1024 ? 2 : 1};
+    int cur = 0, sms = 1;
+    if (cudaGetDevice(&cur) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, cur) != cudaSuccess)
+        sms = 1;
+    const int64_t per_sm = ((R + 3) / 4 + sms - 1) / sms;
+    while (2 * cfg.warps_per_group * per_sm <= 32 && 200 * cfg.warps_per_group <= n) cfg.warps_per_group *= 2;
     // spins_in may equal spins_out: the sweep's CTA for a replica group reads
     // the group's rows completely into shared memory before its first write,
     // and no other CTA touches those rows
