@@ -190,11 +190,15 @@ k_sweep_ising_staged(SweepDesc d, int cwarps, int nb) {
         }
     }
     __syncthreads();
-    // one lane polls, the others learn the outcome from it
+    // one lane polls, the others learn the outcome from it; the warp barrier
+    // orders their accesses to the slot after what that lane acquired (a
+    // shuffle orders no memory)
     auto wait = [&](uint64_t *b, uint32_t parity, uint32_t pause_ns) -> bool {
         bool ok = true;
         if (lane == 0) ok = mbar_try_wait(b, parity) || st_wait_slow(b, parity, pause_ns, &s_err, ctl);
-        return __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
+        ok = __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
+        __syncwarp();
+        return ok;
     };
 
     uint32_t nflip = 0;
@@ -386,8 +390,11 @@ k_sweep_ising_staged(SweepDesc d, int cwarps, int nb) {
             // then the next pass is read while the other set works
             if (cur < (fsw < S ? glev : glev - 1)) level_barrier();
             read(b);
-            // blocks before this warp's next pass are not read by it any more
+            // blocks before this warp's next pass are not read by it any more: the
+            // warp barrier puts every lane's reads (the long rows' loop above ends
+            // at each lane's own degree) before the arrival that hands them back
             const int32_t upto = b.sw < S ? b.sw * nblk + (b.base >> 5) : S * nblk;
+            __syncwarp();
             if (lane == 0)
                 for (int32_t x = freed; x < upto; ++x) st_arrive(&empty[(uint32_t)x & nbm]);
             freed = upto;

@@ -237,6 +237,34 @@ def test_staged_sweep(pg, monkeypatch, cfg):
         compare_run(pg, inst, 3, **p)
 
 
+@pytest.mark.parametrize("cfg", ["1,1,1,1", "1,2,1,1", "1,3,2,1"])
+def test_staged_sweep_uneven_rows(pg, monkeypatch, cfg):
+    """Lanes of one warp whose rows end far apart (hubs of up to 120 couplings
+    beside rows of a few): a block goes back to the producers only when the
+    slowest lane has read it, over a ring that wraps many times."""
+    n, rng = 400, np.random.default_rng(5)
+    adj = np.triu(rng.random((n, n)) < 0.05, 1)
+    for hub in rng.choice(n, 24, replace=False):
+        for x in rng.choice(n, 95, replace=False):
+            adj[min(hub, x), max(hub, x)] |= hub != x
+    i, j = np.nonzero(adj)
+    keep = np.ones(i.shape[0], dtype=bool)
+    deg = np.zeros(n, dtype=int)
+    for e, (a, b) in enumerate(zip(i, j)):
+        keep[e] = deg[a] < 120 and deg[b] < 120
+        deg[a] += keep[e]
+        deg[b] += keep[e]
+    inst = W.csr_from_edges(n, i[keep], j[keep], rng.choice([-1, 1], int(keep.sum())), "hubs")
+    assert deg.max() == 120 and deg.min() < 16
+    monkeypatch.setenv("PAMC_SWEEP_CFG", cfg)
+    s = pg.Solver(inst.row_ptr, inst.col, inst.w)
+    s.init(R=7, sweeps=8, steps=3, seed=2)
+    assert pg.pamc_sweep_mode(s.h) == 1 and tuple(pg.pamc_sweep_shape(s.h)) == tuple(int(x) for x in cfg.split(",")[:3])
+    s.close()
+    for rule in (0, 1):
+        compare_run(pg, inst, 3, R=7, sweeps=8, beta0=0.05, beta1=1.0, rule=rule, seed=2)
+
+
 @pytest.mark.parametrize("cfg", ["1,1,1,0,8", "1,2,2,0,3", "1,4,4,0,7", "1,3,4,0,1", "1,32,1,0,5"])
 def test_bit_lanes(pg, monkeypatch, cfg):
     """One bit a replica: words of 1 to 8 quads, one to four lanes a vertex,
