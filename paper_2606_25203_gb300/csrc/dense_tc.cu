@@ -189,7 +189,7 @@ k_dense_recompute_tc(const __grid_constant__ CUtensorMap tmJ, const __grid_const
             for (int32_t u = lo; ok && u < hi; ++u) {
                 const bool first = u == lo || u % nch == 0;
                 if (first && seg > 0) {   // the accumulators of the last block have been read
-                    if (!wait(&drained, (uint32_t)((seg - 1) & 1))) break;
+                    if (!wait(&drained, (uint32_t)((seg - 1) & 1))) break;   // (nothing issued since the commit)
                     tc_fence_after();
                 }
                 const int32_t ns = slices(u);
@@ -215,7 +215,11 @@ k_dense_recompute_tc(const __grid_constant__ CUtensorMap tmJ, const __grid_const
                     ++seg;
                 }
             }
-            if (!ok) {   // MMAs issued before a wait ran out complete before tensor memory is freed
+            // every MMA issued has completed before tensor memory is freed (bounded):
+            // first the last block's commit -- whatever became of the warps that
+            // read it -- then what a wait that ran out left uncommitted
+            if (seg > 0) mbar_wait(&done, (uint32_t)((seg - 1) & 1));
+            if (!ok) {
                 tc_commit(&done);
                 mbar_wait(&done, (uint32_t)(seg & 1));
             }
