@@ -473,7 +473,9 @@ bits_body(const SweepDesc &d, const KeyT &key, int32_t t, int32_t slot, const in
         const size_t sb = (size_t)slot * S + (S - 1);   // S >= 1
         const uint32_t *es = d.sell + sb * ell_stride;
         const int2 *pos = d.spos + sb * (size_t)n;
-        for (int32_t i0 = li; i0 < n; i0 += 1024 * tpg) {   // (1024 x 63 < 2^16)
+        // (a warp's lanes run it together for the reduction; 1024 x 63 < 2^16)
+        for (int32_t w0 = li - lane; w0 < n; w0 += 1024 * tpg) {
+            const int32_t i0 = w0 + lane;
             uint32_t acc[16];
 #pragma unroll
             for (int q = 0; q < 16; ++q) acc[q] = 0u;
@@ -502,9 +504,8 @@ bits_body(const SweepDesc &d, const KeyT &key, int32_t t, int32_t slot, const in
                 const int b = q & 3;
                 int32_t s = (int32_t)((acc[2 * (q >> 2) + (b & 1)] >> (16 * (b >> 1))) & 0xFFFFu) * 2 - (int32_t)dsum;
                 if (q < nrep) {   // (the same for the whole group)
-                    const unsigned mask = __activemask();
-                    s = __reduce_add_sync(mask, s);
-                    if ((__ffs(mask) - 1) == lane) atomicAdd(&red[q], (unsigned long long)(long long)s);
+                    s = __reduce_add_sync(0xffffffffu, s);
+                    if (lane == 0) atomicAdd(&red[q], (unsigned long long)(long long)s);
                 }
             }
         }
