@@ -19,7 +19,8 @@
 // Decision.  For a vertex of weight D the new spin depends on the draw and an
 // index x in [0, D], the threshold rising with x: heat-bath x = N (s = +1 iff
 // u < T(2x - D)), Metropolis x = the unsatisfied weight D - N for s = +1, N for
-// s = -1 (flip iff u < T_M(D - 2x)).  Shared memory holds a row of 32-bit
+// s = -1 (flip iff u < T_M(D - 2x)).  At a negative beta, heat-bath, the
+// threshold falls with the field: x = D - N, T(D - 2x).  Shared memory holds a row of 32-bit
 // thresholds for each D, 256 bytes apart, so that the address of a replica's
 // entry is the row address with its lowest byte replaced by 4 x: one byte
 // permute.  A threshold of 2^32 (always) does not fit 32 bits: those entries
@@ -101,8 +102,18 @@ __host__ __device__ constexpr size_t nib_table_bytes(int32_t H) { return (size_t
 // mark word, X the index nibbles (one half only).
 template <int RULE, bool TWO>
 __device__ __forceinline__ uint32_t nib_decide(uint32_t X, uint32_t E, uint32_t O, uint32_t D, uint32_t row,
-                                               uint32_t force, const u32x4 &ua, const u32x4 &ub, uint32_t old) {
-    if constexpr (RULE == 1) {   // the unsatisfied weight of the replicas with s = +1
+                                               uint32_t force, bool falling, const u32x4 &ua, const u32x4 &ub,
+                                               uint32_t old) {
+    if constexpr (RULE == 0) {
+        if (falling) {   // uniform over the launch: the index counts the other way
+            if constexpr (TWO) {
+                E = D * 0x01010101u - E;
+                O = D * 0x01010101u - O;
+            } else {
+                X = D * 0x11111111u - X;
+            }
+        }
+    } else {   // the unsatisfied weight of the replicas with s = +1
         if constexpr (TWO) {
             const uint32_t me = (old & 0x01010101u) * 0xFFu, mo = ((old >> 4) & 0x01010101u) * 0xFFu;
             const uint32_t D4 = D * 0x01010101u;
@@ -166,16 +177,19 @@ nib_body(const SweepDesc &d, const KeyT &draw, int32_t t, int32_t slot, const in
     const uint32_t marks0 = rows0 + (uint32_t)(H + 1) * (kNibRow * 4);
     uint32_t *spins_all = reinterpret_cast<uint32_t *>(smem + ((nib_table_bytes(H) + 15) & ~(size_t)15));
     unsigned long long *red = reinterpret_cast<unsigned long long *>(spins_all + (size_t)gpc * n_pad);
+    // tab[h + H] (heat-bath), tab[s h + H] (Metropolis): h = 2x - D (D - 2x where
+    // the thresholds fall with the field, beta < 0), s h = D - 2x
+    const bool falling = RULE == 0 && d.tab[0] > d.tab[2 * H];
+    const bool up = RULE == 0 && !falling;
     for (int i = threadIdx.x; i < (H + 1) * (H + 1); i += blockDim.x) {
         const int32_t D = i / (H + 1), x = i % (H + 1);
         if (x > D) continue;
-        // tab[h + H] (heat-bath), tab[s h + H] (Metropolis): h = 2x - D, s h = D - 2x
-        const uint64_t T = d.tab[RULE == 0 ? 2 * x - D + H : D - 2 * x + H];
+        const uint64_t T = d.tab[up ? 2 * x - D + H : D - 2 * x + H];
         tab_s[D * kNibRow + x] = T > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)T;
     }
     for (int32_t D = threadIdx.x; D <= H; D += blockDim.x) {
         int32_t xf = 0;   // first entry of 2^32 (D + 1: none)
-        while (xf <= D && d.tab[RULE == 0 ? 2 * xf - D + H : D - 2 * xf + H] <= 0xFFFFFFFFull) ++xf;
+        while (xf <= D && d.tab[up ? 2 * xf - D + H : D - 2 * xf + H] <= 0xFFFFFFFFull) ++xf;
         mark_s[D] = TWO ? (uint32_t)(128 - xf) * 0x01010101u : (uint32_t)(8 - xf) * 0x11111111u;
     }
     for (int i = threadIdx.x; i < gpc * 8; i += blockDim.x) red[i] = 0ull;
@@ -273,7 +287,7 @@ nib_body(const SweepDesc &d, const KeyT &draw, int32_t t, int32_t slot, const in
                     const uint32_t row = rows0 + (D << 8), force = lds_u32(marks0 + (D << 2));
                     uint32_t E = 0u, O = 0u;
                     if constexpr (TWO) nib_halves(A, A2, E, O);
-                    const uint32_t nw = nib_decide<RULE, TWO>(A, E, O, D, row, force, ua, ub, old);
+                    const uint32_t nw = nib_decide<RULE, TWO>(A, E, O, D, row, force, falling, ua, ub, old);
                     if (nw != old) {
                         sp[k] = nw;
                         nflip += __popc((nw ^ old) & live);

@@ -632,6 +632,22 @@ def test_nibble_lanes(pg, monkeypatch, nib, rule):
                     cooldown_tau=1, win_short=2, win_long=3, seed=4)
 
 
+@pytest.mark.parametrize("rule", [0, 1])
+def test_nibble_lanes_negative_beta(pg, rule):
+    """At a negative beta the heat-bath threshold falls with the field: one and
+    two halves, with saturated rows, through zero to positive beta and back
+    (a schedule that reverses), ragged populations, against the oracle."""
+    for inst, R in ((W.torus(18, 18, signed=True, seed=3), 13), (_max_degree_graph(300, 700, 6, 5), 8),
+                    (_max_degree_graph(600, 3600, 16, 8), 27),
+                    (_max_degree_graph(500, 2000, 16, 10, weights=(-2, -1, -1, 1, 1, 2)), 9)):
+        for beta0, beta1 in ((-3.0, 1.0), (0.2, -4.0), (-0.3, -0.2)):
+            s = pg.Solver(inst.row_ptr, inst.col, inst.w)
+            s.init(R=R, sweeps=2, steps=5, rule=rule, beta0=beta0, beta1=beta1, seed=4)
+            assert pg.pamc_sweep_mode(s.h) == 17, inst.name
+            s.close()
+            compare_run(pg, inst, 5, R=R, sweeps=2, beta0=beta0, beta1=beta1, rule=rule, seed=4)
+
+
 def test_nibble_lanes_limits(pg):
     """A half-row range of 16 (or a row wider than 16) keeps the byte lanes;
     15 takes the biased 4-bit lanes."""
