@@ -10,8 +10,9 @@
 // with the coupling's sign for all replicas of the group; the bits are counted
 // by carry-save adders into P bit planes (x = their sum, up to 2^P - 1), two
 // three-input logic operations a neighbour.  Heat-bath counts x = N, the
-// neighbours with J_kj s_j = +1 (h = 2N - D, D the row's weight); Metropolis
-// the unsatisfied ones, J_kj s_j = -s_k (one more input to the exclusive or).
+// neighbours with J_kj s_j = +1 (h = 2N - D, D the row's weight), at a negative
+// beta, where the threshold falls with the field, x = D - N; Metropolis the
+// unsatisfied ones, J_kj s_j = -s_k (one more input to the exclusive or).
 //
 // Decision.  As in sweep_nibble.cu: shared memory holds, for each D, a row of
 // 32-bit thresholds 256 bytes apart; the planes are merged into bytes 4 x (pairs
@@ -203,8 +204,8 @@ __host__ __device__ __forceinline__ BitLayout bit_layout(int32_t n, int32_t H) {
 
 __device__ __forceinline__ uint32_t sign_mask(uint32_t e) { return (uint32_t)((int32_t)e >> 31); }
 
-// Four neighbours' bits [J_kj s_j = +1] (flip: [J_kj s_j = -1] where it is all
-// ones); slots at or beyond the row's end (left of them in the group) give 0.
+// Four neighbours' bits [J_kj s_j = +1] ([J_kj s_j = -1] in the bits that flip
+// sets); slots at or beyond the row's end (left of them in the group) give 0.
 __device__ __forceinline__ void bit4(uint32_t (&x)[4], const uint4 &e, int32_t left, const uint32_t *sp, uint32_t flip) {
     x[0] = sp[e.x & 0xFFFFFFu] ^ sign_mask(e.x) ^ flip;
     x[1] = sp[e.y & 0xFFFFFFu] ^ sign_mask(e.y) ^ flip;
@@ -304,16 +305,19 @@ bits_body(const SweepDesc &d, const KeyT &key, int32_t t, int32_t slot, const in
     uint32_t *tab_s = reinterpret_cast<uint32_t *>(smem + (rows0 - smem0));
     uint32_t *mark_s = tab_s + (H + 1) * kBitRow;
     const uint32_t marks0 = rows0 + (uint32_t)(H + 1) * (kBitRow * 4);
+    // tab[h + H] (heat-bath), tab[s h + H] (Metropolis): h = 2x - D (D - 2x where
+    // the thresholds fall with the field, beta < 0), s h = D - 2x
+    const bool falling = RULE == 0 && d.tab[0] > d.tab[2 * H];
+    const bool up = RULE == 0 && !falling;
     for (int i = threadIdx.x; i < (H + 1) * (H + 1); i += blockDim.x) {
         const int32_t D = i / (H + 1), x = i % (H + 1);
         if (x > D) continue;
-        // tab[h + H] (heat-bath), tab[s h + H] (Metropolis): h = 2x - D, s h = D - 2x
-        const uint64_t T = d.tab[RULE == 0 ? 2 * x - D + H : D - 2 * x + H];
+        const uint64_t T = d.tab[up ? 2 * x - D + H : D - 2 * x + H];
         tab_s[D * kBitRow + x] = T > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)T;
     }
     for (int32_t D = threadIdx.x; D <= H; D += blockDim.x) {
         int32_t xf = 0;   // first entry of 2^32 (D + 1: none)
-        while (xf <= D && d.tab[RULE == 0 ? 2 * xf - D + H : D - 2 * xf + H] <= 0xFFFFFFFFull) ++xf;
+        while (xf <= D && d.tab[up ? 2 * xf - D + H : D - 2 * xf + H] <= 0xFFFFFFFFull) ++xf;
         // word 0: carry in, words 1..6: the bits of what is added to x
         const uint32_t c = xf == 0 ? 63u : (uint32_t)((1 << P) - xf);
         mark_s[D * 8] = xf == 0 ? 0xFFFFFFFFu : 0u;
@@ -365,6 +369,7 @@ bits_body(const SweepDesc &d, const KeyT &key, int32_t t, int32_t slot, const in
         const uint32_t ctr = (kTagFlip << 24) | (uint32_t)(nc * g + d.gbase);
         uint32_t live = 0u;   // the bits of the group's replicas
         for (int32_t q = 0; q < nrep; ++q) live |= 1u << ((q >> 2) + 8 * (q & 3));
+        const uint32_t other = falling ? 0xFFFFFFFFu : 0u;   // heat-bath: counts D - N
         uint32_t nflip = 0;
         for (int32_t sw = 0; sw < S; ++sw) {
             const size_t sb = (size_t)slot * S + sw;
@@ -400,7 +405,7 @@ bits_body(const SweepDesc &d, const KeyT &key, int32_t t, int32_t slot, const in
                     Planes<P> x;
                     if (run) {
                         old = sp[k];
-                        bit_sum<P, QL, WC>(x, e, es, ip, W, (int32_t)(a0 >> 24), sub, sp, RULE == 0 ? 0u : old);
+                        bit_sum<P, QL, WC>(x, e, es, ip, W, (int32_t)(a0 >> 24), sub, sp, RULE == 0 ? other : old);
                     }
                     if constexpr (WC == kDeep) bit_load<QL, WC>(e, es, inext, W, sub);
                     if (run) {

@@ -306,6 +306,24 @@ def test_bit_lanes(pg, monkeypatch, cfg):
     compare_run(pg, inst, 2, R=1300, sweeps=2, beta0=0.2, beta1=2.0, seed=3)
 
 
+@pytest.mark.parametrize("cfg", ["1,2,1,0,8", "1,2,2,0,3", "1,4,4,0,5"])
+@pytest.mark.parametrize("rule", [0, 1])
+def test_bit_lanes_negative_beta(pg, monkeypatch, cfg, rule):
+    """At a negative beta the heat-bath threshold falls with the field: three,
+    five and six planes, with saturated rows, through zero to positive beta and
+    back, against the oracle."""
+    k64 = W.csr_from_edges(64, *np.triu_indices(64, 1), np.resize([1, -1, 1, 1, 1], 64 * 63 // 2), "k64")
+    monkeypatch.setenv("PAMC_SWEEP_CFG", cfg)
+    for inst, R in ((W.torus(18, 18, seed=3), 37), (_max_degree_graph(300, 900, 7, 6), 33),
+                    (_max_degree_graph(300, 2600, 31, 7), 29), (k64, 9)):
+        for beta0, beta1 in ((-3.0, 1.0), (0.2, -4.0), (-0.3, -0.2)):
+            s = pg.Solver(inst.row_ptr, inst.col, inst.w)
+            s.init(R=R, sweeps=2, steps=5, rule=rule, beta0=beta0, beta1=beta1, seed=4)
+            assert pg.pamc_sweep_mode(s.h) == 33, inst.name
+            s.close()
+            compare_run(pg, inst, 5, R=R, sweeps=2, beta0=beta0, beta1=beta1, rule=rule, seed=4)
+
+
 def test_independent_chains_baseline(pg):
     inst = W.gnm(400, 1100, signed=True, seed=6)
     compare_run(pg, inst, 6, R=9, sweeps=2, resample=0, seed=1)
