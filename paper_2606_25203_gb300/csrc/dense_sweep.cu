@@ -13,7 +13,8 @@
 // their draws; a position is a candidate when it would flip now, or when some
 // field change of at most 2 m (m flips) could change its decision (the
 // acceptance thresholds are monotone in the field, so comparing the draw with
-// the thresholds at h - 2m and h + 2m decides that).  Every other position
+// the thresholds at h - 2m and h + 2m decides that; at a negative beta they
+// fall with the field, and the heat-bath decisions read the table at -h).  Every other position
 // keeps its spin whatever the first m flips of the batch are.  The candidates
 // (at most kCand, in order) are then decided one after the other by one warp
 // from their fields and the bit tile of the couplings among them; before a
@@ -85,35 +86,36 @@ struct DsSmem {               // fixed part of a CTA's shared memory
     int32_t cq[kCand];                // (leader) 2 (margin) + spin bit, see below
     uint4 tile[kCand];                // (leader) J[candidate][candidate], one bit each
     BatchOut out;
-    int32_t lo, hi, nwin;
+    int32_t lo, hi, nwin, dir;
     unsigned long long esum;
 };
 
-// u < T(x): x = h (heat-bath, T rising with h) or s h (Metropolis, T falling
-// with x).  Inside [lo, hi) the threshold lies strictly between 0 and 2^32.
+// u < T(x): x = dir h (heat-bath, dir = -1 at a negative beta: T rising with x)
+// or s h (Metropolis, T falling with x).  Inside [lo, hi) the threshold lies
+// strictly between 0 and 2^32.
 struct Accept {
     const uint32_t *win;
     const uint64_t *tab;
-    int32_t lo, hi, off, rising;
+    int32_t lo, hi, off, rising, dir;
     bool inwin;
     __device__ __forceinline__ bool operator()(int32_t x, uint32_t u) const {
         if (x < lo) return !rising;
         if (x >= hi) return rising;
         // all fields of a run have the parity of n - 1, so every other entry is kept
-        return inwin ? u < win[(x - lo) >> 1] : (uint64_t)u < tab[x + off];
+        return inwin ? u < win[(x - lo) >> 1] : (uint64_t)u < tab[dir * x + off];
     }
     // whether the visit flips spin s (0 or 1) at field h
     __device__ __forceinline__ bool flips(int32_t h, uint32_t s, uint32_t u) const {
-        if (rising) return (*this)(h, u) != (s != 0u);
+        if (rising) return (*this)(dir * h, u) != (s != 0u);
         return (*this)(s ? h : -h, u);
     }
     // whether some field within m of h decides differently from another
     __device__ __forceinline__ bool fragile(int32_t h, uint32_t s, uint32_t u, int32_t m) const {
-        const int32_t x = rising || s ? h : -h;
+        const int32_t x = rising ? dir * h : s ? h : -h;
         return (*this)(x - m, u) != (*this)(x + m, u);
     }
-    // margin of the decision in flips of other spins: with v = h (s = -1) or
-    // -h (s = +1) the visit flips s iff v is at least some value (both rules),
+    // margin of the decision in flips of other spins: with v = dir h (s = -1) or
+    // -dir h (s = +1) the visit flips s iff v is at least some value (both rules),
     // a field changes by 2 a flip, and q >= 0 iff it flips now: the largest
     // number of adverse flips it survives, or minus the favourable ones it
     // needs; clamped to [-m - 1, m]
@@ -121,7 +123,7 @@ struct Accept {
         int32_t lo2 = -m, hi2 = m + 1;   // smallest x in [-m, m] at which v + 2x flips, m + 1 if none
         while (lo2 < hi2) {
             const int32_t mid = (lo2 + hi2) >> 1;
-            if (flips(s ? h - 2 * mid : h + 2 * mid, s, u)) hi2 = mid;
+            if (flips(s ? h - 2 * dir * mid : h + 2 * dir * mid, s, u)) hi2 = mid;
             else lo2 = mid + 1;
         }
         return -lo2;
@@ -171,12 +173,17 @@ __global__ void __launch_bounds__(kDsThreads, 1) k_dense_sweep(DenseSweepArgs a,
     if (threadIdx.x == 0) {
         // [lo, hi): where the threshold is neither 0 nor 2^32
         int32_t lo, hi;
-        if (a.rule == 0) {   // tab[i] = T(i - Hc), rising
-            int32_t l = 0, h2 = 2 * a.Hc + 1;
-            while (l < h2) { const int32_t md = (l + h2) >> 1; if (a.tab[md] > 0ull) h2 = md; else l = md + 1; }
+        sm.dir = 1;
+        if (a.rule == 0) {   // tab[i] = T(i - Hc), rising (falling at a negative beta: read from its end)
+            const int32_t last = 2 * a.Hc;
+            const bool back = a.tab[0] > a.tab[last];
+            auto T = [&](int32_t i) { return a.tab[back ? last - i : i]; };
+            sm.dir = back ? -1 : 1;
+            int32_t l = 0, h2 = last + 1;
+            while (l < h2) { const int32_t md = (l + h2) >> 1; if (T(md) > 0ull) h2 = md; else l = md + 1; }
             lo = l - a.Hc;
-            h2 = 2 * a.Hc + 1;
-            while (l < h2) { const int32_t md = (l + h2) >> 1; if (a.tab[md] >= (1ull << 32)) h2 = md; else l = md + 1; }
+            h2 = last + 1;
+            while (l < h2) { const int32_t md = (l + h2) >> 1; if (T(md) >= (1ull << 32)) h2 = md; else l = md + 1; }
             hi = l - a.Hc;
         } else {             // tab[x] = T_M(2x), falling from tab[0] = 2^32
             int32_t l = 0, h2 = a.Hc + 1;
@@ -193,9 +200,10 @@ __global__ void __launch_bounds__(kDsThreads, 1) k_dense_sweep(DenseSweepArgs a,
         sm.esum = 0ull;
     }
     __syncthreads();
-    Accept acc{sm.win, a.tab, sm.lo, sm.hi, a.rule == 0 ? a.Hc : 0, a.rule == 0 ? 1 : 0, sm.nwin <= kDsWin};
+    Accept acc{sm.win, a.tab, sm.lo, sm.hi, a.rule == 0 ? a.Hc : 0, a.rule == 0 ? 1 : 0, sm.dir,
+               sm.nwin <= kDsWin};
     if (acc.inwin)
-        for (int32_t i = threadIdx.x; i < sm.nwin; i += kDsThreads) sm.win[i] = (uint32_t)a.tab[acc.lo + 2 * i + acc.off];
+        for (int32_t i = threadIdx.x; i < sm.nwin; i += kDsThreads) sm.win[i] = (uint32_t)a.tab[acc.dir * (acc.lo + 2 * i) + acc.off];
     const int32_t nrw = (n + 31) >> 5;
     const uint32_t ctr3 = (kTagFlip << 24) | (uint32_t)((r >> 2) + a.gbase);
     sync_all();   // every CTA of the cluster runs before another one writes its memory
@@ -339,10 +347,11 @@ __global__ void __launch_bounds__(kDsThreads, 1) k_dense_sweep(DenseSweepArgs a,
                         open = 0xfffffffeu << o;   // positions up to this one are decided
                         const uint4 tj = sm.tile[j];
                         const uint32_t neg = (sb[s] >> o) & 1u;   // +1 turns to -1
+                        const uint32_t down = (0u - neg) ^ (acc.dir < 0 ? 0xFFFFFFFFu : 0u);
                         const uint32_t tw[4] = {tj.x, tj.y, tj.z, tj.w};
 #pragma unroll
                         for (int s3 = s; s3 < kCand / 32; ++s3)
-                            q[s3] += 2 * (int32_t)(((tw[s3] ^ sb[s3] ^ (0u - neg)) >> lane) & 1u) - 1;
+                            q[s3] += 2 * (int32_t)(((tw[s3] ^ sb[s3] ^ down) >> lane) & 1u) - 1;
                         if (lane == 0) sm.out.flip[f] = (uint32_t)j | (neg << 31);
                         ++f;
                     }

@@ -97,6 +97,19 @@ def test_dense_clusters(pg, monkeypatch, n, R, betas, cluster, rule):
     compare_dense(pg, n, 3, R=R, sweeps=2, beta0=betas[0], beta1=betas[1], rule=rule, seed=n)
 
 
+@pytest.mark.parametrize("rule", [0, 1])
+@pytest.mark.parametrize("cluster", [1, 2])
+@pytest.mark.parametrize("n,R,betas", [
+    (256, 6, (-0.3, 0.2)),         # through zero, rows saturated at the cold ends
+    (1023, 5, (0.01, -1.0)),       # ragged, from hot to cold on the negative side
+    (2501, 3, (-0.0005, -0.001)),  # thresholds over every field
+])
+def test_dense_negative_beta(pg, monkeypatch, n, R, betas, cluster, rule):
+    """At a negative beta the heat-bath threshold falls with the field."""
+    monkeypatch.setenv("PAMC_DENSE_CLUSTER", str(cluster))
+    compare_dense(pg, n, 4, R=R, sweeps=2, beta0=betas[0], beta1=betas[1], rule=rule, seed=n)
+
+
 def test_dense_restart_and_controller(pg):
     compare_dense(pg, 320, 60, R=16, sweeps=1, beta0=0.01, beta1=0.4, stagnation=1, z_rst=45, seed=5,
                   check_every=3)
