@@ -1735,13 +1735,14 @@ pamc_status rebuild(pamc_batch b) {
     std::vector<RedrawDesc> rds;
     std::vector<int2> rdsi, rdei;             // re-draw items: (member, chunk of draws), (member, replica)
     int32_t ncm_nmax = 1;
-    int32_t nmax[kClasses] = {0, 0, 0}, pnmax[kClasses] = {0, 0, 0}, gnmax[kClasses] = {0, 0, 0},
-            nnmax[kClasses] = {0, 0, 0}, Rmax = 1;
+    int32_t pnmax[kClasses] = {0, 0, 0}, Rmax = 1;
     auto member_global = [&](pamc_handle h) { return h->p.kind == 0 && (h->gsp || b->global[batch_class(h->n)]); };
-    // members whose field ranges fit 4-bit lanes take eight replicas a word, as alone
+    // members whose field ranges fit 4-bit lanes take eight replicas a word, as
+    // alone, where a group's words fit beside the lanes' threshold rows
     auto member_nib = [&](pamc_handle h) {
         return h->p.kind == 0 && !member_global(h) &&
-               sweep_nibble_ok(h->nib_halves, h->p.sweeps, 1, false) && !sweep_push_enabled();
+               sweep_nibble_ok(h->nib_halves, h->p.sweeps, 1, false) && !sweep_push_enabled() &&
+               sweep_nibble_smem_bytes(h->n, h->H, SweepCfg{1, 1, 1}) <= kSmemMax;
     };
     // members on one bit a replica: quads a group so that the batch has about
     // two groups an SM (the largest members' groups bound the step)
@@ -1764,23 +1765,36 @@ pamc_status rebuild(pamc_batch b) {
     // the largest members first: their groups bound the step
     std::vector<pamc_handle> members = b->members;
     std::stable_sort(members.begin(), members.end(), [](pamc_handle x, pamc_handle y) { return x->n > y->n; });
+    std::vector<pamc_handle> byte_of[kClasses], glob_of[kClasses], nib_of[2][kClasses];
     for (pamc_handle h : members)
         if (h->host_t < h->p.steps && !member_bits(h)) {
-            int32_t &m = (h->p.kind != 0 ? pnmax : member_global(h) ? gnmax : member_nib(h) ? nnmax
-                                                                                            : nmax)[batch_class(h->n)];
-            m = std::max(m, h->n);
+            const int c = batch_class(h->n);
+            if (h->p.kind != 0) pnmax[c] = std::max(pnmax[c], h->n);
+            else (member_global(h) ? glob_of : member_nib(h) ? nib_of[h->nib_halves == 2] : byte_of)[c].push_back(h);
         }
-    // the shape of each class, with fewer groups per CTA where the largest
-    // member's spins (Ising: 4n bytes a group, Potts: 8n) need it
-    SweepCfg eff[kClasses], peff[kClasses], geff[kClasses], neff[kClasses];
+    // the shape of each class, with fewer groups per CTA where a member's spins
+    // (Ising: 4n bytes a group, Potts: 8n) and thresholds need it; the launch's
+    // shared memory is what its largest member takes
+    auto bytes = [](const std::vector<pamc_handle> &of, auto &&one) {
+        size_t m = 0;
+        for (pamc_handle h : of) m = std::max(m, one(h->n, h->H));
+        return m;
+    };
+    SweepCfg eff[kClasses], peff[kClasses], geff[kClasses], neff[2][kClasses];
+    size_t smem[kClasses], gsmem[kClasses], nsmem[2][kClasses];
     for (int c = 0; c < kClasses; ++c) {
-        neff[c] = SweepCfg{b->shape[c].groups_per_cta, b->shape[c].warps_per_group, 1};
-        while (neff[c].groups_per_cta > 1 && sweep_nibble_smem_bytes(nnmax[c], kNibbleTwoMaxH, neff[c]) > kSmemMax)
-            neff[c].groups_per_cta -= 1;
+        for (int two = 0; two < 2; ++two) {
+            SweepCfg &q = neff[two][c] = SweepCfg{b->shape[c].groups_per_cta, b->shape[c].warps_per_group, 1};
+            auto one = [&](int32_t n, int32_t H) { return sweep_nibble_smem_bytes(n, H, q); };
+            while (q.groups_per_cta > 1 && bytes(nib_of[two][c], one) > kSmemMax) q.groups_per_cta -= 1;
+            nsmem[two][c] = bytes(nib_of[two][c], one);
+        }
         geff[c] = SweepCfg{b->shape[c].groups_per_cta, b->shape[c].warps_per_group, 1};
+        gsmem[c] = bytes(glob_of[c], [&](int32_t n, int32_t H) { return sweep_ising_smem_bytes(n, H, geff[c], true); });
         eff[c] = b->shape[c];
-        while (eff[c].groups_per_cta > 1 && sweep_ising_smem_bytes(nmax[c], 127, eff[c]) > kSmemMax)
-            eff[c].groups_per_cta -= 1;
+        auto one = [&](int32_t n, int32_t H) { return sweep_ising_smem_bytes(n, H, eff[c]); };
+        while (eff[c].groups_per_cta > 1 && bytes(byte_of[c], one) > kSmemMax) eff[c].groups_per_cta -= 1;
+        smem[c] = bytes(byte_of[c], one);
         peff[c] = SweepCfg{b->shape[c].groups_per_cta, b->shape[c].warps_per_group, 1};
         while (peff[c].groups_per_cta > 1 && sweep_potts_smem_bytes(pnmax[c], 127, peff[c]) > kSmemMax)
             peff[c].groups_per_cta -= 1;
@@ -1837,7 +1851,7 @@ pamc_status rebuild(pamc_batch b) {
         d.gsp = gl ? h->d_gsp : nullptr;
         const bool nb = member_nib(h);
         const bool bt = member_bits(h);
-        const SweepCfg cfg = bt ? bits_shape(h->avg_level, (double)h->nnz / std::max(h->n, 1), bits_nc, false) : p.kind != 0 ? peff[cls] : gl ? geff[cls] : nb ? neff[cls] : eff[cls];
+        const SweepCfg cfg = bt ? bits_shape(h->avg_level, (double)h->nnz / std::max(h->n, 1), bits_nc, false) : p.kind != 0 ? peff[cls] : gl ? geff[cls] : nb ? neff[h->nib_halves == 2][cls] : eff[cls];
         d.push = p.kind == 0 && !gl && !nb && !bt && sweep_push_ok(h->H, p.sweeps, h->d_ell != nullptr, cfg.lanes_per_vertex)
                      ? 1 : 0;
         const int idx = (int)sw.size();
@@ -1930,7 +1944,7 @@ pamc_status rebuild(pamc_batch b) {
             for (int ru = 0; ru < 2; ++ru)
                 for (int c = 0; c < kClasses; ++c)
                     sweep((gl ? gswi : swi)[el][ru][c].size(), [&](const int2 *it, int32_t m, cudaStream_t st) {
-                        return launch_sweep_ising_batched(ru, el != 0, descs, it, m, gl ? gnmax[c] : nmax[c],
+                        return launch_sweep_ising_batched(ru, el != 0, descs, it, m, gl ? gsmem[c] : smem[c],
                                                           gl ? geff[c] : eff[c], st, gl != 0);
                     });
     for (int el = 0; el < 2; ++el)
@@ -1942,7 +1956,7 @@ pamc_status rebuild(pamc_batch b) {
         for (int ru = 0; ru < 2; ++ru)
             for (int c = 0; c < kClasses; ++c)
                 sweep(nswi[bi][ru][c].size(), [&](const int2 *it, int32_t m, cudaStream_t st) {
-                    return launch_sweep_ising_nib_batched(ru, bi != 0, descs, it, m, nnmax[c], neff[c], st);
+                    return launch_sweep_ising_nib_batched(ru, bi != 0, descs, it, m, nsmem[bi][c], neff[bi][c], st);
                 });
     for (auto &[key, v] : bits)
         sweep(v.items.size(), [&, &key = key, &v = v](const int2 *it, int32_t m, cudaStream_t st) {

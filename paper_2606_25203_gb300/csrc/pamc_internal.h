@@ -220,7 +220,7 @@ cudaError_t launch_population_batched(const PrepDesc *prep, const TabDesc *tabs,
 cudaError_t launch_control_batched(const CtlDesc *descs, int32_t ninst, cudaStream_t st);
 size_t prep_smem_bytes(int32_t R);
 cudaError_t launch_sweep_ising_batched(int rule, bool ell, const SweepDesc *descs, const int2 *items,
-                                       int32_t nitems, int32_t n_max, SweepCfg cfg, cudaStream_t st,
+                                       int32_t nitems, size_t smem, SweepCfg cfg, cudaStream_t st,
                                        bool global_spins = false);
 // Batched three-state Potts sweeps (cascaded sampler), one launch per (ELL, size class).
 cudaError_t launch_sweep_potts_batched(bool ell, const SweepDesc *descs, const int2 *items, int32_t nitems,
@@ -269,7 +269,7 @@ cudaError_t launch_sweep_ising_nib(int rule, int32_t n, int32_t H, const pamc_pa
 // halves per member, words on chip); items (member, block of groups of
 // eight).
 cudaError_t launch_sweep_ising_nib_batched(int rule, bool two, const SweepDesc *descs, const int2 *items,
-                                           int32_t nitems, int32_t n_max, SweepCfg cfg, cudaStream_t st);
+                                           int32_t nitems, size_t smem, SweepCfg cfg, cudaStream_t st);
 
 // Ising sweeps with one bit a replica, up to 32 replicas a word
 // (sweep_bits.cu): couplings +-1, at most kBitLaneMaxH neighbours, ELL rows,

@@ -757,11 +757,10 @@ cudaError_t launch_sweep_ising(int rule, int32_t n, const int32_t *rp, const uin
 }
 
 cudaError_t launch_sweep_ising_batched(int rule, bool ell, const SweepDesc *descs, const int2 *items,
-                                       int32_t nitems, int32_t n_max, SweepCfg cfg, cudaStream_t st,
+                                       int32_t nitems, size_t smem, SweepCfg cfg, cudaStream_t st,
                                        bool global_spins) {
     if (nitems <= 0) return cudaSuccess;
     const int gpc = cfg.groups_per_cta, tpg = cfg.warps_per_group * 32;
-    const size_t smem = sweep_ising_smem_bytes(n_max, 127, cfg, global_spins);
     cudaError_t err = cudaSuccess;
     if (global_spins) {   // one lane per vertex
 #define PAMC_LAUNCH_BG(EL, RU)                                                                        \

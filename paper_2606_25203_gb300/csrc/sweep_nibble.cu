@@ -450,10 +450,9 @@ cudaError_t launch_sweep_ising_nib(int rule, int32_t n, int32_t H, const pamc_pa
 }
 
 cudaError_t launch_sweep_ising_nib_batched(int rule, bool two, const SweepDesc *descs, const int2 *items,
-                                           int32_t nitems, int32_t n_max, SweepCfg cfg, cudaStream_t st) {
+                                           int32_t nitems, size_t smem, SweepCfg cfg, cudaStream_t st) {
     if (nitems <= 0) return cudaSuccess;
     const int gpc = cfg.groups_per_cta, tpg = cfg.warps_per_group * 32;
-    const size_t smem = sweep_nibble_smem_bytes(n_max, two ? kNibbleTwoMaxH : kNibbleMaxH, cfg);
     cudaError_t err;
 #define PAMC_NIBB(RU, BI)                                                                    \
     do {                                                                                     \

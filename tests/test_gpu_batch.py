@@ -419,6 +419,34 @@ def test_batch_bit_lane_members(pg):
             pg.pamc_destroy(h)
 
 
+def test_members_that_nearly_fill_shared_memory(pg):
+    """A member whose spin words leave room for its own threshold table only:
+    the launch takes what its largest member needs, not the widest table of
+    the layout beside the largest n of the class (4-bit lanes and, where their
+    rows do not fit, byte lanes), together with members of wider tables."""
+    cases = [(W.torus(240, 240, signed=True, seed=1), dict(R=9, sweeps=1, steps=3, seed=1)),
+             (W.torus(240, 241, signed=True, seed=2), dict(R=5, sweeps=1, steps=3, seed=2)),
+             (W.gnm(9000, 27000, signed=True, seed=3), dict(R=8, sweeps=1, steps=3, seed=3)),
+             (W.er_avg_degree(9000, 40, signed=True, seed=4), dict(R=8, sweeps=1, steps=3, seed=4))]
+    ref = [alone(pg, inst, p) for inst, p in cases]
+    b = pg.pamc_batch_create(0)
+    hs = []
+    try:
+        for inst, p in cases:
+            h = pg.pamc_create_csr(inst.n, inst.row_ptr, inst.col, inst.w)
+            pg.pamc_init(h, **p)
+            pg.pamc_batch_add(b, h)
+            hs.append(h)
+        pg.pamc_batch_step(b, 3)
+        pg.pamc_batch_sync(b)
+        for i, (inst, p) in enumerate(cases):
+            assert_same(snapshot(pg, hs[i], inst.n, p["R"]), ref[i], f"member {i}")
+    finally:
+        pg.pamc_batch_destroy(b)
+        for h in hs:
+            pg.pamc_destroy(h)
+
+
 def test_shapes_change_speed_not_results(pg):
     """Every launch shape of every size class gives the same members' results,
     and the autotuner sets one of the candidates."""
