@@ -1648,7 +1648,6 @@ struct pamc_batch_s {
     int64_t launches = 0;
     int64_t rebuilds = 0;
     SweepCfg shape[3];            // batched sweep launch shape per size class
-    bool shaped[3] = {false, false, false};   // the caller chose it
     cudaStream_t side[4] = {nullptr, nullptr, nullptr, nullptr};   // branches of the captured step
     bool global[3] = {false, false, false};   // Ising members' spin words in device memory
     char err[256] = "";
@@ -1744,12 +1743,13 @@ pamc_status rebuild(pamc_batch b) {
                sweep_nibble_ok(h->nib_halves, h->p.sweeps, 1, false) && !sweep_push_enabled() &&
                sweep_nibble_smem_bytes(h->n, h->H, SweepCfg{1, 1, 1}) <= kSmemMax;
     };
-    // members on one bit a replica: quads a group so that the batch has about
-    // two groups an SM (the largest members' groups bound the step)
+    // members on one bit a replica, whatever shape the caller set for the class's
+    // other layouts (a tuner sets one for every class): quads a group so that the
+    // batch has about two groups an SM (the largest members' groups bound the step)
     int sms = 152;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->device);
     auto bits_can = [&](pamc_handle h) {
-        return h->p.kind == 0 && h->p.sweeps > 0 && h->bits_ok && !member_global(h) && !b->shaped[batch_class(h->n)] &&
+        return h->p.kind == 0 && h->p.sweeps > 0 && h->bits_ok && !member_global(h) &&
                sweep_nibble_enabled() && !sweep_push_enabled() && sweep_bits_smem_bytes(h->n, h->H) <= kSmemMax;
     };
     int64_t bits_R = 0;
@@ -2026,10 +2026,7 @@ pamc_status pamc_batch_create(int cuda_device, void *stream, pamc_batch *out) {
     if (!b) return bfail(nullptr, PAMC_ERR_OOM, "host allocation failed");
     b->device = cuda_device;
     b->stream = (cudaStream_t)stream;
-    for (int c = 0; c < kClasses; ++c) {
-        b->shape[c] = batch_cfg(c);
-        b->shaped[c] = getenv("PAMC_BATCH_CFG") != nullptr;
-    }
+    for (int c = 0; c < kClasses; ++c) b->shape[c] = batch_cfg(c);
     if (!b->stream) {   // graph capture needs a stream other than the legacy default one
         if (cudaStreamCreateWithFlags(&b->stream, cudaStreamNonBlocking) != cudaSuccess) {
             delete b;
@@ -2136,7 +2133,6 @@ pamc_status pamc_batch_set_shape(pamc_batch b, int size_class, int groups_per_ct
         return bfail(b, PAMC_ERR_ARG, "need groups >= 1, warps >= 1 and groups * warps <= 32");
     b->shape[size_class].groups_per_cta = groups_per_cta;
     b->shape[size_class].warps_per_group = warps_per_group;
-    b->shaped[size_class] = true;
     b->dirty = true;
     return PAMC_OK;
 }
@@ -2146,7 +2142,6 @@ pamc_status pamc_batch_set_lanes(pamc_batch b, int size_class, int lanes_per_ver
     if (size_class < 0 || size_class >= kClasses) return bfail(b, PAMC_ERR_ARG, "size class must be 0, 1 or 2");
     if (!batch_lanes_ok(lanes_per_vertex)) return bfail(b, PAMC_ERR_ARG, "lanes per vertex must be 1, 2 or 4");
     b->shape[size_class].lanes_per_vertex = lanes_per_vertex;
-    b->shaped[size_class] = true;
     b->dirty = true;
     return PAMC_OK;
 }

@@ -419,6 +419,51 @@ def test_batch_bit_lane_members(pg):
             pg.pamc_destroy(h)
 
 
+def _kernels_of_a_step(pg, b):
+    """Names of the kernels one batch step launches."""
+    import torch
+    from torch.profiler import ProfilerActivity, profile
+    pg.pamc_batch_step(b, 1)                      # captured before the profile starts
+    pg.pamc_batch_sync(b)
+    with profile(activities=[ProfilerActivity.CUDA]) as prof:
+        pg.pamc_batch_step(b, 1)
+        pg.pamc_batch_sync(b)
+        torch.cuda.synchronize()
+    return [e.name for e in prof.events()]
+
+
+def test_shape_of_a_class_keeps_bit_lane_members(pg):
+    """Setting a class's launch shape (as the autotuner does for every class)
+    leaves the members on one bit a replica there; placing a class's spin words in
+    device memory does not."""
+    cases = [(W.torus(60, 60, signed=True, seed=1), dict(R=1100, sweeps=1, steps=40, seed=1)),
+             (W.er_avg_degree(1500, 20, signed=True, seed=2), dict(R=1100, sweeps=1, steps=40, seed=2))]
+    b = pg.pamc_batch_create(0)
+    hs = []
+    try:
+        for inst, p in cases:
+            h = pg.pamc_create_csr(inst.n, inst.row_ptr, inst.col, inst.w)
+            pg.pamc_init(h, **p)
+            pg.pamc_batch_add(b, h)
+            hs.append(h)
+        names = _kernels_of_a_step(pg, b)
+        if not any("k_control" in x for x in names):
+            pytest.skip("the profiler does not list graph kernels here")
+        assert any("bits" in x for x in names)
+        for c in range(3):
+            pg.pamc_batch_set_shape(b, c, 2, 4)
+            pg.pamc_batch_set_lanes(b, c, 1)
+        names = _kernels_of_a_step(pg, b)
+        assert any("bits" in x for x in names) and not any("k_sweep_ising_batched" in x for x in names)
+        for c in range(3):
+            pg.pamc_batch_set_placement(b, c, True)
+        assert not any("bits" in x for x in _kernels_of_a_step(pg, b))
+    finally:
+        pg.pamc_batch_destroy(b)
+        for h in hs:
+            pg.pamc_destroy(h)
+
+
 def test_members_that_nearly_fill_shared_memory(pg):
     """A member whose spin words leave room for its own threshold table only:
     the launch takes what its largest member needs, not the widest table of
