@@ -79,33 +79,6 @@ def load_peaks():
         return {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0, "sm_max_mhz": 2070.0}, "fallback"
 
 
-# DRAM bytes per launch from the committed ncu captures (profiles/), valid
-# only while the kernel sources still hash to what was captured.
-PROFILED_TRAFFIC = {
-    # k_sweep_ising_nib<heat-bath, width 4> (eight replicas a word), torus
-    # 141x141, R=4096, 10 sweeps: one launch (42.11 MB read + 21.99 MB written)
-    "sweep_torus": (64.10e6, {"paper_2606_25203_gb300/csrc/sweep_nibble.cu":
-                              "69b21e268255bc135dd9ddeb4be65725178d0691"}),
-    # a former k_dense_sweep on byte couplings, 2 sweeps: the n=30,000 capture (1.6856 GB read + 3.3 MB written, the
-    # third step of a fresh run) scaled by n^2 to n=100,000
-    "dense_sweep_100k": (1.6889e9 * (100000 / 30000) ** 2, {"paper_2606_25203_gb300/csrc/dense.cu":
-                                                            "855fcc6f9ccbc2654a4c49491e4e39a2ac464c6a"}),
-}
-
-
-def profiled_traffic(key):
-    import hashlib
-    nbytes, sources = PROFILED_TRAFFIC[key]
-    for path, sha in sources.items():
-        try:
-            with open(os.path.join(ROOT, path), "rb") as f:
-                if hashlib.sha1(f.read()).hexdigest() != sha:
-                    return None
-        except OSError:
-            return None
-    return nbytes
-
-
 class ClockSampler:
     """nvidia-smi clocks and throttle reasons sampled during the timed region.
 
@@ -425,7 +398,7 @@ def run_ours(args):
                                       + (f"; steps 0..{start - 1} untimed" if start else "") + ")",
                        "timed_window": window,
                        "parallelism": "replicas only" if world > 1 else "single GPU"},
-            "roofline": dict(sweep[0], traffic=profiled_traffic("sweep_torus") if ONLY != "sparse" else None,
+            "roofline": dict(sweep[0], traffic=None,
                              kernel=kname[0] + f" ({insts[0].name}, R=4096, 10 sweeps per launch)",
                              peak_source=f"152 SMs x 128 int32 lanes x {sm_max:.0f} MHz ({peak_src} clock)",
                              note="launches of the timed window, beside the other instance's on their own stream "
@@ -852,17 +825,17 @@ def dense_measure(pg, torch, n, steps, warmup, e2e=False):
                        "step_without_sweeps": ms_nosweep},
         "roofline": {"bound": "hbm", "achieved": sw_gbs, "peak": hbm, "unit": "GB/s",
                      "frac": sw_gbs / hbm,
-                     "traffic": (profiled_traffic("dense_sweep_100k") * (n / 100000) ** 2
-                                 if profiled_traffic("dense_sweep_100k") else None),
+                     "traffic": None,
                      "kernel": "k_dense_sweep (bytes = one read of J, one bit a coupling, per sweep)",
                      "peak_source": src},
-        "recompute_roofline": {"bound": "hbm", "achieved": rc_gbs, "peak": hbm, "unit": "GB/s",
+        # (what bounds the recompute is the way of its operands into tensor memory)
+        "recompute_roofline": {"bound": "tensor memory", "achieved": rc_gbs, "peak": hbm, "unit": "GB/s",
                                "frac": rc_gbs / hbm},
         # the rows the flips needed: positions that flipped in at least one
-        # replica; their rows are all a sweep's field updates read of J
+        # replica; their rows (n bits each) are all a sweep's field updates read of J
         "rows_needed": {"rows": rows1 - rows0, "positions": pos1 - pos0,
                         "fraction": (rows1 - rows0) / max(pos1 - pos0, 1),
-                        "achieved_gbs": (rows1 - rows0) * n / (ms_sweep * steps / 1e3) / 1e9},
+                        "achieved_gbs": (rows1 - rows0) * n / 8 / (ms_sweep * steps / 1e3) / 1e9},
         "e2e": e2e_obj,
         "clocks": clk.summary(), "gpu_launches": launches,
         "timed_steps": f"steps 0..{steps - 1} of a fresh run (beta {P['beta0']} -> {P['beta1']} over {P['steps']})",
