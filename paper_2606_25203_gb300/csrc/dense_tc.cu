@@ -52,10 +52,6 @@ constexpr uint32_t kRcACol = 64 * kRcTiles;        // tensor memory: accumulator
 constexpr uint32_t kRcCols = 512;
 constexpr int32_t kBoxRows = 256;                  // rows of one TMA box
 
-__device__ __forceinline__ void mbar_arrive(uint64_t *b) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(b)) : "memory");
-}
-
 __device__ __forceinline__ void tc_mma_ts(uint32_t tmem_d, uint32_t tmem_a, uint64_t bdesc, uint32_t idesc,
                                           uint32_t accumulate) {
     asm volatile(

@@ -39,16 +39,6 @@ namespace {
 constexpr int kStMaxThreads = 640;
 constexpr int kStRingMax = 64;   // blocks in flight (a power of two)
 
-__device__ __forceinline__ void st_arrive(uint64_t *b) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(b)) : "memory");
-}
-__device__ __forceinline__ void bulk_load(void *dst, const void *src, uint32_t bytes, uint64_t *bar) {
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                     smem_u32(dst)),
-                 "l"(src), "r"(bytes), "r"(smem_u32(bar))
-                 : "memory");
-}
-
 // (volatile: ordered against the barriers that hand the slots over)
 __device__ __forceinline__ uint32_t lds32(uint32_t a) {
     uint32_t v;
@@ -236,7 +226,7 @@ k_sweep_ising_staged(SweepDesc d, int cwarps, int nb) {
             reinterpret_cast<int2 *>(slot + 128u * (uint32_t)W)[lane] = pr;
             reinterpret_cast<uint4 *>(slot + 128u * (uint32_t)W + 256u)[lane] = make_uint4(u.x, u.y, u.z, u.w);
             __syncwarp();
-            if (lane == 0) st_arrive(&full[s]);
+            if (lane == 0) mbar_arrive(&full[s]);
         }
         // the consumers wait for every block they read; on an error this warp's
         // last copies are waited for here (bounded) before the CTA leaves
@@ -396,7 +386,7 @@ k_sweep_ising_staged(SweepDesc d, int cwarps, int nb) {
             const int32_t upto = b.sw < S ? b.sw * nblk + (b.base >> 5) : S * nblk;
             __syncwarp();
             if (lane == 0)
-                for (int32_t x = freed; x < upto; ++x) st_arrive(&empty[(uint32_t)x & nbm]);
+                for (int32_t x = freed; x < upto; ++x) mbar_arrive(&empty[(uint32_t)x & nbm]);
             freed = upto;
             return true;
         };
