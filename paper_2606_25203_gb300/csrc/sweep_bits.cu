@@ -305,24 +305,8 @@ bits_body(const SweepDesc &d, const KeyT &key, int32_t t, int32_t slot, const in
     uint32_t *tab_s = reinterpret_cast<uint32_t *>(smem + (rows0 - smem0));
     uint32_t *mark_s = tab_s + (H + 1) * kBitRow;
     const uint32_t marks0 = rows0 + (uint32_t)(H + 1) * (kBitRow * 4);
-    // tab[h + H] (heat-bath), tab[s h + H] (Metropolis): h = 2x - D (D - 2x where
-    // the thresholds fall with the field, beta < 0), s h = D - 2x
-    const bool falling = RULE == 0 && d.tab[0] > d.tab[2 * H];
-    const bool up = RULE == 0 && !falling;
-    for (int i = threadIdx.x; i < (H + 1) * (H + 1); i += blockDim.x) {
-        const int32_t D = i / (H + 1), x = i % (H + 1);
-        if (x > D) continue;
-        const uint64_t T = d.tab[up ? 2 * x - D + H : D - 2 * x + H];
-        tab_s[D * kBitRow + x] = T > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)T;
-    }
-    for (int32_t D = threadIdx.x; D <= H; D += blockDim.x) {
-        int32_t xf = 0;   // first entry of 2^32 (D + 1: none)
-        while (xf <= D && d.tab[up ? 2 * xf - D + H : D - 2 * xf + H] <= 0xFFFFFFFFull) ++xf;
-        // word 0: carry in, words 1..6: the bits of what is added to x
-        const uint32_t c = xf == 0 ? 63u : (uint32_t)((1 << P) - xf);
-        mark_s[D * 8] = xf == 0 ? 0xFFFFFFFFu : 0u;
-        for (int i = 0; i < 7; ++i) mark_s[D * 8 + 1 + i] = 0u - ((c >> i) & 1u);
-    }
+    // (on its way while the spins are read; used below)
+    const uint64_t first = (int)threadIdx.x < 2 * H + 1 ? d.tab[threadIdx.x] : 0ull;
 
     const int li = threadIdx.x, tpg = blockDim.x;
     const int32_t r0 = g * 4 * nc;
@@ -357,6 +341,29 @@ bits_body(const SweepDesc &d, const KeyT &key, int32_t t, int32_t slot, const in
             for (int j = 0; j < 4; ++j)
                 if (k0 + j * tpg < n) sp[k0 + j * tpg] = w[j];
         }
+    }
+    // entries below 2^32 of the table, in rising order: row D's first one of 2^32
+    // is at 2 xf - D + H >= below (D + 1: none)
+    int32_t below = 0;
+    for (int32_t b = 0; b < 2 * H + 1; b += blockDim.x)
+        below += __syncthreads_count(b + (int)threadIdx.x < 2 * H + 1 &&
+                                     (b == 0 ? first : d.tab[b + threadIdx.x]) <= 0xFFFFFFFFull);
+    // tab[h + H] (heat-bath), tab[s h + H] (Metropolis): h = 2x - D (D - 2x where
+    // the thresholds fall with the field, beta < 0), s h = D - 2x
+    const bool falling = RULE == 0 && d.tab[0] > d.tab[2 * H];
+    const bool up = RULE == 0 && !falling;
+    for (int i = threadIdx.x; i < (H + 1) * (H + 1); i += blockDim.x) {
+        const int32_t D = i / (H + 1), x = i % (H + 1);
+        if (x > D) continue;
+        const uint64_t T = d.tab[up ? 2 * x - D + H : D - 2 * x + H];
+        tab_s[D * kBitRow + x] = T > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)T;
+    }
+    for (int32_t D = threadIdx.x; D <= H; D += blockDim.x) {
+        const int32_t xf = min(max((below + D - H + 1) >> 1, 0), D + 1);
+        // word 0: carry in, words 1..6: the bits of what is added to x
+        const uint32_t c = xf == 0 ? 63u : (uint32_t)((1 << P) - xf);
+        mark_s[D * 8] = xf == 0 ? 0xFFFFFFFFu : 0u;
+        for (int i = 0; i < 7; ++i) mark_s[D * 8 + 1 + i] = 0u - ((c >> i) & 1u);
     }
     __syncthreads();
 

@@ -177,21 +177,8 @@ nib_body(const SweepDesc &d, const KeyT &draw, int32_t t, int32_t slot, const in
     const uint32_t marks0 = rows0 + (uint32_t)(H + 1) * (kNibRow * 4);
     uint32_t *spins_all = reinterpret_cast<uint32_t *>(smem + ((nib_table_bytes(H) + 15) & ~(size_t)15));
     unsigned long long *red = reinterpret_cast<unsigned long long *>(spins_all + (size_t)gpc * n_pad);
-    // tab[h + H] (heat-bath), tab[s h + H] (Metropolis): h = 2x - D (D - 2x where
-    // the thresholds fall with the field, beta < 0), s h = D - 2x
-    const bool falling = RULE == 0 && d.tab[0] > d.tab[2 * H];
-    const bool up = RULE == 0 && !falling;
-    for (int i = threadIdx.x; i < (H + 1) * (H + 1); i += blockDim.x) {
-        const int32_t D = i / (H + 1), x = i % (H + 1);
-        if (x > D) continue;
-        const uint64_t T = d.tab[up ? 2 * x - D + H : D - 2 * x + H];
-        tab_s[D * kNibRow + x] = T > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)T;
-    }
-    for (int32_t D = threadIdx.x; D <= H; D += blockDim.x) {
-        int32_t xf = 0;   // first entry of 2^32 (D + 1: none)
-        while (xf <= D && d.tab[up ? 2 * xf - D + H : D - 2 * xf + H] <= 0xFFFFFFFFull) ++xf;
-        mark_s[D] = TWO ? (uint32_t)(128 - xf) * 0x01010101u : (uint32_t)(8 - xf) * 0x11111111u;
-    }
+    // (on its way while the spins are read; used below)
+    const uint64_t first = (int)threadIdx.x < 2 * H + 1 ? d.tab[threadIdx.x] : 0ull;
     for (int i = threadIdx.x; i < gpc * 8; i += blockDim.x) red[i] = 0ull;
 
     const int gl = threadIdx.x / tpg, li = threadIdx.x % tpg;
@@ -223,6 +210,26 @@ nib_body(const SweepDesc &d, const KeyT &draw, int32_t t, int32_t slot, const in
                 if (rows[q] != nullptr) w |= (uint32_t)(rows[q][k] > 0) << (4 * q);
             sp[k] = w;
         }
+    }
+    // entries below 2^32 of the table, in rising order: row D's first one of 2^32
+    // is at 2 xf - D + H >= below (D + 1: none)
+    int32_t below = 0;
+    for (int32_t b = 0; b < 2 * H + 1; b += blockDim.x)
+        below += __syncthreads_count(b + (int)threadIdx.x < 2 * H + 1 &&
+                                     (b == 0 ? first : d.tab[b + threadIdx.x]) <= 0xFFFFFFFFull);
+    // tab[h + H] (heat-bath), tab[s h + H] (Metropolis): h = 2x - D (D - 2x where
+    // the thresholds fall with the field, beta < 0), s h = D - 2x
+    const bool falling = RULE == 0 && d.tab[0] > d.tab[2 * H];
+    const bool up = RULE == 0 && !falling;
+    for (int i = threadIdx.x; i < (H + 1) * (H + 1); i += blockDim.x) {
+        const int32_t D = i / (H + 1), x = i % (H + 1);
+        if (x > D) continue;
+        const uint64_t T = d.tab[up ? 2 * x - D + H : D - 2 * x + H];
+        tab_s[D * kNibRow + x] = T > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)T;
+    }
+    for (int32_t D = threadIdx.x; D <= H; D += blockDim.x) {
+        const int32_t xf = min(max((below + D - H + 1) >> 1, 0), D + 1);
+        mark_s[D] = TWO ? (uint32_t)(128 - xf) * 0x01010101u : (uint32_t)(8 - xf) * 0x11111111u;
     }
     __syncthreads();
 
