@@ -351,10 +351,14 @@ SweepCfg choose_cfg(int kind, int32_t n, int32_t R, int32_t H, double avg_level,
     if (kind == 0 && ell_w > 0) {
         // Groups sized for the latency of a level: lanes per vertex so that
         // the eight slots a lane loads ahead cover an average row (half that
-        // where four or more groups share an SM, and two groups to a CTA
-        // there), halved while an average level needs more lanes than a
-        // group's share of the SM (1024 threads over the groups an SM
-        // holds), then warps so that an average level takes one pass.
+        // where four or more groups share an SM and an average level of all of
+        // them takes more than 400 lanes, and two groups to a CTA there), halved
+        // while an average level needs more lanes than a group's share of the
+        // SM (1024 threads over the groups an SM holds), then warps so that an
+        // average level takes one pass, twice that on the narrowest levels.  (us per
+        // launch of 5 sweeps, half the lanes / all: degree 48, N=200, levels of 3, R=2,048
+        // 207 / 151, R=4,096 211 / 156; N=800, levels of 9, 335 / 252 and 365 / 451;
+        // one / two warps, N=200, R=1,000: 150 / 137.)
         // Where that leaves one lane per vertex on a shared SM, the scoring
         // below decides.
         const int64_t per_sm = (groups + sms - 1) / std::max(sms, 1);
@@ -364,10 +368,13 @@ SweepCfg choose_cfg(int kind, int32_t n, int32_t R, int32_t H, double avg_level,
         SweepCfg c{per_sm >= 4 ? 2 : 1, 1, 1};
         if (lpv_ok)
             while (c.lanes_per_vertex < 32 && 8.0 * c.lanes_per_vertex < avg_deg) c.lanes_per_vertex *= 2;
-        if (per_sm >= 4 && c.lanes_per_vertex > 1) c.lanes_per_vertex >>= 1;
+        if (per_sm >= 4 && c.lanes_per_vertex > 1 && lev * c.lanes_per_vertex * per_sm > 400.0) c.lanes_per_vertex >>= 1;
         while (c.lanes_per_vertex > 1 && lev * c.lanes_per_vertex > lanes) c.lanes_per_vertex >>= 1;
         while (c.warps_per_group * 32 < lanes && 32.0 * c.warps_per_group < lev * c.lanes_per_vertex)
             c.warps_per_group *= 2;
+        if (per_sm < 4 && c.lanes_per_vertex > 1 && lev * c.lanes_per_vertex <= 48.0)
+            while (c.warps_per_group * 32 < lanes && 16.0 * c.warps_per_group < lev * c.lanes_per_vertex)
+                c.warps_per_group *= 2;
         if ((per_sm <= 1 || c.lanes_per_vertex > 1) && sweep_smem_bytes(kind, n, H, c) <= 227 * 1024) return c;
     }
     if (kind != 0) {

@@ -207,6 +207,24 @@ def test_lanes_per_vertex_default_choice(pg, monkeypatch):
         assert (lpv > 1) == want_many, (inst.name, lpv)
 
 
+def _shape(pg, inst, **params):
+    s = pg.Solver(inst.row_ptr, inst.col, inst.w)
+    s.init(sweeps=1, steps=2, seed=1, **params)
+    out = (pg.pamc_sweep_mode(s.h) if not params.get("kind") else None, tuple(pg.pamc_sweep_shape(s.h)))
+    s.close()
+    return out
+
+
+def test_lanes_of_long_rows_on_narrow_levels(pg):
+    """Long rows keep all their lanes where the groups an SM holds leave room for
+    them on narrow levels, and halve them where not."""
+    narrow, wide = W.er_avg_degree(200, 60, signed=True, seed=3), W.er_avg_degree(1500, 60, signed=True, seed=3)
+    for inst, R, lanes in ((narrow, 2048, 8), (wide, 4096, 4)):
+        mode, shape = _shape(pg, inst, R=R)
+        assert (mode, shape[0], shape[2]) == (1, 2, lanes)
+    compare_run(pg, narrow, 2, R=2048, sweeps=1, beta0=0.05, beta1=1.0, seed=3)
+
+
 @pytest.mark.parametrize("cfg", ["1,1,1,1", "1,2,2,1", "1,3,8,1", "1,8,4,1"])
 def test_staged_sweep(pg, monkeypatch, cfg):
     """The staged sweep (rows and draws through a ring in shared memory, two
