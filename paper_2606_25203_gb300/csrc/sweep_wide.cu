@@ -62,7 +62,7 @@ __device__ __forceinline__ uint2 wide_decide(uint2 A, int32_t c0, const u32x4 &u
 }
 
 template <bool ELLP, int RULE, bool GSP>
-__global__ void __launch_bounds__(1024) k_sweep_ising_wide(SweepDesc d, int gpc, int tpg) {
+__global__ void __launch_bounds__(1024, 2) k_sweep_ising_wide(SweepDesc d, int gpc, int tpg) {
     extern __shared__ __align__(16) uint8_t smem[];
     const DevCtl *ctl = d.ctl;
     if (ctl->done) return;
@@ -123,20 +123,30 @@ __global__ void __launch_bounds__(1024) k_sweep_ising_wide(SweepDesc d, int gpc,
                     uint2 A = make_uint2(0x80008000u, 0x80008000u);
                     int32_t k, jsum;
                     if (ELLP) {
+                        // the record and the first two groups of four couplings are
+                        // requested together, the rest two groups at a time
                         const int2 pr = pos[i];
+                        uint4 e0 = ell4(es, i, W, 0), e1 = W > 4 ? ell4(es, i, W, 1) : make_uint4(0u, 0u, 0u, 0u);
                         k = pr.x & 0xFFFFFF;
                         const int32_t deg = (int32_t)((uint32_t)pr.x >> 24);
                         jsum = pos_jsum(pr.y);
-                        for (int32_t v = 0; 4 * v < deg; ++v) {
-                            const uint4 e4 = ell4(es, i, W, v);
+                        auto add4 = [&](const uint4 &e4) {   // padding slots: coupling 0
                             const uint32_t e[4] = {e4.x, e4.y, e4.z, e4.w};
 #pragma unroll
-                            for (int s = 0; s < 4; ++s) {   // padding slots: coupling 0
+                            for (int s = 0; s < 4; ++s) {
                                 const uint2 w = sp[e[s] & 0xFFFFFFu];
                                 const uint32_t J = (uint32_t)((int32_t)e[s] >> 24);
                                 A.x += w.x * J;
                                 A.y += w.y * J;
                             }
+                        };
+                        add4(e0);
+                        if (deg > 4) add4(e1);
+                        for (int32_t v = 2; 4 * v < deg; v += 2) {
+                            e0 = ell4(es, i, W, v);
+                            if (4 * v + 4 < deg) e1 = ell4(es, i, W, v + 1);
+                            add4(e0);
+                            if (4 * v + 4 < deg) add4(e1);
                         }
                     } else {
                         k = ord[i] & 0xFFFFFF;
