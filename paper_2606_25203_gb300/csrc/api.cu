@@ -452,8 +452,11 @@ SweepCfg choose_cfg(int kind, int32_t n, int32_t R, int32_t H, double avg_level,
 
 // The staged sweep (sweep_staged.cu) where every group of four has an SM to
 // itself and a launch is bound by its levels: byte lanes up to an average level
-// of 125 vertices (wider ones have the lanes of the plain sweep busy), 16-bit
-// lanes up to 400.  A pass of a set covers an average level with a little room;
+// of 25 + 2 degree vertices, at most 125 (wider levels of shorter rows have the
+// lanes of the plain sweep busy; us a step of 5 sweeps, staged / plain, R=64: degree 10
+// levels of 32 112 / 122, of 60 142 / 136, of 100 185 / 162; degree 20 of 55 236 /
+// 250, of 78 275 / 257, of 111 342 / 295; degree 36 of 62 470 / 591), 16-bit lanes up
+// to 400.  A pass of a set covers an average level with a little room;
 // rows of more than five couplings take two lanes a vertex, beyond 32 four.
 // us per launch, plain against staged sweep: N=800 degree 48 R=128 329 / 214,
 // N=3,000 degree 20 R=64 279 / 231 (levels of 59), N=2,000 R=256 187 / 189
@@ -462,7 +465,7 @@ SweepCfg choose_cfg(int kind, int32_t n, int32_t R, int32_t H, double avg_level,
 SweepCfg staged_cfg(int32_t n, int32_t R, int32_t H, double avg_level, double avg_deg, int sms, int32_t ell_w) {
     const bool wide = H > kByteLaneMaxH;
     SweepCfg c{1, 2, avg_deg > 32.0 ? 4 : avg_deg > 5.0 ? 2 : 1, 0};
-    if ((R + 3) / 4 > sms || avg_level > (wide ? 400.0 : 125.0)) return c;
+    if ((R + 3) / 4 > sms || avg_level > (wide ? 400.0 : std::min(125.0, 25.0 + 2.0 * avg_deg))) return c;
     const double warps = 1.15 * avg_level * c.lanes_per_vertex / 32.0;
     c.warps_per_group = warps <= 2.0 ? 2 : warps <= 4.0 ? 4 : warps <= 6.0 ? 6 : 8;
     c.staged = sweep_staged_ring(n, H, ell_w, c) > 0 ? 1 : 0;
