@@ -505,7 +505,11 @@ SweepCfg bits_shape(double avg_level, double avg_deg, int nc, bool alone) {
 // bits: N=2,000 degree 20 R=1,024 (two) 456 / 413, N=10,007 degree 20 R=1,100
 // (two) 1,136 / 1,138, R=4,096 (seven) 2,962 / 1,335.  Narrow levels stay with the
 // 4-bit lanes where these apply (N=1,024 torus, R=2,700: 106 / 122).
-bool bits_pay(int nc, double avg_level, bool nib) { return nib ? nc >= 3 && avg_level >= 256.0 : nc >= 2; }
+// Words of two quads on levels of a few vertices stay with the byte lanes (N=100
+// degree 20, levels of 3, R=1,000: 114 / 125 us a step; R=2,048, four quads: 141 / 131).
+bool bits_pay(int nc, double avg_level, bool nib) {
+    return nib ? nc >= 3 && avg_level >= 256.0 : nc >= 3 || (nc == 2 && avg_level >= 5.0);
+}
 SweepCfg bits_cfg(int32_t n, int32_t R, int32_t H, double avg_level, double avg_deg, int sms, bool nib) {
     SweepCfg c{1, 1, 1, 0, 0};
     if (const char *env = getenv("PAMC_SWEEP_CFG")) {   // "1,warps,lanes,0,quads" forces it

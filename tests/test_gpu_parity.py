@@ -342,6 +342,13 @@ def test_bit_lanes_negative_beta(pg, monkeypatch, cfg, rule):
             compare_run(pg, inst, 5, R=R, sweeps=2, beta0=beta0, beta1=beta1, rule=rule, seed=4)
 
 
+def test_bit_lanes_by_level_width(pg):
+    """Words of two quads are taken from levels of five vertices on, more quads
+    on any level."""
+    for n, R, mode in ((100, 1000, 1), (100, 2048, 33), (500, 1000, 33)):
+        assert _shape(pg, W.er_avg_degree(n, 20, signed=True, seed=3), R=R)[0] == mode, (n, R)
+
+
 def test_independent_chains_baseline(pg):
     inst = W.gnm(400, 1100, signed=True, seed=6)
     compare_run(pg, inst, 6, R=9, sweeps=2, resample=0, seed=1)
