@@ -396,6 +396,21 @@ SweepCfg choose_cfg(int kind, int32_t n, int32_t R, int32_t H, double avg_level,
             // / 922 (586); N=12,000 degree 5 R=2,048 2,183 / 1,481 / 1,413 (1,379); of
             // quads: N=2,000 R=256 585 / 453 / 400, R=2,048 710 / 809 / 1,064;
             // N=12,000 2,740 / 2,557 / 2,548
+            if (kind == 1) {
+                // the cascaded sampler's groups that share an SM at a time are
+                // those its shared memory holds (us per launch of 5 sweeps, N=12,000
+                // degree 11, R=4,096, two at a time: 4 warps 2,614, 16 warps 1,780)
+                const size_t one = sweep_smem_bytes(kind, n, H, SweepCfg{1, 4, 2});
+                const int64_t held = std::max<int64_t>(1, std::min<int64_t>(per_sm, (int64_t)(227 * 1024 / one)));
+                while (lanes < 1024 && 2 * lanes * held <= 1024) lanes *= 2;
+                // many groups an SM on narrow levels: two warps a group, two groups a
+                // CTA (four warps, one group / this: N=100 degree 11 R=2,048 87 / 75,
+                // R=4,096 156 / 94; N=500 R=2,048 123 / 115, R=4,096 220 / 146; N=2,000
+                // R=2,048 239 / 284, R=4,096 426 / 382)
+                if (avg_level <= std::min(100.0, 25.0 * (per_sm - 3)) &&
+                    sweep_smem_bytes(kind, n, H, SweepCfg{2, 2, 2}) <= 227 * 1024)
+                    return SweepCfg{2, 2, 2};
+            }
             SweepCfg q{1, 4, kind == 2 ? 4 : avg_level >= lanes ? 1 : 2};
             const double want = avg_level * (kind == 2 ? 2.0 : 1.0) / (per_sm <= 1 ? 8.0 : kind == 2 ? 32.0 : 16.0);
             const int most = per_sm <= 1 ? 32 : std::max(4, lanes / 32);

@@ -349,6 +349,17 @@ def test_bit_lanes_by_level_width(pg):
         assert _shape(pg, W.er_avg_degree(n, 20, signed=True, seed=3), R=R)[0] == mode, (n, R)
 
 
+def test_potts_shapes_by_groups_an_sm_holds(pg):
+    """The cascaded sampler: narrow levels and many groups an SM take two small
+    groups a CTA; groups whose labels fill shared memory take the lanes of those
+    the SM holds at a time."""
+    small, large = W.gnm(100, 550, seed=5), W.gnm(12000, 66000, seed=5)
+    assert _shape(pg, small, R=4096, kind=1)[1] == (2, 2, 2)
+    assert _shape(pg, small, R=256, kind=1)[1] == (1, 4, 2)
+    assert _shape(pg, large, R=4096, kind=1)[1] == (1, 16, 2)
+    compare_run(pg, small, 2, R=4096, sweeps=1, kind=1, beta0=0.1, beta1=2.0, seed=3)
+
+
 def test_independent_chains_baseline(pg):
     inst = W.gnm(400, 1100, signed=True, seed=6)
     compare_run(pg, inst, 6, R=9, sweeps=2, resample=0, seed=1)
