@@ -293,9 +293,10 @@ int pamc_size_class(int32_t n);
  * class's largest member needs it, fewer groups per CTA are used so that the
  * spins fit shared memory.  Members on one bit a replica (see pamc_sweep_mode;
  * in a batch of about 1,800 such replicas or more) have a shape of their own,
- * chosen from the batch, which is not changed here.  The shape changes speed
- * only, never results.  Takes effect at the next pamc_batch_step.  PAMC_ERR_ARG
- * when out of range. */
+ * chosen from the batch, which is not changed here; members on byte lanes take
+ * a shape by the batch's groups unless one was set here.  The shape changes
+ * speed only, never results.  Takes effect at the next pamc_batch_step.
+ * PAMC_ERR_ARG when out of range. */
 pamc_status pamc_batch_set_shape(pamc_batch b, int size_class, int groups_per_cta, int warps_per_group);
 pamc_status pamc_batch_get_shape(pamc_batch b, int size_class, int *groups_per_cta, int *warps_per_group);
 /* Lanes that share one vertex's couplings in the batched Ising sweep of a size

@@ -1677,6 +1677,7 @@ struct pamc_batch_s {
     int64_t launches = 0;
     int64_t rebuilds = 0;
     SweepCfg shape[3];            // batched sweep launch shape per size class
+    bool shaped[3] = {false, false, false};   // the caller chose it
     cudaStream_t side[4] = {nullptr, nullptr, nullptr, nullptr};   // branches of the captured step
     bool global[3] = {false, false, false};   // Ising members' spin words in device memory
     char err[256] = "";
@@ -1820,7 +1821,16 @@ pamc_status rebuild(pamc_batch b) {
         }
         geff[c] = SweepCfg{b->shape[c].groups_per_cta, b->shape[c].warps_per_group, 1};
         gsmem[c] = bytes(glob_of[c], [&](int32_t n, int32_t H) { return sweep_ising_smem_bytes(n, H, geff[c], true); });
+        // byte lanes: unless the caller chose the shape, fewer warps a group where
+        // the groups fill the SMs, by us a step of 5 sweeps, weights to 5, degree 10:
+        // n <= 2,048, {2, 4} / {4, 2}: 1,024 groups 436 / 528, 2,048 557 / 491, 8,192 1,857 /
+        // 1,431; n > 8,192, {1, 32} / {1, 16}: 64 groups 518 / 535, 256 1,122 / 987, 2,048
+        // 5,085 / 3,700
         eff[c] = b->shape[c];
+        int64_t groups = 0;
+        for (pamc_handle h : byte_of[c]) groups += (h->p.R + 3) / 4;
+        if (!b->shaped[c] && c == 0 && groups >= 10 * sms) eff[c] = SweepCfg{4, 2, 1};
+        if (!b->shaped[c] && c == 2 && groups > sms) eff[c] = SweepCfg{1, 16, 1};
         auto one = [&](int32_t n, int32_t H) { return sweep_ising_smem_bytes(n, H, eff[c]); };
         while (eff[c].groups_per_cta > 1 && bytes(byte_of[c], one) > kSmemMax) eff[c].groups_per_cta -= 1;
         smem[c] = bytes(byte_of[c], one);
@@ -2055,7 +2065,10 @@ pamc_status pamc_batch_create(int cuda_device, void *stream, pamc_batch *out) {
     if (!b) return bfail(nullptr, PAMC_ERR_OOM, "host allocation failed");
     b->device = cuda_device;
     b->stream = (cudaStream_t)stream;
-    for (int c = 0; c < kClasses; ++c) b->shape[c] = batch_cfg(c);
+    for (int c = 0; c < kClasses; ++c) {
+        b->shape[c] = batch_cfg(c);
+        b->shaped[c] = getenv("PAMC_BATCH_CFG") != nullptr;
+    }
     if (!b->stream) {   // graph capture needs a stream other than the legacy default one
         if (cudaStreamCreateWithFlags(&b->stream, cudaStreamNonBlocking) != cudaSuccess) {
             delete b;
@@ -2162,6 +2175,7 @@ pamc_status pamc_batch_set_shape(pamc_batch b, int size_class, int groups_per_ct
         return bfail(b, PAMC_ERR_ARG, "need groups >= 1, warps >= 1 and groups * warps <= 32");
     b->shape[size_class].groups_per_cta = groups_per_cta;
     b->shape[size_class].warps_per_group = warps_per_group;
+    b->shaped[size_class] = true;
     b->dirty = true;
     return PAMC_OK;
 }
@@ -2171,6 +2185,7 @@ pamc_status pamc_batch_set_lanes(pamc_batch b, int size_class, int lanes_per_ver
     if (size_class < 0 || size_class >= kClasses) return bfail(b, PAMC_ERR_ARG, "size class must be 0, 1 or 2");
     if (!batch_lanes_ok(lanes_per_vertex)) return bfail(b, PAMC_ERR_ARG, "lanes per vertex must be 1, 2 or 4");
     b->shape[size_class].lanes_per_vertex = lanes_per_vertex;
+    b->shaped[size_class] = true;
     b->dirty = true;
     return PAMC_OK;
 }
