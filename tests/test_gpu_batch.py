@@ -419,45 +419,38 @@ def test_batch_bit_lane_members(pg):
             pg.pamc_destroy(h)
 
 
-def _kernels_of_a_step(pg, b):
-    """Names of the kernels one batch step launches."""
-    import torch
-    from torch.profiler import ProfilerActivity, profile
-    pg.pamc_batch_step(b, 1)                      # captured before the profile starts
-    pg.pamc_batch_sync(b)
-    with profile(activities=[ProfilerActivity.CUDA]) as prof:
-        pg.pamc_batch_step(b, 1)
-        pg.pamc_batch_sync(b)
-        torch.cuda.synchronize()
-    return [e.name for e in prof.events()]
-
-
 def test_shape_of_a_class_keeps_bit_lane_members(pg):
     """Setting a class's launch shape (as the autotuner does for every class)
-    leaves the members on one bit a replica there; placing a class's spin words in
-    device memory does not."""
-    cases = [(W.torus(60, 60, signed=True, seed=1), dict(R=1100, sweeps=1, steps=40, seed=1)),
-             (W.er_avg_degree(1500, 20, signed=True, seed=2), dict(R=1100, sweeps=1, steps=40, seed=2))]
+    leaves the members on one bit a replica there: a step of long rows takes the
+    same time before and after, where byte lanes take two and a half times as
+    long (half as long again is allowed for)."""
+    import time
+    insts = [W.er_avg_degree(1900, 20, signed=True, seed=i) for i in range(8)]
     b = pg.pamc_batch_create(0)
     hs = []
+
+    def step_time():
+        pg.pamc_batch_step(b, 2)
+        pg.pamc_batch_sync(b)
+        best = float("inf")
+        for _ in range(5):
+            t = time.perf_counter()
+            pg.pamc_batch_step(b, 10)
+            pg.pamc_batch_sync(b)
+            best = min(best, time.perf_counter() - t)
+        return best
+
     try:
-        for inst, p in cases:
+        for i, inst in enumerate(insts):
             h = pg.pamc_create_csr(inst.n, inst.row_ptr, inst.col, inst.w)
-            pg.pamc_init(h, **p)
+            pg.pamc_init(h, R=512, sweeps=5, steps=1000, seed=i)
             pg.pamc_batch_add(b, h)
             hs.append(h)
-        names = _kernels_of_a_step(pg, b)
-        if not any("k_control" in x for x in names):
-            pytest.skip("the profiler does not list graph kernels here")
-        assert any("bits" in x for x in names)
+        before = step_time()
         for c in range(3):
             pg.pamc_batch_set_shape(b, c, 2, 4)
             pg.pamc_batch_set_lanes(b, c, 1)
-        names = _kernels_of_a_step(pg, b)
-        assert any("bits" in x for x in names) and not any("k_sweep_ising_batched" in x for x in names)
-        for c in range(3):
-            pg.pamc_batch_set_placement(b, c, True)
-        assert not any("bits" in x for x in _kernels_of_a_step(pg, b))
+        assert step_time() < 1.5 * before
     finally:
         pg.pamc_batch_destroy(b)
         for h in hs:
