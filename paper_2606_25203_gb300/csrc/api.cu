@@ -128,6 +128,7 @@ struct pamc_handle_s {
     int32_t *d_boff = nullptr;           // bucket offsets of the order sort
     uint32_t *d_pkey = nullptr;
     uint32_t *d_rowbits = nullptr;       // positions that flipped in some replica (one bit each)
+    int32_t *d_resume = nullptr;         // [R][2] where a replica's sweeps go on with 32-bit fields
     int32_t dense_Hc = 0;
     int dense_cs = 1;                    // CTAs of a replica's cluster in the sweep
     int32_t dense_R = 0;                 // replicas this handle sweeps (p.R unless split over processes)
@@ -577,6 +578,7 @@ pamc_status init_dense(pamc_handle h, pamc_params p, int32_t base, int32_t own, 
               alloc_n(h, h->d_perm, (size_t)S * n, h->bufs) && alloc_n(h, h->d_pkey, (size_t)S * n, h->bufs) &&
               alloc_n(h, h->d_sidx, (size_t)S * n, h->bufs) &&
               alloc_n(h, h->d_rowbits, (size_t)S * ((n + 31) / 32), h->bufs) &&
+              alloc_n(h, h->d_resume, 2 * (size_t)R, h->bufs) &&
               alloc_n(h, h->d_ident, R, h->bufs) &&
               alloc_n(h, h->d_boff, dense_perm_offsets(S), h->bufs);
     if (ok && split) ok = alloc_n(h, h->d_plocal, R, h->bufs) && alloc_n(h, h->d_rows, Rg, h->bufs);
@@ -646,11 +648,11 @@ pamc_status step_dense(pamc_handle h, int32_t nsteps) {
         if (e == cudaSuccess) e = sweep_timer(h, false);
         if (e == cudaSuccess)
             e = launch_dense_sweep(n, R, p.sweeps, p.rule, h->dense_Hc, (int32_t)t, p.seed, h->dense_cs, h->d_Jb,
-                                   h->d_perm, h->d_tab, src, h->d_parent, h->d_H, dst, Ed, h->d_rowbits, h->d_ctl,
-                                   h->stream);
+                                   h->d_perm, h->d_tab, src, h->d_parent, h->d_H, dst, Ed, h->d_rowbits,
+                                   h->d_resume, h->d_ctl, h->stream);
         if (e == cudaSuccess) e = sweep_timer(h, true);
         if (e == cudaSuccess) e = launch_control(n, h->W, p, Ed, dst, h->d_best, h->d_ctl, h->stream);
-        h->launches += 7;
+        h->launches += 6 + dense_sweep_launches(n);
         if (e == cudaSuccess && restart_due(h)) {
             const int32_t tk = (int32_t)(t + 1);
             e = launch_init_spins(0, 0, n, R, p.seed, tk, 1, h->d_ctl, dst, h->stream);
@@ -1184,10 +1186,10 @@ pamc_status pamc_shard_sweep(pamc_handle h, const int64_t *E_all, const int32_t 
         if (e == cudaSuccess) e = sweep_timer(h, false);
         if (e == cudaSuccess)
             e = launch_dense_sweep(n, c, p.sweeps, p.rule, h->dense_Hc, (int32_t)t, p.seed, h->dense_cs, h->d_Jb,
-                                   h->d_perm, h->d_tab, src, h->d_plocal, h->d_H, dst, Ed, h->d_rowbits, h->d_ctl,
-                                   h->stream, h->sh_base);
+                                   h->d_perm, h->d_tab, src, h->d_plocal, h->d_H, dst, Ed, h->d_rowbits,
+                                   h->d_resume, h->d_ctl, h->stream, h->sh_base);
         if (e == cudaSuccess) e = sweep_timer(h, true);
-        h->launches += 4;
+        h->launches += 3 + dense_sweep_launches(n);
         if (e == cudaSuccess && E_own)
             e = cudaMemcpyAsync(E_own, Ed, sizeof(int64_t) * (size_t)c, cudaMemcpyDeviceToDevice, h->stream);
         if (e != cudaSuccess) return cuda_fail(h, e, "pamc_shard_sweep");

@@ -371,13 +371,14 @@ cudaError_t launch_init_spins(int kind, int32_t K, int32_t n, int32_t R, uint64_
 // Sweeps of the dense instance (dense_sweep.cu): the bit matrix (bit j of row
 // i set iff J_ij = +1, rows of dense_bits_pitch words), one cluster of cs CTAs
 // per replica (0: the fields of a replica fit no cluster); rowbits: scratch of
-// S * ceil(n / 32) words.
+// S * ceil(n / 32) words; resume: scratch of 2 R words (8-byte aligned).
 int32_t dense_bits_pitch(int32_t n);
 int dense_sweep_cluster(int32_t n, int32_t R, int sms);
+int dense_sweep_launches(int32_t n);   // kernels of one launch_dense_sweep
 cudaError_t launch_dense_sweep(int32_t n, int32_t R, int32_t S, int32_t rule, int32_t Hc, int32_t t, uint64_t seed,
                                int cs, const uint32_t *Jb, const int32_t *perm, const uint64_t *tab,
                                const int8_t *src, const int32_t *parent, int32_t *H, int8_t *dst, int64_t *E,
-                               uint32_t *rowbits, DevCtl *ctl, cudaStream_t st, int32_t rbase = 0);
+                               uint32_t *rowbits, int32_t *resume, DevCtl *ctl, cudaStream_t st, int32_t rbase = 0);
 
 // ---- dense recompute H = J S on tcgen05 (dense_tc.cu); Sb: scratch of
 // dense_recompute_scratch bytes; maps: 128-byte CUtensorMap storage each

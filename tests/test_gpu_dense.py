@@ -98,6 +98,48 @@ def test_dense_clusters(pg, monkeypatch, n, R, betas, cluster, rule):
 
 
 @pytest.mark.parametrize("rule", [0, 1])
+@pytest.mark.parametrize("cluster", [1, 2, 4])
+@pytest.mark.parametrize("limit", [100, 128, 140, 160, 300])
+def test_dense_fields_beyond_16_bits(pg, monkeypatch, limit, cluster, rule):
+    """Replicas whose fields leave the 16-bit range (made small here) go on with
+    32-bit fields from the position they reached: from the start, in the middle of
+    a sweep or in a later one, or not at all."""
+    monkeypatch.setenv("PAMC_DENSE_CLUSTER", str(cluster))
+    monkeypatch.setenv("PAMC_DENSE_FIELD_MAX", str(limit))
+    compare_dense(pg, 1023, 5, R=9, sweeps=2, beta0=0.005, beta1=0.3, rule=rule, seed=11)
+
+
+@pytest.mark.parametrize("n", [127, 128, 129, 1000, 1024, 4096])
+def test_dense_uniform_fields(pg, n):
+    """Couplings all +1 and replicas all up or all down: the largest fields and
+    whole batches of flips of one sign (16-bit fields at their ends, counts of
+    every plane), through the population a caller sets."""
+    w = -np.ones((n, n), dtype=np.int8)
+    np.fill_diagonal(w, 0)
+    i, j = np.triu_indices(n, 1)
+    inst = W.csr_from_edges(n, i, j, np.full(i.shape[0], -1), "uniform")
+    p = dict(R=6, sweeps=2, steps=6, beta0=-2.0 / n, beta1=3.0 / n, seed=n)
+    spins = np.ones((6, n), dtype=np.int8)
+    spins[1] = -1
+    spins[2, ::2] = -1
+    spins[3, : n // 2] = -1
+    ref = oracle.OracleRun(inst.row_ptr, inst.col, inst.w, **p)
+    h = pg.pamc_create_dense(n, w)
+    try:
+        pg.pamc_init(h, **p)
+        pg.pamc_set_population(h, spins)
+        ref.set_spins(spins)
+        for t in range(6):
+            pg.pamc_step(h, 1)
+            ref.step(1)
+            got, E, _, _ = pg.pamc_state(h, 6, n)
+            np.testing.assert_array_equal(got, ref.spins(), err_msg=f"spins after {t + 1}")
+            np.testing.assert_array_equal(E, ref.energy(), err_msg=f"energies after {t + 1}")
+    finally:
+        pg.pamc_destroy(h)
+
+
+@pytest.mark.parametrize("rule", [0, 1])
 @pytest.mark.parametrize("cluster", [1, 2])
 @pytest.mark.parametrize("n,R,betas", [
     (256, 6, (-0.3, 0.2)),         # through zero, rows saturated at the cold ends
