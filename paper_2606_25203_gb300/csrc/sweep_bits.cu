@@ -10,9 +10,10 @@
 // with the coupling's sign for all replicas of the group; the bits are counted
 // by carry-save adders into P bit planes (x = their sum, up to 2^P - 1), two
 // three-input logic operations a neighbour.  Heat-bath counts x = N, the
-// neighbours with J_kj s_j = +1 (h = 2N - D, D the row's weight), at a negative
-// beta, where the threshold falls with the field, x = D - N; Metropolis the
-// unsatisfied ones, J_kj s_j = -s_k (one more input to the exclusive or).
+// neighbours with J_kj s_j = +1 (h = 2N - D, D the row's weight); Metropolis the
+// unsatisfied ones, J_kj s_j = -s_k (one more input to the exclusive or).  At a
+// negative beta, heat-bath, the threshold falls with the field: the words then
+// hold the spins inverted, which makes the count x = D - N.
 //
 // Decision.  As in sweep_nibble.cu: shared memory holds, for each D, a row of
 // 32-bit thresholds 256 bytes apart; the planes are merged into bytes 4 x (pairs
@@ -204,8 +205,8 @@ __host__ __device__ __forceinline__ BitLayout bit_layout(int32_t n, int32_t H) {
 
 __device__ __forceinline__ uint32_t sign_mask(uint32_t e) { return (uint32_t)((int32_t)e >> 31); }
 
-// Four neighbours' bits [J_kj s_j = +1] ([J_kj s_j = -1] in the bits that flip
-// sets); slots at or beyond the row's end (left of them in the group) give 0.
+// Four neighbours' bits [J_kj s_j = +1] (flip: [J_kj s_j = -1] where it is all
+// ones); slots at or beyond the row's end (left of them in the group) give 0.
 __device__ __forceinline__ void bit4(uint32_t (&x)[4], const uint4 &e, int32_t left, const uint32_t *sp, uint32_t flip) {
     x[0] = sp[e.x & 0xFFFFFFu] ^ sign_mask(e.x) ^ flip;
     x[1] = sp[e.y & 0xFFFFFFu] ^ sign_mask(e.y) ^ flip;
@@ -305,6 +306,8 @@ bits_body(const SweepDesc &d, const KeyT &key, int32_t t, int32_t slot, const in
     uint32_t *tab_s = reinterpret_cast<uint32_t *>(smem + (rows0 - smem0));
     uint32_t *mark_s = tab_s + (H + 1) * kBitRow;
     const uint32_t marks0 = rows0 + (uint32_t)(H + 1) * (kBitRow * 4);
+    // thresholds that fall with the field: inverted spins
+    const uint32_t inv = RULE == 0 && d.tab[0] > d.tab[2 * H] ? 0xFFFFFFFFu : 0u;
     // (on its way while the spins are read; used below)
     const uint64_t first = (int)threadIdx.x < 2 * H + 1 ? d.tab[threadIdx.x] : 0ull;
 
@@ -339,7 +342,7 @@ bits_body(const SweepDesc &d, const KeyT &key, int32_t t, int32_t slot, const in
             }
 #pragma unroll
             for (int j = 0; j < 4; ++j)
-                if (k0 + j * tpg < n) sp[k0 + j * tpg] = w[j];
+                if (k0 + j * tpg < n) sp[k0 + j * tpg] = w[j] ^ inv;
         }
     }
     // entries below 2^32 of the table, in rising order: row D's first one of 2^32
@@ -350,8 +353,7 @@ bits_body(const SweepDesc &d, const KeyT &key, int32_t t, int32_t slot, const in
                                      (b == 0 ? first : d.tab[b + threadIdx.x]) <= 0xFFFFFFFFull);
     // tab[h + H] (heat-bath), tab[s h + H] (Metropolis): h = 2x - D (D - 2x where
     // the thresholds fall with the field, beta < 0), s h = D - 2x
-    const bool falling = RULE == 0 && d.tab[0] > d.tab[2 * H];
-    const bool up = RULE == 0 && !falling;
+    const bool up = RULE == 0 && inv == 0u;
     for (int i = threadIdx.x; i < (H + 1) * (H + 1); i += blockDim.x) {
         const int32_t D = i / (H + 1), x = i % (H + 1);
         if (x > D) continue;
@@ -376,7 +378,6 @@ bits_body(const SweepDesc &d, const KeyT &key, int32_t t, int32_t slot, const in
         const uint32_t ctr = (kTagFlip << 24) | (uint32_t)(nc * g + d.gbase);
         uint32_t live = 0u;   // the bits of the group's replicas
         for (int32_t q = 0; q < nrep; ++q) live |= 1u << ((q >> 2) + 8 * (q & 3));
-        const uint32_t other = falling ? 0xFFFFFFFFu : 0u;   // heat-bath: counts D - N
         uint32_t nflip = 0;
         for (int32_t sw = 0; sw < S; ++sw) {
             const size_t sb = (size_t)slot * S + sw;
@@ -412,7 +413,7 @@ bits_body(const SweepDesc &d, const KeyT &key, int32_t t, int32_t slot, const in
                     Planes<P> x;
                     if (run) {
                         old = sp[k];
-                        bit_sum<P, QL, WC>(x, e, es, ip, W, (int32_t)(a0 >> 24), sub, sp, RULE == 0 ? other : old);
+                        bit_sum<P, QL, WC>(x, e, es, ip, W, (int32_t)(a0 >> 24), sub, sp, RULE == 0 ? 0u : old);
                     }
                     if constexpr (WC == kDeep) bit_load<QL, WC>(e, es, inext, W, sub);
                     if (run) {
@@ -458,7 +459,7 @@ bits_body(const SweepDesc &d, const KeyT &key, int32_t t, int32_t slot, const in
                             for (int o = NVW; o < 32; o <<= 1) nw |= __shfl_xor_sync(0xffffffffu, nw, o);
                         }
                         nw |= force;
-                        const uint32_t flips = (RULE == 0 ? nw ^ old : nw) & live;
+                        const uint32_t flips = (RULE == 0 ? nw ^ old ^ inv : nw) & live;
                         if (act && sub == 0 && flips != 0u) {
                             sp[k] = old ^ flips;
                             nflip += __popc(flips);
@@ -525,7 +526,7 @@ bits_body(const SweepDesc &d, const KeyT &key, int32_t t, int32_t slot, const in
         for (int32_t k0 = li; k0 < n; k0 += 4 * tpg) {
             uint32_t w[4];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) w[j] = k0 + j * tpg < n ? sp[k0 + j * tpg] : 0u;
+            for (int j = 0; j < 4; ++j) w[j] = k0 + j * tpg < n ? sp[k0 + j * tpg] ^ inv : 0u;
             int8_t *row = dst + (size_t)r0 * n + k0;
             for (int32_t q = 0; q < nrep; ++q, row += n) {
                 const int sh = (q >> 2) + 8 * (q & 3);
