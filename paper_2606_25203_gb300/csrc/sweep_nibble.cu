@@ -102,18 +102,15 @@ __host__ __device__ constexpr size_t nib_table_bytes(int32_t H) { return (size_t
 // mark word, X the index nibbles (one half only).
 template <int RULE, bool TWO>
 __device__ __forceinline__ uint32_t nib_decide(uint32_t X, uint32_t E, uint32_t O, uint32_t D, uint32_t row,
-                                               uint32_t force, bool falling, const u32x4 &ua, const u32x4 &ub,
-                                               uint32_t old) {
-    if constexpr (RULE == 0) {
-        if (falling) {   // uniform over the launch: the index counts the other way
-            if constexpr (TWO) {
-                E = D * 0x01010101u - E;
-                O = D * 0x01010101u - O;
-            } else {
-                X = D * 0x11111111u - X;
-            }
+                                               uint32_t force, const u32x4 &ua, const u32x4 &ub, uint32_t old) {
+    if constexpr (RULE == 2) {   // the index counts the other way
+        if constexpr (TWO) {
+            E = D * 0x01010101u - E;
+            O = D * 0x01010101u - O;
+        } else {
+            X = D * 0x11111111u - X;
         }
-    } else {   // the unsatisfied weight of the replicas with s = +1
+    } else if constexpr (RULE == 1) {   // the unsatisfied weight of the replicas with s = +1
         if constexpr (TWO) {
             const uint32_t me = (old & 0x01010101u) * 0xFFu, mo = ((old >> 4) & 0x01010101u) * 0xFFu;
             const uint32_t D4 = D * 0x01010101u;
@@ -155,6 +152,11 @@ __device__ __forceinline__ void nib_halves(uint32_t A1, uint32_t A2, uint32_t &E
     E = (A1 & 0x0F0F0F0Fu) + (A2 & 0x0F0F0F0Fu);
     O = ((A1 >> 4) & 0x0F0F0F0Fu) + ((A2 >> 4) & 0x0F0F0F0Fu);
 }
+
+// Whether the heat-bath thresholds fall with the field (beta < 0): RULE 2 of the
+// bodies below, chosen once a launch (a branch at every visit cost 2 % of a small
+// instance's launch).
+__device__ __forceinline__ bool nib_falling(const SweepDesc &d) { return d.tab[0] > d.tab[2 * d.H]; }
 
 // The sweeps of one CTA's groups of eight (groups bid*gpc .. bid*gpc+gpc-1
 // of the instance), shared by the single-instance and the batched kernels;
@@ -219,12 +221,10 @@ nib_body(const SweepDesc &d, const KeyT &draw, int32_t t, int32_t slot, const in
                                      (b == 0 ? first : d.tab[b + threadIdx.x]) <= 0xFFFFFFFFull);
     // tab[h + H] (heat-bath), tab[s h + H] (Metropolis): h = 2x - D (D - 2x where
     // the thresholds fall with the field, beta < 0), s h = D - 2x
-    const bool falling = RULE == 0 && d.tab[0] > d.tab[2 * H];
-    const bool up = RULE == 0 && !falling;
     for (int i = threadIdx.x; i < (H + 1) * (H + 1); i += blockDim.x) {
         const int32_t D = i / (H + 1), x = i % (H + 1);
         if (x > D) continue;
-        const uint64_t T = d.tab[up ? 2 * x - D + H : D - 2 * x + H];
+        const uint64_t T = d.tab[RULE == 0 ? 2 * x - D + H : D - 2 * x + H];
         tab_s[D * kNibRow + x] = T > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)T;
     }
     for (int32_t D = threadIdx.x; D <= H; D += blockDim.x) {
@@ -294,7 +294,7 @@ nib_body(const SweepDesc &d, const KeyT &draw, int32_t t, int32_t slot, const in
                     const uint32_t row = rows0 + (D << 8), force = lds_u32(marks0 + (D << 2));
                     uint32_t E = 0u, O = 0u;
                     if constexpr (TWO) nib_halves(A, A2, E, O);
-                    const uint32_t nw = nib_decide<RULE, TWO>(A, E, O, D, row, force, falling, ua, ub, old);
+                    const uint32_t nw = nib_decide<RULE, TWO>(A, E, O, D, row, force, ua, ub, old);
                     if (nw != old) {
                         sp[k] = nw;
                         nflip += __popc((nw ^ old) & live);
@@ -363,7 +363,10 @@ nib_body(const SweepDesc &d, const KeyT &draw, int32_t t, int32_t slot, const in
 
 template <int RULE, int WC, bool TWO>
 __global__ void __launch_bounds__(1024) k_sweep_ising_nib(SweepDesc d, int gpc, int tpg) {
-    nib_body<RULE, WC, TWO>(d, NibKeys{d.K}, d.t, d.slot, d.src, d.dst, d.E_dst, gpc, tpg, blockIdx.x);
+    if (RULE == 0 && nib_falling(d))
+        nib_body<2, WC, TWO>(d, NibKeys{d.K}, d.t, d.slot, d.src, d.dst, d.E_dst, gpc, tpg, blockIdx.x);
+    else
+        nib_body<RULE, WC, TWO>(d, NibKeys{d.K}, d.t, d.slot, d.src, d.dst, d.E_dst, gpc, tpg, blockIdx.x);
 }
 
 // Many instances in one launch: CTA b works on member items[b].x, its block
@@ -375,8 +378,12 @@ k_sweep_ising_nib_batched(const SweepDesc *__restrict__ descs, const int2 *__res
     const SweepDesc &d = descs[it.x];
     const int32_t t = d.ctl->t;
     if (t >= d.t_end) return;
-    nib_body<RULE, 0, TWO>(d, NibKeysSeed{d.K.k0[0], d.K.k1[0]}, t, t % d.slots, d.sp[t & 1],
-                              d.sp[(t + 1) & 1], d.en[(t + 1) & 1], gpc, tpg, it.y);
+    if (RULE == 0 && nib_falling(d))
+        nib_body<2, 0, TWO>(d, NibKeysSeed{d.K.k0[0], d.K.k1[0]}, t, t % d.slots, d.sp[t & 1], d.sp[(t + 1) & 1],
+                            d.en[(t + 1) & 1], gpc, tpg, it.y);
+    else
+        nib_body<RULE, 0, TWO>(d, NibKeysSeed{d.K.k0[0], d.K.k1[0]}, t, t % d.slots, d.sp[t & 1], d.sp[(t + 1) & 1],
+                               d.en[(t + 1) & 1], gpc, tpg, it.y);
 }
 
 }  // namespace
