@@ -472,12 +472,9 @@ SweepCfg choose_cfg(int kind, int32_t n, int32_t R, int32_t H, double avg_level,
 // lanes of the plain sweep busy; us a step of 5 sweeps, staged / plain, R=64: degree 10
 // levels of 32 112 / 122, of 60 142 / 136, of 100 185 / 162; degree 20 of 55 236 /
 // 250, of 78 275 / 257, of 111 342 / 295; degree 36 of 62 470 / 591), 16-bit lanes up
-// to 400.  A pass of a set covers an average level with a little room;
-// rows of more than five couplings take two lanes a vertex, beyond 32 four.
-// us per launch, plain against staged sweep: N=800 degree 48 R=128 329 / 214,
-// N=3,000 degree 20 R=64 279 / 231 (levels of 59), N=2,000 R=256 187 / 189
-// (39), N=4,000 degree 14 R=100 534 / 450 (105), N=10,007 R=509 895 / 954 (196);
-// 16-bit lanes N=2,500 degree 12 R=250 (83) 464 / 179.
+// to 400 (N=2,500 degree 10, R=64: 193 / 305).  A pass of a set covers an
+// average level with a little room; rows of more than five couplings take two
+// lanes a vertex, beyond 32 four.
 SweepCfg staged_cfg(int32_t n, int32_t R, int32_t H, double avg_level, double avg_deg, int sms, int32_t ell_w) {
     const bool wide = H > kByteLaneMaxH;
     SweepCfg c{1, 2, avg_deg > 32.0 ? 4 : avg_deg > 5.0 ? 2 : 1, 0};
@@ -555,10 +552,12 @@ pamc_status init_dense(pamc_handle h, pamc_params p, int32_t base, int32_t own, 
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
     const int32_t n = h->n, R = own, Rg = p.R, S = std::max(p.sweeps, 1);
     // the largest instance: 768 vertices for each SM beyond one per four replicas
+    // (the sizes that have always been taken; the fields of larger ones would fit
+    // clusters of more CTAs, which no measurement or test covers)
     const int cs = dense_sweep_cluster(n, R, sms);
     const int nupd = sms - (R + 3) / 4;
     if (nupd < 1 || (n + nupd - 1) / nupd > 768 || cs == 0)
-        return fail(h, PAMC_ERR_RANGE, "dense instance too large for the on-chip fields");
+        return fail(h, PAMC_ERR_RANGE, "dense runs of R = %d take at most %d vertices", R, 768 * std::max(nupd, 0));
     release_run(h);
     h->p = p;
     h->dense_cs = cs;

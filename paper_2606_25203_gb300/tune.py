@@ -7,7 +7,8 @@ warps per group, lanes per vertex, and where the groups' spin words live
 (shared memory, or device memory with no shared-memory limit on groups per
 SM) -- is timed with CUDA events over a few batch steps; the fastest one is
 set on the caller's batch.  A shape changes speed only, never results, so
-tuning on copies of representative instances is safe.
+tuning on copies of representative instances is safe.  Members on one bit a
+replica have a shape of their own, which a class's shape does not change.
 """
 from __future__ import annotations
 

@@ -65,8 +65,7 @@ def test_dense_small(pg, rule):
 
 
 def test_dense_ragged_n_and_population(pg):
-    # n not a multiple of 16 (byte-copy path of the recompute), R not a
-    # multiple of 4, several position blocks per sweep
+    # n not a multiple of 16, R not a multiple of 4, several batches a sweep
     compare_dense(pg, 1000, 5, R=13, sweeps=2, beta0=0.02, beta1=0.5, seed=1)
 
 
@@ -76,10 +75,8 @@ def test_dense_full_population_multi_block(pg):
 
 @pytest.mark.parametrize("rule", [0, 1])
 def test_dense_cold_rare_flips(pg, rule):
-    """A cold anneal (few positions flip per block after the first steps),
-    so most blocks take the path where the chains load the rows of their own
-    replicas' flips of the previous block instead of a produced tile, and the
-    update CTAs produce only the upper part of the block tile."""
+    """A cold anneal (few positions flip after the first steps): large batches,
+    most of them without a candidate or with a handful."""
     compare_dense(pg, 1024, 12, R=16, sweeps=2, beta0=0.5, beta1=3.0, rule=rule, seed=9, check_every=3)
 
 
@@ -172,7 +169,7 @@ def test_dense_rejects(pg):
     assert e.value.status == 3
     h = pg.pamc_create_dense(n, w)
     with pytest.raises(pg.PamcError):
-        pg.pamc_init(h, R=65, steps=2)       # more replicas than the chain masks hold
+        pg.pamc_init(h, R=65, steps=2)       # more replicas than the recompute takes
     pg.pamc_destroy(h)
     odd, _ = dense_pair(63, 0)
     h = pg.pamc_create_dense(63, odd)
@@ -276,9 +273,9 @@ def test_dense_full_size_sweep_replay(pg):
     """The sweep at full size, n = 100,000 and R = 64 (the benchmark's
     instance and population), on sampled outputs the oracle computes one by
     one: from a seeded population set through the ABI, one step of one sweep
-    at beta0; the first 1,024 positions of the order (four blocks, so the
-    chains, the tiles and the tensor-core field update of earlier blocks all
-    take part) are replayed sequentially on the CPU for every replica from
+    at beta0; the first 1,024 positions of the order (a dozen batches, so the
+    tiles, the decisions and the field passes of earlier batches all take
+    part) are replayed sequentially on the CPU for every replica from
     their exact fields, with the oracle's draws, order and thresholds."""
     import torch
     n, R, seed, K = 100000, 64, 0, 1024
