@@ -929,6 +929,8 @@ static pamc_status init_run(pamc_handle h, const pamc_params *pp, int32_t rank, 
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
     h->cfg = choose_cfg(sweep_kind(p), n, own, h->H, avg_level, (double)h->nnz / std::max(n, 1), sms, h->ell_w);
     const char *genv = getenv("PAMC_SWEEP_GLOBAL");
+    // a forced staged shape is the plain one where the staged sweep has no part
+    if (p.sweeps == 0 || sweep_push_enabled() || (genv && genv[0] == '1')) h->cfg.staged = 0;
     const bool nib_ok = p.kind == 0 && sweep_nibble_ok(h->nib_halves, p.sweeps, 1, false) && !sweep_push_enabled();
     if (p.kind == 0 && p.sweeps > 0 && h->ell_w > 0 && !nib_ok && !sweep_push_enabled() &&
         !(genv && genv[0] == '1') && !getenv("PAMC_SWEEP_CFG")) {

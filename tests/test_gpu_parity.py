@@ -255,6 +255,20 @@ def test_staged_sweep(pg, monkeypatch, cfg):
         compare_run(pg, inst, 3, **p)
 
 
+def test_staged_shape_without_a_staged_sweep(pg, monkeypatch):
+    """A forced staged shape where no staged sweep runs: no sweeps (resampling
+    only), spin words in device memory, the push variant."""
+    monkeypatch.setenv("PAMC_SWEEP_CFG", "1,2,2,1")
+    for inst in (W.torus(12, 12, signed=True, seed=2), W.erdos_renyi(100, 0.3, signed=True, seed=1)):
+        compare_run(pg, inst, 3, R=9, sweeps=0, beta0=0.2, beta1=1.0, seed=3)
+        for var, mode in (("PAMC_SWEEP_GLOBAL", 5), ("PAMC_SWEEP_PUSH", None)):
+            with monkeypatch.context() as m:
+                m.setenv(var, "1")
+                got, shape = _shape(pg, inst, R=9)
+                assert mode is None or got == mode
+                compare_run(pg, inst, 3, R=9, sweeps=2, beta0=0.2, beta1=1.0, seed=3)
+
+
 @pytest.mark.parametrize("cfg", ["1,1,1,1", "1,2,1,1", "1,3,2,1"])
 def test_staged_sweep_uneven_rows(pg, monkeypatch, cfg):
     """Lanes of one warp whose rows end far apart (hubs of up to 120 couplings
